@@ -37,7 +37,8 @@ struct md_ctx {
     int n_rep = 1;
     std::vector<int64_t> rep_off;        // [n_rep + 1] first atom of each replica
     std::vector<double> L;               // [3 n_rep] host mirror of the device boxes
-    double r_cut = 0, skin = 0, r_list = 0, rl2 = 0, lim2 = 0;
+    double r_cut = 0, skin = 0, r_list = 0, rl2 = 0;
+    SkinLimit lim{};
     double dt = 0, half_dt = 0, strain_scale = 1.0;
     Atoms A{};
     Cells C{};
@@ -147,6 +148,19 @@ float cut_skin_bound(const md_ctx *c, double r_cut) {
     const double delta = 3.0 * u + 0.5 * ulp32(r_cut);
     const double bound = 2.0 * std::sqrt(3.0) * r_cut * delta + 3.0 * delta * delta + 6e-7 * rc2;
     return std::nextafter((float)(rc2 + 4.0 * bound), INFINITY);
+}
+
+// The displacement limit and its FP32 screen (ph::place): each FP32 coordinate, and its value at
+// the build, lies within u/2 of the FP64 one (u = ulp32 of the largest box edge plus the skin: an atom
+// further outside is far beyond the limit in FP32 too), so near the limit each component of the FP32
+// displacement is within u of the exact one (their difference is exact or rounded by 2^-24 of
+// itself, counted in the last term); the screen lies 4x the bound below the limit.
+SkinLimit skin_limit(const md_ctx *c) {
+    double Lmax = 0.0;
+    for (double l : c->L) Lmax = std::fmax(Lmax, l);
+    const double u = ulp32(Lmax + c->skin), h = 0.5 * c->skin, d2 = 0.25 * c->skin * c->skin;
+    const double bound = 2.0 * std::sqrt(3.0) * h * u + 3.0 * u * u + 6e-7 * d2;
+    return SkinLimit{d2, std::nextafter((float)(d2 - 4.0 * bound), -INFINITY)};
 }
 
 void list_band(const md_ctx *c, float &lo, float &hi) {
@@ -268,7 +282,7 @@ cudaError_t enqueue_sur_net(md_ctx *ctx, cudaStream_t s) {
 // One velocity-Verlet step of the surrogate: half kick + drift (+ skin check), list rebuild
 // when flagged (the rebuild kernels return at once otherwise), network, force + half kick.
 cudaError_t enqueue_sur_step(md_ctx *ctx, bool energy, bool scheduled_rebuild, int *rows, cudaStream_t s) {
-    cudaError_t e = launch_sur_kick_drift(ctx->A, ctx->half_dt, ctx->dt, ctx->lim2, s);
+    cudaError_t e = launch_sur_kick_drift(ctx->A, ctx->half_dt, ctx->dt, ctx->lim, s);
     if (e == cudaSuccess && scheduled_rebuild) e = launch_set_rebuild(ctx->d_flags, s);
     float lo, hi;
     list_band(ctx, lo, hi);
@@ -286,7 +300,7 @@ cudaError_t enqueue_sur_step(md_ctx *ctx, bool energy, bool scheduled_rebuild, i
 cudaError_t enqueue_forces(md_ctx *ctx) {
     if (ctx->sur) {
         ctx->launches += 4 + kRebuildLaunches + (ctx->list_valid ? 0 : 1);
-        cudaError_t e = launch_check_displacement(ctx->A, ctx->lim2, ctx->stream);
+        cudaError_t e = launch_check_displacement(ctx->A, ctx->lim, ctx->stream);
         if (e == cudaSuccess && !ctx->list_valid) e = launch_set_rebuild(ctx->d_flags, ctx->stream);
         if (e == cudaSuccess) e = enqueue_rebuild(ctx);
         if (e == cudaSuccess) e = launch_clear_rebuild(ctx->d_flags, ctx->stream);
@@ -302,7 +316,7 @@ cudaError_t enqueue_forces(md_ctx *ctx) {
         return e;
     }
     ctx->launches += 4 + kRebuildLaunches + (ctx->list_valid ? 0 : 1);
-    cudaError_t e = launch_check_displacement(ctx->A, ctx->lim2, ctx->stream);
+    cudaError_t e = launch_check_displacement(ctx->A, ctx->lim, ctx->stream);
     if (e == cudaSuccess && !ctx->list_valid) e = launch_set_rebuild(ctx->d_flags, ctx->stream);
     if (e == cudaSuccess) e = enqueue_rebuild(ctx);
     if (e == cudaSuccess) e = launch_density(ctx->A, ctx->P, ctx->precision, ctx->lanes, ctx->stream);
@@ -367,7 +381,7 @@ StepParams step_params(md_ctx *ctx, int n_steps) {
     sp.half_dt = ctx->half_dt;
     sp.dt = ctx->dt;
     sp.strain_scale = ctx->strain_scale;
-    sp.lim2 = ctx->lim2;
+    sp.lim = ctx->lim;
     sp.rebuild_every = ctx->cfg.rebuild_every;
     sp.rl2 = ctx->rl2;
     list_band(ctx, sp.band_lo, sp.band_hi);
@@ -553,7 +567,7 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
     ctx->skin = cfg->skin;
     ctx->r_list = pot->r_cut + cfg->skin;
     ctx->rl2 = ctx->r_list * ctx->r_list;
-    ctx->lim2 = 0.25 * cfg->skin * cfg->skin;
+    ctx->lim = skin_limit(ctx);
     ctx->dt = cfg->dt_fs;
     ctx->half_dt = 0.5 * cfg->dt_fs;
     ctx->strain_scale = 1.0 + cfg->strain_rate_zz * cfg->dt_fs * 1.0e-15;
@@ -639,7 +653,7 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t r) { if (r != cudaSuccess && e == cudaSuccess) e = r; };
     chk(dalloc(ctx, &A.pos, n)); chk(dalloc(ctx, &A.vel, n)); chk(dalloc(ctx, &A.force, n));
-    chk(dalloc(ctx, &A.ref, n)); chk(dalloc(ctx, &A.pos_tmp, n)); chk(dalloc(ctx, &A.vel_tmp, n));
+    chk(dalloc(ctx, &A.ref, n)); chk(dalloc(ctx, &A.reff, n)); chk(dalloc(ctx, &A.pos_tmp, n)); chk(dalloc(ctx, &A.vel_tmp, n));
     chk(dalloc(ctx, &A.force_tmp, n)); chk(dalloc(ctx, &A.posf, n)); chk(dalloc(ctx, &A.p2f, n));
     chk(dalloc(ctx, &A.p2d, n));
     chk(dalloc(ctx, &A.rho, n)); chk(dalloc(ctx, &A.dF, n)); chk(dalloc(ctx, &A.e_atom, n));
@@ -886,17 +900,24 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
             }
         for (int a = 0; a < ns; a++)
             cubic_rows(pot->tables + (2 * npair + a) * tl, nk, hrho, &F64[(size_t)a * nk]);
-        double4_32a *dVP64, *dVP32, *dF64;
+        std::vector<double4_32a> FD64(F64.size());   // F' rows (see Pot::FD64)
+        for (size_t k = 0; k < F64.size(); k++)
+            FD64[k] = make_double4_32a(F64[k].y * P.inv_drho, 2.0 * F64[k].z * P.inv_drho, 3.0 * F64[k].w * P.inv_drho, 0.0);
+        P.xmax_rho = nk - 1;
+        double4_32a *dVP64, *dVP32, *dF64, *dFD64;
         chk(dalloc(ctx, &dVP64, VP64.size()));
         chk(dalloc(ctx, &dVP32, VP32.size() / 8));
         chk(dalloc(ctx, &dF64, F64.size()));
+        chk(dalloc(ctx, &dFD64, FD64.size()));
         if (e != cudaSuccess) return fail(ctx, MD_ERR_OOM, "table allocation", e);
         chk(cudaMemcpy(dVP64, VP64.data(), VP64.size() * sizeof(double4_32a), cudaMemcpyHostToDevice));
         chk(cudaMemcpy(dVP32, VP32.data(), VP32.size() * sizeof(float), cudaMemcpyHostToDevice));
         chk(cudaMemcpy(dF64, F64.data(), F64.size() * sizeof(double4_32a), cudaMemcpyHostToDevice));
         P.VP64 = dVP64;
         P.VP32 = dVP32;
+        chk(cudaMemcpy(dFD64, FD64.data(), FD64.size() * sizeof(double4_32a), cudaMemcpyHostToDevice));
         P.F64 = dF64;
+        P.FD64 = dFD64;
         if (!D64.empty()) {
             double4_32a *dD64;
             float4 *dTX, *dTV;
@@ -969,6 +990,7 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
     chk(cudaMemcpy(ctx->d_flags, &flags, sizeof(Flags), cudaMemcpyHostToDevice));
     chk(cudaMemset(C.cell_count, 0, sizeof(int32_t) * C.ncell));
     chk(cudaMemset(A.wrap, 1, n));   // every atom takes the minimum image until the first build
+    chk(cudaMemset(A.reff, 0, sizeof(float4) * (n > 0 ? n : 1)));   // set by the first build
     chk(cudaMemset(A.partials, 0, sizeof(double) * rows * kPartials));
     chk(cudaDeviceSynchronize());
     chk(launch_wrap(A, ctx->stream));
@@ -1041,7 +1063,7 @@ md_status sur_alloc(md_ctx *ctx) {
 // Neighbour list valid for the current positions (rebuilt when any atom moved > skin/2).
 md_status sur_ensure_list(md_ctx *ctx) {
     MD_CK(reset_errors(ctx));
-    MD_CK(launch_check_displacement(ctx->A, ctx->lim2, ctx->stream));
+    MD_CK(launch_check_displacement(ctx->A, ctx->lim, ctx->stream));
     if (!ctx->list_valid) MD_CK(launch_set_rebuild(ctx->d_flags, ctx->stream));
     MD_CK(enqueue_rebuild(ctx));
     MD_CK(launch_clear_rebuild(ctx->d_flags, ctx->stream));
@@ -1632,7 +1654,7 @@ md_status md_tune(md_ctx *ctx, int32_t *lanes_out) {
         StepParams sp = step_params(ctx, 3);
         sp.thermo = nullptr;   // trial steps leave the thermostat alone
         sp.motion = kMotionVerlet;   // and the predictor-corrector's Taylor terms (same passes)
-        sp.lim2 = 1e300;
+        sp.lim = SkinLimit{1e300, 3e38f};
         sp.rebuild_every = 0;
         sp.strain_scale = 1.0;
         cudaEvent_t e0 = nullptr, e1 = nullptr;

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kThreads) k_density64_pairs(Atoms A, Pot P) {
 
 __global__ void __launch_bounds__(kThreads) k_embed64_pairs(Atoms A, Pot P) {
     const int i = blockIdx.x * kThreads + threadIdx.x;
-    if (i < A.n) ps::pairs_embed64(A, P, i);
+    if (i < A.n) ps::pairs_embed64<true>(A, P, i);
 }
 
 template <int T, int KIND, bool ENERGY>

@@ -8,43 +8,11 @@
 
 #include <cuda_runtime.h>
 
+#include "md_bits.cuh"
 #include "md_internal.cuh"
 
 namespace mdk {
 namespace eam {
-
-// Conversions between FP64 and FP32 by the IEEE bit fields, in integer registers (the FP64 pipe,
-// which the FP64 passes keep busy, also executes the conversion instructions): the exponent is
-// rebiased by 1023 - 127 = 896 and the significand shifted by 29 bits.  f32_trunc: x >= 0 below
-// the FP32 overflow threshold, rounded toward zero (relative error < 2^-23), and 0 below the
-// normal FP32 range (so that coincident atoms still give 1/sqrt(0) = inf); f64_exact: f positive,
-// normal or +inf, exact.
-__device__ __forceinline__ float f32_trunc(double x) {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    return __uint_as_float(hi < (897u << 20) ? 0u : ((hi - (896u << 20)) << 3) | (lo >> 29));
-}
-__device__ __forceinline__ double f64_exact(float f) {
-    const unsigned b = __float_as_uint(f);
-    return b >= 0x7f800000u ? __hiloint2double(0x7ff00000, 0)
-                            : __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
-}
-
-// The rest x - f32_trunc(x) of a positive normal x, as FP32: its 29 low significand bits m, worth
-// m 2^(E - 52), rounded to nearest (0 where m = 0 or E < -70, below which the exponent field
-// would not hold it; the FP64 path's r^2 lie far inside).
-__device__ __forceinline__ float f32_rest(double x) {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const unsigned m = lo & 0x1FFFFFFFu;
-    const int E = (int)(hi >> 20) - 1023;
-    const float mf = __uint2float_rn(m);
-    return (m == 0u || E < -70) ? 0.f : __int_as_float(__float_as_int(mf) + (E - 52) * (1 << 23));
-}
-// f as a double, exact, any sign: 0 for |f| below the normal FP32 range, NaN for inf or NaN.
-__device__ __forceinline__ double f64_of_f32(float f) {
-    const unsigned b = __float_as_uint(f), mag = b & 0x7fffffffu;
-    const double v = __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + (896u << 20))), (int)(mag << 29));
-    return mag >= 0x7f800000u ? __hiloint2double(0x7ff80000, 0) : (mag < 0x00800000u ? 0.0 : v);
-}
 
 // d = dh + dl for any sign: dh = d truncated to FP32, dl the rest rounded to FP32 (|dl| < 2^-23
 // |dh|, relative rounding 2^-24), both on the bit fields in integer registers; 0 and 0 where |d|
@@ -149,11 +117,6 @@ __device__ __forceinline__ int knot_row(R x, int nk, R &t, bool &below) {
 // comparisons and the conversions between double and int act on the IEEE bit patterns in integer
 // registers (non-negative doubles order as their bit patterns do), which leaves the FP64 pipe to
 // the arithmetic.
-// v / 2 by the exponent field (no FP64 operation); |v| below 2^-1021 (a subnormal half) gives 0.
-__device__ __forceinline__ double half64(double v) {
-    const long long b = __double_as_longlong(v);
-    return (b & 0x7FF0000000000000LL) > (1LL << 52) ? __longlong_as_double(b - (1LL << 52)) : 0.0;
-}
 // r2 < rc2 for r2 >= 0 (or NaN, which is never inside) and rc2 > 0.
 __device__ __forceinline__ bool inside64(double r2, double rc2) {
     return __double_as_longlong(r2) < __double_as_longlong(rc2);
@@ -231,7 +194,13 @@ __device__ __forceinline__ R knot_sum(const R2 *__restrict__ k, int n, R r, R &d
     return v;
 }
 
-// F and F' in FP64 (one evaluation per atom, both precisions).
+// F' in FP64 (one evaluation per atom, every precision) and, with WANT_F, F (returned).  F' takes
+// the same operations either way, so a run does not depend on which of its steps want energies.
+//  - F = -A sqrt(rho): 1/sqrt(rho) from rsqrt64 and one Newton step in FP64 (to FP64 rounding; 4
+//    FP64 operations, where the square root and the division of CUDA's library take about 25);
+//  - knot table: the knot interval on bit patterns (knot_row64), F' from the table of the rows'
+//    derivatives (Pot::FD64).  Outside the span: linear continuation, counted.
+template <bool WANT_F = true>
 __device__ __forceinline__ double embed64(const Pot &P, int a, double rho, double &dF, Flags *flags) {
     if (P.kind == MD_POT_FS_ANALYTIC || P.kind == MD_POT_KNOTS) {
         const double Aa = P.kind == MD_POT_KNOTS ? P.A64[a] : P.fs[2];
@@ -239,18 +208,33 @@ __device__ __forceinline__ double embed64(const Pot &P, int a, double rho, doubl
             dF = 0.0;
             return 0.0;
         }
-        double s = sqrt(rho);
+        const unsigned hi = (unsigned)__double2hiint(rho);
+        if (hi - (963u << 20) < (160u << 20)) {   // 2^-60 <= rho < 2^100
+            const double y0 = rsqrt64(rho);
+            const double y = fma(half64(y0), fma(-rho * y0, y0, 1.0), y0);
+            dF = -0.5 * Aa * y;
+            return WANT_F ? -Aa * (rho * y) : 0.0;
+        }
+        const double s = sqrt(rho);
         dF = -0.5 * Aa / s;
         return -Aa * s;
     }
-    double x = (rho - P.rho_min) * P.inv_drho, t, d;
+    const double x = (rho - P.rho_min) * P.inv_drho;
+    double t;
     bool below;
-    int k = knot_row(x, P.nk, t, below);
-    if (below || x > (double)(P.nk - 1)) atomicAdd(&flags->range_violations, 1ull);
-    double4_32a c = P.F64[(size_t)a * P.nk + k];
-    double F = cubic(t, c.x, c.y, c.z, c.w, below, d);
-    dF = d * P.inv_drho;
-    return F;
+    int k;
+    if ((unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(P.xmax_rho)) {
+        k = knot_row64(x, P.nk, t, below);   // inside the span
+    } else {
+        k = knot_row(x, P.nk, t, below);
+        if (below || x > P.xmax_rho) atomicAdd(&flags->range_violations, 1ull);
+    }
+    const double4_32a d = P.FD64[(size_t)a * P.nk + k];
+    dF = below ? d.x : fma(t, fma(t, d.z, d.y), d.x);
+    if (!WANT_F) return 0.0;
+    const double4_32a c = P.F64[(size_t)a * P.nk + k];
+    double unused;
+    return cubic(t, c.x, c.y, c.z, c.w, below, unused);
 }
 
 // Butterfly sum over the T lanes of an atom (all 32 lanes of the warp take part).

@@ -79,6 +79,8 @@ struct Pot {
     const double4_32a *VP64;  // [((a*ns+b)*nk + k)*2 + {0: V, 1: phi_ab}]
     const double4_32a *VP32;  // [(a*ns+b)*nk + k], 8 floats
     const double4_32a *F64;   // [a*nk + k]
+    const double4_32a *FD64;  // [a*nk + k]: (c1, 2 c2, 3 c3, 0) * inv_drho of the F64 row: F' as a quadratic in t
+    double xmax_rho;          // nk - 1: the last knot of the F tables
     // one species: [k] derivative rows of the force pass (mixed, table in shared memory): c1 of V,
     // c1 of phi, then (2 c2, 3 c3) of V and of phi as binary16 pairs scaled by 1/dsv and 1/dsp
     const float4 *D32;
@@ -101,6 +103,13 @@ struct Pot {
     const double2 *K64;
     const float2 *K32;
     double A64[8];
+};
+
+// Skin limit of the displacement check: (skin/2)^2, and the FP32 value of a squared displacement
+// formed from the FP32 positions at or below which the exact one is certainly within it.
+struct SkinLimit {
+    double d2;
+    float d2f;
 };
 
 // Link-cell grid of one replica: its cells are the global cells [base, base + nc0*nc1*nc2).
@@ -127,6 +136,8 @@ struct Atoms {
                                                  // build (as posf; NULL on the mixed path)
     double4_32a *pos_tmp, *vel_tmp, *force_tmp;  // renumbering scratch
     float4 *posf;                            // FP32 wrapped position, w = species bits
+    float4 *reff;                            // posf at the last build (ph::place's skin screen); w = the
+                                             // box edges wrapped off there (ph::pack_image)
     float4 *posx;                            // double-float path: [2 i] = high parts, [2 i + 1] = low parts
                                              // of the image coordinates plus Box::xoff
     float4 *p2x;                             // double-float pass 2: as posx, w = F'(rho) (hi, then lo)
@@ -280,7 +291,7 @@ cudaError_t launch_set_rebuild(Flags *f, cudaStream_t s);
 cudaError_t launch_clear_rebuild(Flags *f, cudaStream_t s);
 cudaError_t launch_rebuild(const Atoms &A, const Cells &C, double rl2, float band_lo, float band_hi,
                            int list_group, cudaStream_t s);
-cudaError_t launch_check_displacement(const Atoms &A, double lim2, cudaStream_t s);
+cudaError_t launch_check_displacement(const Atoms &A, SkinLimit lim, cudaStream_t s);
 cudaError_t launch_wrap(const Atoms &A, cudaStream_t s);
 // lanes = T lanes per atom (1, 2, 4, 8, 16 or 32)
 cudaError_t launch_density(const Atoms &A, const Pot &P, int precision, int lanes, cudaStream_t s);
@@ -316,7 +327,8 @@ constexpr int kKeChunk = 1024;               // atoms per chunk of the kinetic-e
 struct StepParams {
     int n_steps;
     int energy_last;      // FP64 partial sums on the last step
-    double half_dt, dt, strain_scale, lim2;
+    double half_dt, dt, strain_scale;
+    SkinLimit lim;        // displacement since the last build above which the list is rebuilt
     int rebuild_every;    // scheduled rebuild period (0: none)
     double rl2;
     float band_lo, band_hi;
@@ -381,7 +393,7 @@ struct SurNet {
 };
 
 // Surrogate launchers (md_sur_*.cu).  Atom ranges [a0, a1) are contiguous replicas.
-cudaError_t launch_sur_kick_drift(const Atoms &A, double half_dt, double dt, double lim2, cudaStream_t s);
+cudaError_t launch_sur_kick_drift(const Atoms &A, double half_dt, double dt, SkinLimit lim, cudaStream_t s);
 cudaError_t launch_sur_descriptors(const Atoms &A, const SurNet &S, int a0, int a1, cudaStream_t s);
 cudaError_t launch_sur_net32(const Atoms &A, const SurNet &S, int a0, int a1, cudaStream_t s);
 cudaError_t launch_sur_net_tc(const Atoms &A, const SurNet &S, cudaStream_t s);

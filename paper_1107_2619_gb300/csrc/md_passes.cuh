@@ -282,17 +282,21 @@ __device__ __forceinline__ void pair32(const Pot &P, int si, int sj, float Fpi, 
     }
 }
 
-// End of the density pass for atom i (lane 0 after the lane sum): rho, F(rho), F'(rho) and the
-// pass-2 copy (position, F').
+// End of the density pass for atom i: rho, F(rho), F'(rho) and the pass-2 copy (position, F').
+// The per-atom arrays (rho, F', energy) are stored with `keep` only: the steps inside an md_step
+// call need none of them, nor F itself.
+template <bool KEEP = true>
 __device__ __forceinline__ void density32_finish(const Atoms &A, const Pot &P, int i, int si, const float4 &pi,
                                                  float hi, float lo) {
-    const double rho = (double)hi + (double)lo;
+    const double rho = f64_of_f32(hi) + f64_of_f32(lo);
     double dF;
-    const double F = embed64(P, si, rho, dF, A.flags);
-    A.rho[i] = rho;
-    A.dF[i] = dF;
-    A.e_atom[i] = F;
-    A.p2f[i] = make_float4(pi.x, pi.y, pi.z, (float)dF);
+    const double F = embed64<KEEP>(P, si, rho, dF, A.flags);
+    if (KEEP) {
+        A.rho[i] = rho;
+        A.dF[i] = dF;
+        A.e_atom[i] = F;
+    }
+    A.p2f[i] = make_float4(pi.x, pi.y, pi.z, f32_rn(dF));
 }
 
 // Lane sums of the force-pass accumulators over the T lanes of an atom.
@@ -328,20 +332,21 @@ __device__ __forceinline__ void force32_finish(const Atoms &A, int i, const Acc3
     }
 }
 
+// The walk of one lane of atom i and the lane sums: rho_i = hi + lo in all T lanes of the atom.
 template <int T, int KIND, bool MULTI, bool SMT = false>
-__device__ __forceinline__ void density32_item(const Atoms &A, const Pot &P, const Box *boxes, long long g) {
+__device__ __forceinline__ void density32_sum(const Atoms &A, const Pot &P, const Box *boxes, long long g, float &hi,
+                                              float &lo) {
     const int i = (int)(g / T), lane = (int)(g & (T - 1));
     const bool live = i < A.n;
-    float hi = 0.f, lo = 0.f;
-    float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
-    int si = 0;
+    hi = 0.f;
+    lo = 0.f;
     const bool wrap = needs_image(A, i, live);
     if (live) {
         const Box &B = boxes[ph::replica_of(A, i)];
         const float Lx = B.Lf[0], Ly = B.Lf[1], Lz = B.Lf[2];
         const float ix = B.invLf[0], iy = B.invLf[1], iz = B.invLf[2];
-        pi = A.posf[i];
-        si = MULTI ? __float_as_int(pi.w) : 0;
+        const float4 pi = A.posf[i];
+        const int si = MULTI ? __float_as_int(pi.w) : 0;
         const int cnt = min(A.count[i], A.k_max);
         const NbrRow row = nbr_row(A, i);
         unsigned viol = 0;
@@ -376,16 +381,25 @@ __device__ __forceinline__ void density32_item(const Atoms &A, const Pot &P, con
         if (viol) atomicAdd(&A.flags->range_violations, (unsigned long long)viol);
     }
     lane_sum_df<T>(hi, lo);
-    if (live && lane == 0) density32_finish(A, P, i, si, pi, hi, lo);
 }
 
-// Returns the atom index for the lane that finished atom i (lane 0 of a live atom), else -1.
+template <int T, int KIND, bool MULTI, bool SMT = false>
+__device__ __forceinline__ void density32_item(const Atoms &A, const Pot &P, const Box *boxes, long long g) {
+    const int i = (int)(g / T);
+    float hi, lo;
+    density32_sum<T, KIND, MULTI, SMT>(A, P, boxes, g, hi, lo);
+    if (i < A.n && (g & (T - 1)) == 0) {
+        const float4 pi = A.posf[i];
+        density32_finish(A, P, i, MULTI ? __float_as_int(pi.w) : 0, pi, hi, lo);
+    }
+}
+
+// The walk of one lane of atom i and the lane sums: the atom's sums in all its T lanes.
 template <int T, int KIND, bool MULTI, bool ENERGY, bool SMT = false>
-__device__ __forceinline__ int force32_item(const Atoms &A, const Pot &P, const Box *boxes, long long g,
-                                            double half_dt, int motion, double (&part)[kPartials]) {
+__device__ __forceinline__ void force32_sum(const Atoms &A, const Pot &P, const Box *boxes, long long g, Acc32 &a) {
     const int i = (int)(g / T), lane = (int)(g & (T - 1));
     const bool live = i < A.n;
-    Acc32 a;
+    a = Acc32();
     const bool wrap = needs_image(A, i, live);
     if (live) {
         const Box &B = boxes[ph::replica_of(A, i)];
@@ -422,27 +436,77 @@ __device__ __forceinline__ int force32_item(const Atoms &A, const Pot &P, const 
         if (viol) atomicAdd(&A.flags->range_violations, (unsigned long long)viol);
     }
     lane_sum_acc<T, ENERGY>(a);
-    if (!(live && lane == 0)) return -1;
-    force32_finish<ENERGY>(A, i, a, half_dt, motion, part);
-    return i;
+}
+
+template <int T, int KIND, bool MULTI, bool ENERGY, bool SMT = false>
+__device__ __forceinline__ void force32_item(const Atoms &A, const Pot &P, const Box *boxes, long long g,
+                                             double half_dt, int motion, double (&part)[kPartials]) {
+    const int i = (int)(g / T);
+    Acc32 a;
+    force32_sum<T, KIND, MULTI, ENERGY, SMT>(A, P, boxes, g, a);
+    if (i < A.n && (g & (T - 1)) == 0) force32_finish<ENERGY>(A, i, a, half_dt, motion, part);
 }
 
 // ======================================================================= FP64
+// Per-atom sums of the FP64 force pass (and of the double-float pass, converted).
+struct Acc64 {
+    double fx = 0.0, fy = 0.0, fz = 0.0, ep = 0.0;
+    double wxx = 0.0, wyy = 0.0, wzz = 0.0, wyz = 0.0, wxz = 0.0, wxy = 0.0;
+};
+
+template <int T, bool ENERGY>
+__device__ __forceinline__ void lane_sum_acc64(Acc64 &a) {
+    a.fx = lane_sum<T>(a.fx);
+    a.fy = lane_sum<T>(a.fy);
+    a.fz = lane_sum<T>(a.fz);
+    if (ENERGY) {
+        a.ep = lane_sum<T>(a.ep);
+        a.wxx = lane_sum<T>(a.wxx); a.wyy = lane_sum<T>(a.wyy); a.wzz = lane_sum<T>(a.wzz);
+        a.wyz = lane_sum<T>(a.wyz); a.wxz = lane_sum<T>(a.wxz); a.wxy = lane_sum<T>(a.wxy);
+    }
+}
+
+// The FP64 partial sums of atom i on the energy step: e its energy, v its velocity record after the
+// step's second half kick (or corrector), a its virial.
+template <typename ACC>
+__device__ __forceinline__ void add_partials(double (&part)[kPartials], double e, const double4_32a &v, const ACC &a) {
+    const double m = 1.0 / (kMvv2e * v.w);
+    part[0] += e;
+    part[1] += m * fma(v.x, v.x, fma(v.y, v.y, v.z * v.z));
+    part[2] += a.wxx; part[3] += a.wyy; part[4] += a.wzz;
+    part[5] += a.wyz; part[6] += a.wxz; part[7] += a.wxy;
+    part[8] += m * v.x; part[9] += m * v.y; part[10] += m * v.z;
+}
+
+// End of the FP64 force pass for atom i of the stand-alone kernels.
+template <bool ENERGY>
+__device__ __forceinline__ void force64_finish(const Atoms &A, int i, const Acc64 &a, double half_dt, int motion,
+                                               double (&part)[kPartials]) {
+    A.force[i] = make_double4_32a(a.fx, a.fy, a.fz, 0.0);
+    if (!isfinite(a.fx + a.fy + a.fz)) atomicOr(&A.flags->error, FLAG_NONFINITE);
+    double4_32a v = A.vel[i];
+    finish_motion(A, i, v, a.fx, a.fy, a.fz, half_dt, motion);
+    if (ENERGY) {
+        const double e = A.e_atom[i] + a.ep;
+        A.e_atom[i] = e;
+        add_partials(part, e, v, a);
+    }
+}
+
 // energy (one species, derivative cache kept): the pair energies 1/2 V(r) of the atom are summed
 // here too, into E_i, and the force pass adds only the virial.
 template <int T, int KIND, bool MULTI>
-__device__ __forceinline__ void density64_item(const Atoms &A, const Pot &P, const Box *boxes, long long g,
-                                               bool energy = false) {
+__device__ __forceinline__ void density64_sum(const Atoms &A, const Pot &P, const Box *boxes, long long g, bool energy,
+                                              double &rho, double &ep) {
     const int i = (int)(g / T), lane = (int)(g & (T - 1));
     const bool live = i < A.n;
-    double rho = 0.0, ep = 0.0;
-    double4_32a pi = make_double4_32a(0.0, 0.0, 0.0, 0.0);
-    int si = 0;
+    rho = 0.0;
+    ep = 0.0;
     const bool wrap = needs_image(A, i, live);
     if (live) {
         const Box &B = boxes[ph::replica_of(A, i)];
-        pi = ld_phase(A.posd + i);
-        si = MULTI ? A.spec[i] : 0;
+        const double4_32a pi = ld_phase(A.posd + i);
+        const int si = MULTI ? A.spec[i] : 0;
         const int cnt = min(A.count[i], A.k_max);
         const NbrRow row = nbr_row(A, i);
         // one species: keep (V'/r, phi'/r) of every entry for the force passes without energies
@@ -509,14 +573,28 @@ __device__ __forceinline__ void density64_item(const Atoms &A, const Pot &P, con
     }
     rho = lane_sum<T>(rho);
     if (energy) ep = lane_sum<T>(ep);
-    if (live && lane == 0) {
-        double dF;
-        const double F = embed64(P, si, rho, dF, A.flags);
+}
+
+// End of the FP64 density pass for atom i (as density32_finish); ep: the pair energies of the atom.
+template <bool KEEP = true>
+__device__ __forceinline__ void density64_finish(const Atoms &A, const Pot &P, int i, int si, double rho, double ep) {
+    double dF;
+    const double F = embed64<KEEP>(P, si, rho, dF, A.flags);
+    if (KEEP) {
         A.rho[i] = rho;
         A.dF[i] = dF;
         A.e_atom[i] = F + ep;
-        A.p2d[i] = make_double4_32a(pi.x, pi.y, pi.z, dF);
     }
+    const double4_32a p = ld_phase(A.posd + i);
+    A.p2d[i] = make_double4_32a(p.x, p.y, p.z, dF);
+}
+
+template <int T, int KIND, bool MULTI>
+__device__ __forceinline__ void density64_item(const Atoms &A, const Pot &P, const Box *boxes, long long g, bool energy) {
+    const int i = (int)(g / T);
+    double rho, ep;
+    density64_sum<T, KIND, MULTI>(A, P, boxes, g, energy, rho, ep);
+    if (i < A.n && (g & (T - 1)) == 0) density64_finish(A, P, i, MULTI ? A.spec[i] : 0, rho, ep);
 }
 
 // The FP64 force pass from the derivative cache of the density pass (one species): per entry the
@@ -525,12 +603,11 @@ __device__ __forceinline__ void density64_item(const Atoms &A, const Pot &P, con
 // summed into E_i by the density pass of the same step), while the force takes the same
 // operations as without, so that a run does not depend on which of its steps evaluate energies.
 template <int T, int KIND, bool ENERGY>
-__device__ __forceinline__ int force64_cached_item(const Atoms &A, const Pot &P, const Box *boxes, long long g,
-                                                   double half_dt, int motion, double (&part)[kPartials]) {
+__device__ __forceinline__ void force64_cached_sum(const Atoms &A, const Pot &P, const Box *boxes, long long g, Acc64 &a) {
     const int i = (int)(g / T), lane = (int)(g & (T - 1));
     const bool live = i < A.n;
-    double fx = 0.0, fy = 0.0, fz = 0.0, ep = 0.0;
-    double wxx = 0.0, wyy = 0.0, wzz = 0.0, wyz = 0.0, wxz = 0.0, wxy = 0.0;
+    double &fx = a.fx, &fy = a.fy, &fz = a.fz;
+    double &wxx = a.wxx, &wyy = a.wyy, &wzz = a.wzz, &wyz = a.wyz, &wxz = a.wxz, &wxy = a.wxy;
     const bool wrap = needs_image(A, i, live);
     if (live) {
         const Box &B = boxes[ph::replica_of(A, i)];
@@ -566,42 +643,23 @@ __device__ __forceinline__ int force64_cached_item(const Atoms &A, const Pot &P,
         if (wrap) walk(std::true_type{});
         else walk(std::false_type{});
     }
-    fx = lane_sum<T>(fx);
-    fy = lane_sum<T>(fy);
-    fz = lane_sum<T>(fz);
-    if (ENERGY) {
-        ep = lane_sum<T>(ep);
-        wxx = lane_sum<T>(wxx); wyy = lane_sum<T>(wyy); wzz = lane_sum<T>(wzz);
-        wyz = lane_sum<T>(wyz); wxz = lane_sum<T>(wxz); wxy = lane_sum<T>(wxy);
-    }
-    if (!(live && lane == 0)) return -1;
-    A.force[i] = make_double4_32a(fx, fy, fz, 0.0);
-    if (!isfinite(fx + fy + fz)) atomicOr(&A.flags->error, FLAG_NONFINITE);
-    double4_32a v = A.vel[i];
-    finish_motion(A, i, v, fx, fy, fz, half_dt, motion);
-    if (ENERGY) {
-        const double e = A.e_atom[i] + ep;
-        A.e_atom[i] = e;
-        const double m = 1.0 / (kMvv2e * v.w);
-        part[0] += e;
-        part[1] += m * fma(v.x, v.x, fma(v.y, v.y, v.z * v.z));
-        part[2] += wxx; part[3] += wyy; part[4] += wzz;
-        part[5] += wyz; part[6] += wxz; part[7] += wxy;
-        part[8] += m * v.x; part[9] += m * v.y; part[10] += m * v.z;
-    }
-    return i;
 }
 
+// The walk of one lane of atom i and the lane sums: the atom's sums in all its T lanes.
 template <int T, int KIND, bool MULTI, bool ENERGY>
-__device__ __forceinline__ int force64_item(const Atoms &A, const Pot &P, const Box *boxes, long long g,
-                                            double half_dt, int motion, double (&part)[kPartials]) {
+__device__ __forceinline__ void force64_sum(const Atoms &A, const Pot &P, const Box *boxes, long long g, Acc64 &a) {
+    a = Acc64();
     if constexpr (!MULTI) {
-        if (A.dcache) return force64_cached_item<T, KIND, ENERGY>(A, P, boxes, g, half_dt, motion, part);
+        if (A.dcache) {
+            force64_cached_sum<T, KIND, ENERGY>(A, P, boxes, g, a);
+            lane_sum_acc64<T, ENERGY>(a);
+            return;
+        }
     }
     const int i = (int)(g / T), lane = (int)(g & (T - 1));
     const bool live = i < A.n;
-    double fx = 0.0, fy = 0.0, fz = 0.0, ep = 0.0;
-    double wxx = 0.0, wyy = 0.0, wzz = 0.0, wyz = 0.0, wxz = 0.0, wxy = 0.0;
+    double &fx = a.fx, &fy = a.fy, &fz = a.fz, &ep = a.ep;
+    double &wxx = a.wxx, &wyy = a.wyy, &wzz = a.wzz, &wyz = a.wyz, &wxz = a.wxz, &wxy = a.wxy;
     const bool wrap = needs_image(A, i, live);
     if (live) {
         const Box &B = boxes[ph::replica_of(A, i)];
@@ -682,30 +740,16 @@ __device__ __forceinline__ int force64_item(const Atoms &A, const Pot &P, const 
         if (wrap) walk(std::true_type{});
         else walk(std::false_type{});
     }
-    fx = lane_sum<T>(fx);
-    fy = lane_sum<T>(fy);
-    fz = lane_sum<T>(fz);
-    if (ENERGY) {
-        ep = lane_sum<T>(ep);
-        wxx = lane_sum<T>(wxx); wyy = lane_sum<T>(wyy); wzz = lane_sum<T>(wzz);
-        wyz = lane_sum<T>(wyz); wxz = lane_sum<T>(wxz); wxy = lane_sum<T>(wxy);
-    }
-    if (!(live && lane == 0)) return -1;
-    A.force[i] = make_double4_32a(fx, fy, fz, 0.0);
-    if (!isfinite(fx + fy + fz)) atomicOr(&A.flags->error, FLAG_NONFINITE);
-    double4_32a v = A.vel[i];
-    finish_motion(A, i, v, fx, fy, fz, half_dt, motion);
-    if (ENERGY) {
-        const double e = A.e_atom[i] + ep;
-        A.e_atom[i] = e;
-        const double m = 1.0 / (kMvv2e * v.w);
-        part[0] += e;
-        part[1] += m * fma(v.x, v.x, fma(v.y, v.y, v.z * v.z));
-        part[2] += wxx; part[3] += wyy; part[4] += wzz;
-        part[5] += wyz; part[6] += wxz; part[7] += wxy;
-        part[8] += m * v.x; part[9] += m * v.y; part[10] += m * v.z;
-    }
-    return i;
+    lane_sum_acc64<T, ENERGY>(a);
+}
+
+template <int T, int KIND, bool MULTI, bool ENERGY>
+__device__ __forceinline__ void force64_item(const Atoms &A, const Pot &P, const Box *boxes, long long g,
+                                             double half_dt, int motion, double (&part)[kPartials]) {
+    const int i = (int)(g / T);
+    Acc64 a;
+    force64_sum<T, KIND, MULTI, ENERGY>(A, P, boxes, g, a);
+    if (i < A.n && (g & (T - 1)) == 0) force64_finish<ENERGY>(A, i, a, half_dt, motion, part);
 }
 
 // ======================================================================= FP64, each pair once
@@ -789,15 +833,19 @@ __device__ __forceinline__ void density64_pairs_item(const Atoms &A, const Pot &
 }
 
 // After the pair density pass, per atom: rho = own share + the neighbours' shares; F, F'; the
-// pass-2 copy; the accumulators cleared for the force pass.
+// pass-2 copy; the accumulators cleared for the force pass.  KEEP as in density32_finish, and
+// on the energy step: the pair-energy accumulators are zero on every other.
+template <bool KEEP>
 __device__ __forceinline__ void pairs_embed64(const Atoms &A, const Pot &P, int i) {
     const double rho = A.rho[i] + A.rho_acc[i];
     double dF;
-    const double F = embed64(P, 0, rho, dF, A.flags);
-    A.rho[i] = rho;
-    A.dF[i] = dF;
-    A.e_atom[i] = F + A.e_acc[i];   // the pair energies (energy steps; else 0)
-    A.e_acc[i] = 0.0;
+    const double F = embed64<KEEP>(P, 0, rho, dF, A.flags);
+    if (KEEP) {
+        A.rho[i] = rho;
+        A.dF[i] = dF;
+        A.e_atom[i] = F + A.e_acc[i];
+        A.e_acc[i] = 0.0;
+    }
     const double4_32a p = A.posd[i];
     A.p2d[i] = make_double4_32a(p.x, p.y, p.z, dF);
     A.rho_acc[i] = 0.0;
@@ -1147,8 +1195,65 @@ __device__ __forceinline__ void force64_pairs(const Atoms &A, const Pot &P, cons
     else force64_pairs_item<T, KIND, ENERGY>(A, P, boxes, g, part);
 }
 
+// After an atom's force f inside the step kernel: velocity Verlet, the second half kick and, with
+// `open` (the next step follows in the same launch, with nothing between), the next step's first
+// half kick and drift at once, from registers: the kicks share their increment (dt/2) f/m, and the
+// force itself is not stored, as nothing reads it before the next pass replaces it.  The
+// predictor-corrector takes the stored force.  Returns the velocity record after the step.
+__device__ __forceinline__ double4_32a close_step(const Atoms &A, const Box *boxes, const StepParams &sp, int i,
+                                                  double fx, double fy, double fz, bool open) {
+    if (!(finite64(fx) && finite64(fy) && finite64(fz))) atomicOr(&A.flags->error, FLAG_NONFINITE);
+    double4_32a v = A.vel[i];
+    if (sp.motion == kMotionVerlet) {
+        const double ax = __dmul_rn(__dmul_rn(sp.half_dt, fx), v.w), ay = __dmul_rn(__dmul_rn(sp.half_dt, fy), v.w),
+                     az = __dmul_rn(__dmul_rn(sp.half_dt, fz), v.w);
+        v.x = __dadd_rn(v.x, ax);
+        v.y = __dadd_rn(v.y, ay);
+        v.z = __dadd_rn(v.z, az);
+        if (open) {
+            double4_32a u = v, p = A.pos[i];
+            u.x = __dadd_rn(u.x, ax);
+            u.y = __dadd_rn(u.y, ay);
+            u.z = __dadd_rn(u.z, az);
+            p.x = __dadd_rn(p.x, __dmul_rn(sp.dt, u.x));
+            p.y = __dadd_rn(p.y, __dmul_rn(sp.dt, u.y));
+            p.z = __dadd_rn(p.z, __dmul_rn(sp.dt, u.z));
+            A.vel[i] = u;
+            A.pos[i] = p;
+            ph::place(A, boxes, i, p, sp.lim);
+        } else {
+            A.force[i] = make_double4_32a(fx, fy, fz, 0.0);
+            A.vel[i] = v;
+        }
+        return v;
+    }
+    A.force[i] = make_double4_32a(fx, fy, fz, 0.0);
+    finish_motion(A, i, v, fx, fy, fz, sp.half_dt, sp.motion);
+    if (open) ph::predict_pc3(A, boxes, i, sp.dt, sp.lim);
+    return v;
+}
+
 // After the pair force pass, per atom: the force = own share + the neighbours' shares, then what
-// follows it (the kick or the corrector), on the energy step the atom's energy and partial sums.
+// follows it; on the energy step the atom's energy and partial sums (v: the velocity after it).
+template <bool ENERGY>
+__device__ __forceinline__ void pairs_partials64(const Atoms &A, int i, double fx, double fy, double fz,
+                                                 const double4_32a &v, double (&part)[kPartials]) {
+    if (!ENERGY) return;
+    // the virial's per-atom part x_a F_b (virial_shift), x as the force pass took it
+    const double4_32a x = A.p2d[i];
+    part[2] = fma(x.x, fx, part[2]);
+    part[3] = fma(x.y, fy, part[3]);
+    part[4] = fma(x.z, fz, part[4]);
+    part[5] = fma(x.y, fz, part[5]);
+    part[6] = fma(x.x, fz, part[6]);
+    part[7] = fma(x.x, fy, part[7]);
+    const double e = A.e_atom[i];
+    const double m = 1.0 / (kMvv2e * v.w);
+    part[0] += e;
+    part[1] += m * fma(v.x, v.x, fma(v.y, v.y, v.z * v.z));
+    part[8] += m * v.x; part[9] += m * v.y; part[10] += m * v.z;
+}
+
 template <bool ENERGY>
 __device__ __forceinline__ void pairs_kick64(const Atoms &A, int i, double half_dt, int motion,
                                              double (&part)[kPartials]) {
@@ -1158,21 +1263,17 @@ __device__ __forceinline__ void pairs_kick64(const Atoms &A, int i, double half_
     if (!isfinite(fx + fy + fz)) atomicOr(&A.flags->error, FLAG_NONFINITE);
     double4_32a v = A.vel[i];
     finish_motion(A, i, v, fx, fy, fz, half_dt, motion);
-    if (ENERGY) {
-        // the virial's per-atom part x_a F_b (virial_shift), x as the force pass took it
-        const double4_32a x = A.p2d[i];
-        part[2] = fma(x.x, fx, part[2]);
-        part[3] = fma(x.y, fy, part[3]);
-        part[4] = fma(x.z, fz, part[4]);
-        part[5] = fma(x.y, fz, part[5]);
-        part[6] = fma(x.x, fz, part[6]);
-        part[7] = fma(x.x, fy, part[7]);
-        const double e = A.e_atom[i];
-        const double m = 1.0 / (kMvv2e * v.w);
-        part[0] += e;
-        part[1] += m * fma(v.x, v.x, fma(v.y, v.y, v.z * v.z));
-        part[8] += m * v.x; part[9] += m * v.y; part[10] += m * v.z;
-    }
+    pairs_partials64<ENERGY>(A, i, fx, fy, fz, v, part);
+}
+
+// The same inside the step kernel.
+template <bool ENERGY>
+__device__ __forceinline__ void pairs_close64(const Atoms &A, const Box *boxes, const StepParams &sp, int i, bool open,
+                                              double (&part)[kPartials]) {
+    const double4_32a own = A.force[i], acc = A.f_acc[i];
+    const double fx = own.x + acc.x, fy = own.y + acc.y, fz = own.z + acc.z;
+    const double4_32a v = close_step(A, boxes, sp, i, fx, fy, fz, open);
+    pairs_partials64<ENERGY>(A, i, fx, fy, fz, v, part);
 }
 
 // ======================================================================= double-float (MD_PREC_DF)
@@ -1246,17 +1347,15 @@ __device__ __forceinline__ df::F2 dcubic_df(df::F2 t, float4 r1, float e3, bool 
 }
 
 template <int T>
-__device__ __forceinline__ void density_df_item(const Atoms &A, const Pot &P, const Box *boxes, long long g,
-                                                bool energy = false) {
+__device__ __forceinline__ void density_df_sum(const Atoms &A, const Pot &P, const Box *boxes, long long g, bool energy,
+                                               df::F2 &rho, df::F2 &ep) {
     const int i = (int)(g / T), lane = (int)(g & (T - 1));
     const bool live = i < A.n;
     df::Acc rho_acc{0.f, 0.f}, e_acc{0.f, 0.f};
-    float4 pih = make_float4(0.f, 0.f, 0.f, 0.f), pil = pih;
     const bool wrap = needs_image(A, i, live);
     if (live) {
         const Box &B = boxes[ph::replica_of(A, i)];
-        pih = ld_phase(A.posx + 2 * (size_t)i);
-        pil = ld_phase(A.posx + 2 * (size_t)i + 1);
+        const float4 pih = ld_phase(A.posx + 2 * (size_t)i), pil = ld_phase(A.posx + 2 * (size_t)i + 1);
         const int cnt = min(A.count[i], A.k_max);
         const NbrRow row = nbr_row(A, i);
         const DRow drow = dcache_row(A, i);
@@ -1296,29 +1395,43 @@ __device__ __forceinline__ void density_df_item(const Atoms &A, const Pot &P, co
         if (wrap) walk(std::true_type{});
         else walk(std::false_type{});
     }
-    const df::F2 rho = df::lane_sum<T>(df::acc_value(rho_acc));
-    const df::F2 ep = energy ? df::lane_sum<T>(df::acc_value(e_acc)) : df::make(0.f);
-    if (live && lane == 0) {
-        const double rr = df::to_double(rho);
-        double dF;
-        const double F = embed64(P, 0, rr, dF, A.flags);
+    rho = df::lane_sum<T>(df::acc_value(rho_acc));
+    ep = energy ? df::lane_sum<T>(df::acc_value(e_acc)) : df::make(0.f);
+}
+
+// End of the double-float density pass for atom i (as density32_finish).
+template <bool KEEP = true>
+__device__ __forceinline__ void density_df_finish(const Atoms &A, const Pot &P, int i, df::F2 rho, df::F2 ep) {
+    const double rr = df::to_double(rho);
+    double dF;
+    const double F = embed64<KEEP>(P, 0, rr, dF, A.flags);
+    if (KEEP) {
         A.rho[i] = rr;
         A.dF[i] = dF;
         A.e_atom[i] = F + df::to_double(ep);
-        const df::F2 f2 = df::from_double(dF);
-        A.p2x[2 * (size_t)i] = make_float4(pih.x, pih.y, pih.z, f2.h);
-        A.p2x[2 * (size_t)i + 1] = make_float4(pil.x, pil.y, pil.z, f2.l);
     }
+    const float4 pih = ld_phase(A.posx + 2 * (size_t)i), pil = ld_phase(A.posx + 2 * (size_t)i + 1);
+    const df::F2 f2 = df::from_double(dF);
+    A.p2x[2 * (size_t)i] = make_float4(pih.x, pih.y, pih.z, f2.h);
+    A.p2x[2 * (size_t)i + 1] = make_float4(pil.x, pil.y, pil.z, f2.l);
+}
+
+template <int T>
+__device__ __forceinline__ void density_df_item(const Atoms &A, const Pot &P, const Box *boxes, long long g, bool energy) {
+    const int i = (int)(g / T);
+    df::F2 rho, ep;
+    density_df_sum<T>(A, P, boxes, g, energy, rho, ep);
+    if (i < A.n && (g & (T - 1)) == 0) density_df_finish(A, P, i, rho, ep);
 }
 
 template <int T, bool ENERGY>
-__device__ __forceinline__ int force_df_item(const Atoms &A, const Pot &P, const Box *boxes, long long g,
-                                             double half_dt, int motion, double (&part)[kPartials]) {
+__device__ __forceinline__ void force_df_sum(const Atoms &A, const Pot &P, const Box *boxes, long long g, Acc64 &out) {
+    out = Acc64();
     const int i = (int)(g / T), lane = (int)(g & (T - 1));
     const bool live = i < A.n;
     df::Acc ax{0.f, 0.f}, ay = ax, az = ax;
-    df::F2 ep = df::make(0.f);
-    df::F2 wv[6] = {ep, ep, ep, ep, ep, ep};
+    const df::F2 zero = df::make(0.f);
+    df::F2 wv[6] = {zero, zero, zero, zero, zero, zero};
     const bool wrap = needs_image(A, i, live);
     if (live) {
         const Box &B = boxes[ph::replica_of(A, i)];
@@ -1356,57 +1469,167 @@ __device__ __forceinline__ int force_df_item(const Atoms &A, const Pot &P, const
         if (wrap) walk(std::true_type{});
         else walk(std::false_type{});
     }
-    const df::F2 fx = df::lane_sum<T>(df::acc_value(ax)), fy = df::lane_sum<T>(df::acc_value(ay)),
-                 fz = df::lane_sum<T>(df::acc_value(az));
+    out.fx = df::to_double(df::lane_sum<T>(df::acc_value(ax)));
+    out.fy = df::to_double(df::lane_sum<T>(df::acc_value(ay)));
+    out.fz = df::to_double(df::lane_sum<T>(df::acc_value(az)));
     if (ENERGY) {
-        ep = df::lane_sum<T>(ep);
 #pragma unroll
         for (int q = 0; q < 6; q++) wv[q] = df::lane_sum<T>(wv[q]);
-    }
-    if (!(live && lane == 0)) return -1;
-    const double Fx = df::to_double(fx), Fy = df::to_double(fy), Fz = df::to_double(fz);
-    A.force[i] = make_double4_32a(Fx, Fy, Fz, 0.0);
-    if (!isfinite(Fx + Fy + Fz)) atomicOr(&A.flags->error, FLAG_NONFINITE);
-    double4_32a v = A.vel[i];
-    finish_motion(A, i, v, Fx, Fy, Fz, half_dt, motion);
-    if (ENERGY) {
-        const double e = A.e_atom[i] + df::to_double(ep);
-        A.e_atom[i] = e;
-        const double m = 1.0 / (kMvv2e * v.w);
-        part[0] += e;
-        part[1] += m * fma(v.x, v.x, fma(v.y, v.y, v.z * v.z));
-#pragma unroll
-        for (int q = 0; q < 6; q++) part[2 + q] += df::to_double(wv[q]);
-        part[8] += m * v.x; part[9] += m * v.y; part[10] += m * v.z;
-    }
-    return i;
-}
-
-// Precision-generic front ends.
-// energy: the step's energies are wanted (the FP64 path with the derivative cache and the
-// double-float path sum the pair energies in this pass; the mixed path in the force pass).
-template <int PREC, int T, int KIND, bool MULTI, bool SMT = false>
-__device__ __forceinline__ void density_item(const Atoms &A, const Pot &P, const Box *boxes, long long g,
-                                             bool energy = false) {
-    if constexpr (PREC == MD_PREC_DF) {
-        if constexpr (KIND == MD_POT_TABLES && !MULTI) density_df_item<T>(A, P, boxes, g, energy);
-    } else if constexpr (PREC == MD_PREC_FP64) {
-        density64_item<T, KIND, MULTI>(A, P, boxes, g, energy);
-    } else {
-        density32_item<T, KIND, MULTI, SMT>(A, P, boxes, g);
+        out.wxx = df::to_double(wv[0]); out.wyy = df::to_double(wv[1]); out.wzz = df::to_double(wv[2]);
+        out.wyz = df::to_double(wv[3]); out.wxz = df::to_double(wv[4]); out.wxy = df::to_double(wv[5]);
     }
 }
 
-template <int PREC, int T, int KIND, bool MULTI, bool ENERGY, bool SMT = false>
-__device__ __forceinline__ int force_item(const Atoms &A, const Pot &P, const Box *boxes, long long g,
-                                          double half_dt, int motion, double (&part)[kPartials]) {
-    if constexpr (PREC == MD_PREC_DF) {
-        if constexpr (KIND == MD_POT_TABLES && !MULTI) return force_df_item<T, ENERGY>(A, P, boxes, g, half_dt, motion, part);
-        return -1;
-    } else if constexpr (PREC == MD_PREC_FP64) {
-        return force64_item<T, KIND, MULTI, ENERGY>(A, P, boxes, g, half_dt, motion, part);
-    } else {
-        return force32_item<T, KIND, MULTI, ENERGY, SMT>(A, P, boxes, g, half_dt, motion, part);
+template <int T, bool ENERGY>
+__device__ __forceinline__ void force_df_item(const Atoms &A, const Pot &P, const Box *boxes, long long g,
+                                              double half_dt, int motion, double (&part)[kPartials]) {
+    const int i = (int)(g / T);
+    Acc64 a;
+    force_df_sum<T, ENERGY>(A, P, boxes, g, a);
+    if (i < A.n && (g & (T - 1)) == 0) force64_finish<ENERGY>(A, i, a, half_dt, motion, part);
+}
+
+// ======================================================================= the step kernel's list walk
+// The two passes over the items g = tid, tid + stride, ... of the step kernel (tid, stride: the
+// thread's and the launch's, stride a multiple of 32; items rounded up to whole warps).  The
+// walk of an item leaves an atom's sums in its T lanes; what follows per atom (F', the kicks, the
+// drift) is FP64 work whose cost does not depend on the number of active lanes (md_bits.cuh), so it
+// is put off until T items' worth of atoms, 32 of them, are at hand, one per lane: lane l then
+// finishes atom l % (32 / T) of item l / (32 / T).  On fcc Cu 500,000 atoms (mixed, 2 lanes per
+// atom) lane 0 of each atom finishing on its own took FP64 warp instructions for 16 atoms each,
+// now for 32, whatever T.
+template <int T>
+struct Batch {
+    static constexpr int AW = 32 / T;   // atoms per item of a warp
+    int lane;
+    long long base;                     // the batch's first item of this warp's lane 0
+    __device__ __forceinline__ Batch(long long g0) : lane((int)(threadIdx.x & 31)), base(g0 - lane) {}
+    // The sum of the atom this lane finishes, once item `sub` has produced it (in its T lanes).
+    template <typename V>
+    __device__ __forceinline__ void take(V &keep, V x, int sub) const {
+        if (T == 1) {
+            keep = x;
+            return;
+        }
+        const V y = __shfl_sync(0xffffffffu, x, (lane & (AW - 1)) * T);
+        if (lane / AW == sub) keep = y;
+    }
+    // The atom this lane finishes, or -1.
+    __device__ __forceinline__ int atom(long long stride, long long items, int n) const {
+        const long long g = base + (long long)(lane / AW) * stride;
+        const long long i = g / T + (lane & (AW - 1));
+        return g < items && i < n ? (int)i : -1;
+    }
+};
+
+// KEEP: the last step of the call (rho, F', the energies are stored); energy: and its energies.
+template <int PREC, int T, int KIND, bool MULTI, bool SMT, bool KEEP>
+__device__ __forceinline__ void density_walk(const Atoms &A, const Pot &P, const Box *boxes, long long tid,
+                                             long long stride, long long items, bool energy) {
+    for (long long g0 = tid; g0 < items; g0 += stride * T) {
+        const Batch<T> b(g0);
+        if constexpr (PREC == MD_PREC_MIXED) {
+            float khi = 0.f, klo = 0.f;
+#pragma unroll 1
+            for (int sub = 0; sub < T && g0 + sub * stride < items; sub++) {
+                float hi, lo;
+                density32_sum<T, KIND, MULTI, SMT>(A, P, boxes, g0 + sub * stride, hi, lo);
+                b.take(khi, hi, sub);
+                b.take(klo, lo, sub);
+            }
+            const int i = b.atom(stride, items, A.n);
+            if (i >= 0) {
+                const float4 pi = A.posf[i];
+                density32_finish<KEEP>(A, P, i, MULTI ? __float_as_int(pi.w) : 0, pi, khi, klo);
+            }
+        } else if constexpr (PREC == MD_PREC_FP64) {
+            double krho = 0.0, kep = 0.0;
+#pragma unroll 1
+            for (int sub = 0; sub < T && g0 + sub * stride < items; sub++) {
+                double rho, ep;
+                density64_sum<T, KIND, MULTI>(A, P, boxes, g0 + sub * stride, energy, rho, ep);
+                b.take(krho, rho, sub);
+                if (KEEP) b.take(kep, ep, sub);
+            }
+            const int i = b.atom(stride, items, A.n);
+            if (i >= 0) density64_finish<KEEP>(A, P, i, MULTI ? A.spec[i] : 0, krho, kep);
+        } else if constexpr (KIND == MD_POT_TABLES && !MULTI) {
+            df::F2 krho = df::make(0.f), kep = krho;
+#pragma unroll 1
+            for (int sub = 0; sub < T && g0 + sub * stride < items; sub++) {
+                df::F2 rho, ep;
+                density_df_sum<T>(A, P, boxes, g0 + sub * stride, energy, rho, ep);
+                b.take(krho.h, rho.h, sub);
+                b.take(krho.l, rho.l, sub);
+                if (KEEP) {
+                    b.take(kep.h, ep.h, sub);
+                    b.take(kep.l, ep.l, sub);
+                }
+            }
+            const int i = b.atom(stride, items, A.n);
+            if (i >= 0) density_df_finish<KEEP>(A, P, i, krho, kep);
+        }
+    }
+}
+
+// open: see close_step.
+template <int PREC, int T, int KIND, bool MULTI, bool SMT, bool ENERGY>
+__device__ __forceinline__ void force_walk(const Atoms &A, const Pot &P, const Box *boxes, const StepParams &sp,
+                                           long long tid, long long stride, long long items, bool open,
+                                           double (&part)[kPartials]) {
+    for (long long g0 = tid; g0 < items; g0 += stride * T) {
+        const Batch<T> b(g0);
+        if constexpr (PREC == MD_PREC_MIXED) {
+            Acc32 k;
+#pragma unroll 1
+            for (int sub = 0; sub < T && g0 + sub * stride < items; sub++) {
+                Acc32 a;
+                force32_sum<T, KIND, MULTI, ENERGY, SMT>(A, P, boxes, g0 + sub * stride, a);
+                b.take(k.fx, a.fx, sub);
+                b.take(k.fy, a.fy, sub);
+                b.take(k.fz, a.fz, sub);
+                if (ENERGY) {
+                    b.take(k.ep, a.ep, sub);
+                    b.take(k.wxx, a.wxx, sub); b.take(k.wyy, a.wyy, sub); b.take(k.wzz, a.wzz, sub);
+                    b.take(k.wyz, a.wyz, sub); b.take(k.wxz, a.wxz, sub); b.take(k.wxy, a.wxy, sub);
+                }
+            }
+            const int i = b.atom(stride, items, A.n);
+            if (i >= 0) {
+                // (an infinite sum becomes NaN here: not finite either way)
+                const double4_32a v = close_step(A, boxes, sp, i, f64_of_f32(k.fx), f64_of_f32(k.fy), f64_of_f32(k.fz), open);
+                if (ENERGY) {
+                    const double e = A.e_atom[i] + (double)k.ep;
+                    A.e_atom[i] = e;
+                    add_partials(part, e, v, k);
+                }
+            }
+        } else {
+            Acc64 k;
+#pragma unroll 1
+            for (int sub = 0; sub < T && g0 + sub * stride < items; sub++) {
+                Acc64 a;
+                if constexpr (PREC == MD_PREC_FP64) force64_sum<T, KIND, MULTI, ENERGY>(A, P, boxes, g0 + sub * stride, a);
+                else if constexpr (KIND == MD_POT_TABLES && !MULTI) force_df_sum<T, ENERGY>(A, P, boxes, g0 + sub * stride, a);
+                b.take(k.fx, a.fx, sub);
+                b.take(k.fy, a.fy, sub);
+                b.take(k.fz, a.fz, sub);
+                if (ENERGY) {
+                    b.take(k.ep, a.ep, sub);
+                    b.take(k.wxx, a.wxx, sub); b.take(k.wyy, a.wyy, sub); b.take(k.wzz, a.wzz, sub);
+                    b.take(k.wyz, a.wyz, sub); b.take(k.wxz, a.wxz, sub); b.take(k.wxy, a.wxy, sub);
+                }
+            }
+            const int i = b.atom(stride, items, A.n);
+            if (i >= 0) {
+                const double4_32a v = close_step(A, boxes, sp, i, k.fx, k.fy, k.fz, open);
+                if (ENERGY) {
+                    const double e = A.e_atom[i] + k.ep;
+                    A.e_atom[i] = e;
+                    add_partials(part, e, v, k);
+                }
+            }
+        }
     }
 }
 

@@ -10,6 +10,7 @@
 
 #include <cuda_runtime.h>
 
+#include "md_bits.cuh"
 #include "md_internal.cuh"
 
 namespace mdk {
@@ -29,20 +30,7 @@ __device__ __forceinline__ int cell_coord(double x, double invL, int nc) {
     return min(max(c, 0), nc - 1);
 }
 
-__device__ __forceinline__ float wrap1(double x, double L, double invL) {
-    return (float)(x - L * floor(x * invL));
-}
-
-__device__ __forceinline__ float4 wrapped(const double4_32a &p, const Box &B, int species) {
-    return make_float4(wrap1(p.x, B.L[0], B.invL[0]), wrap1(p.y, B.L[1], B.invL[1]),
-                       wrap1(p.z, B.L[2], B.invL[2]), __int_as_float(species));
-}
-
-// FP64 positions wrapped into the box, and in the image of the last build (as below).
-__device__ __forceinline__ double4_32a wrapped64(const double4_32a &p, const Box &B) {
-    return make_double4_32a(p.x - B.L[0] * floor(p.x * B.invL[0]), p.y - B.L[1] * floor(p.y * B.invL[1]),
-                            p.z - B.L[2] * floor(p.z * B.invL[2]), p.w);
-}
+// Positions in the image of the last build (ref: the position at that build), FP64 and FP32.
 __device__ __forceinline__ double4_32a build_image64(const double4_32a &p, const double4_32a &ref, const Box &B) {
     return make_double4_32a(p.x - B.L[0] * floor(ref.x * B.invL[0]), p.y - B.L[1] * floor(ref.y * B.invL[1]),
                             p.z - B.L[2] * floor(ref.z * B.invL[2]), p.w);
@@ -60,12 +48,22 @@ __device__ __forceinline__ float4 build_image(const double4_32a &p, const double
 }
 
 // Double-float copy of an FP64 image coordinate q (MD_PREC_DF): q + xoff split into an FP32 high
-// part and the FP32 rounding of the remainder.
+// part and the FP32 rounding of the remainder (conversions on the bit fields).
 __device__ __forceinline__ void store_dfpos(const Atoms &A, int i, const double4_32a &q, const Box &B) {
     const double x = q.x + B.xoff[0], y = q.y + B.xoff[1], z = q.z + B.xoff[2];
-    const float xh = (float)x, yh = (float)y, zh = (float)z;
+    const float xh = eam::f32_rn(x), yh = eam::f32_rn(y), zh = eam::f32_rn(z);
     A.posx[2 * (size_t)i] = make_float4(xh, yh, zh, 0.f);
-    A.posx[2 * (size_t)i + 1] = make_float4((float)(x - (double)xh), (float)(y - (double)yh), (float)(z - (double)zh), 0.f);
+    A.posx[2 * (size_t)i + 1] = make_float4(eam::f32_rn(x - eam::f64_of_f32(xh)), eam::f32_rn(y - eam::f64_of_f32(yh)),
+                                            eam::f32_rn(z - eam::f64_of_f32(zh)), 0.f);
+}
+
+// The whole box edges to take off per axis, floor(r / L), as three signed 10-bit fields (0: none, as
+// for most atoms); kImageFar where one does not fit.
+constexpr int kImageFar = (int)0x80000000;
+__device__ __forceinline__ int pack_image(double fx, double fy, double fz) {
+    const float x = eam::f32_rn(fx), y = eam::f32_rn(fy), z = eam::f32_rn(fz);   // whole numbers: exact where they fit
+    if (!(fabsf(x) < 512.f && fabsf(y) < 512.f && fabsf(z) < 512.f)) return kImageFar;
+    return (((int)x & 1023) << 20) | (((int)y & 1023) << 10) | ((int)z & 1023);
 }
 
 __device__ __forceinline__ int global_cell(const double4_32a &p, const Box &B, const RepCells &g) {
@@ -103,10 +101,64 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_sums, int &
 }
 
 // ---------------------------------------------------------------- integration (§2.3, §2.2)
-// v += (dt/2) F/m;  r += dt v;  [z *= s];  skin check against the positions of the last build.
-// Separately rounded FP64 operations, as in the definition.
+// The exact displacement check: an atom more than skin/2 from its position at the last build (or
+// not finite) asks for a rebuild.
+__device__ __forceinline__ void check_exact(const Atoms &A, const double4_32a &p, const double4_32a &r, double lim2) {
+    const double ex = __dsub_rn(p.x, r.x), ey = __dsub_rn(p.y, r.y), ez = __dsub_rn(p.z, r.z);
+    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
+    if (d2 > lim2 || !(d2 == d2)) {
+        A.flags->need_rebuild = 1;
+        A.flags->skin_exceeded = 1;
+    }
+}
+
+// What follows a move of atom i to p: the skin check and the copies of the position that the
+// passes read, in the periodic image of the last build.  The FP64 pipe bounds the per-atom work
+// (see md_bits.cuh), so without a strain ramp (A.image_fixed) none of this runs on it for most
+// atoms: the box edges to take off come from the build (reff.w, 0 for most), the FP32 copy is
+// rounded on the bit fields, and the displacement is first formed from the FP32 positions, the
+// exact check following only where that lies within its rounding of the limit (lim.d2f).  The
+// copies, and the decision, are the same bits as with the exact operations throughout.
+__device__ __forceinline__ void place(const Atoms &A, const Box *boxes, int i, const double4_32a &p, SkinLimit lim) {
+    if (!A.image_fixed) {
+        const double4_32a r = A.ref[i];
+        check_exact(A, p, r, lim.d2);
+        const Box &B = boxes[replica_of(A, i)];
+        A.posf[i] = build_image(p, r, B, A.spec[i]);
+        if (A.posd) {
+            const double4_32a q = build_image64(p, r, B);
+            A.posd[i] = q;
+            if (A.posx) store_dfpos(A, i, q, B);
+        }
+        return;
+    }
+    const float4 rf = A.reff[i];
+    const int im = __float_as_int(rf.w);
+    double4_32a q = p;
+    if (im != 0) {
+        const Box &B = boxes[replica_of(A, i)];
+        if (im == kImageFar) {
+            q = build_image64(p, A.ref[i], B);
+        } else {   // small whole numbers, exact through FP32
+            q.x = fma(-B.L[0], eam::f64_of_f32((float)((im << 2) >> 22)), p.x);
+            q.y = fma(-B.L[1], eam::f64_of_f32((float)((im << 12) >> 22)), p.y);
+            q.z = fma(-B.L[2], eam::f64_of_f32((float)((im << 22) >> 22)), p.z);
+        }
+    }
+    const float fx = eam::f32_rn(q.x), fy = eam::f32_rn(q.y), fz = eam::f32_rn(q.z);
+    const float ex = fx - rf.x, ey = fy - rf.y, ez = fz - rf.z;
+    if (!(fmaf(ex, ex, fmaf(ey, ey, ez * ez)) <= lim.d2f)) check_exact(A, p, A.ref[i], lim.d2);
+    A.posf[i] = make_float4(fx, fy, fz, __int_as_float(A.spec[i]));
+    if (A.posd) {
+        A.posd[i] = q;
+        if (A.posx) store_dfpos(A, i, q, boxes[replica_of(A, i)]);
+    }
+}
+
+// v += (dt/2) F/m;  r += dt v;  [z *= s];  then place().  Separately rounded FP64 operations, as in
+// the definition.
 __device__ __forceinline__ void kick_drift(const Atoms &A, const Box *boxes, int i, double half_dt, double dt,
-                                           double s, bool strain, double lim2, const Thermo *th = nullptr) {
+                                           double s, bool strain, SkinLimit lim, const Thermo *th = nullptr) {
     double4_32a v = A.vel[i];
     if (th) {  // the thermostat half steps before this kick: v *= s_b, then v *= s_a
         const Thermo &t = th[replica_of(A, i)];
@@ -125,27 +177,14 @@ __device__ __forceinline__ void kick_drift(const Atoms &A, const Box *boxes, int
     if (strain) p.z = __dmul_rn(p.z, s);
     A.vel[i] = v;
     A.pos[i] = p;
-    const double4_32a r = A.ref[i];
-    const double ex = __dsub_rn(p.x, r.x), ey = __dsub_rn(p.y, r.y), ez = __dsub_rn(p.z, r.z);
-    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
-    if (d2 > lim2 || !(d2 == d2)) {
-        A.flags->need_rebuild = 1;
-        A.flags->skin_exceeded = 1;
-    }
-    A.posf[i] = build_image(p, r, boxes[replica_of(A, i)], A.spec[i]);
-    if (A.posd) {
-        const Box &B = boxes[replica_of(A, i)];
-        const double4_32a q = build_image64(p, r, B);
-        A.posd[i] = q;
-        if (A.posx) store_dfpos(A, i, q, B);
-    }
+    place(A, boxes, i, p, lim);
 }
 
 // The predictor of the third-order predictor-corrector (md.h MD_INTEGRATOR_PC3): from the force f
 // of the last evaluation (acceleration term q2 = (dt^2/2) f/m) and the third-derivative term q3,
 //   r += dt v + q2 + q3,  v += (2 q2 + 3 q3) / dt,  g2 = q2 + 3 q3 (the predicted acceleration
 // term, for the corrector), then the skin check and the pass copies, as after a drift.
-__device__ __forceinline__ void predict_pc3(const Atoms &A, const Box *boxes, int i, double dt, double lim2) {
+__device__ __forceinline__ void predict_pc3(const Atoms &A, const Box *boxes, int i, double dt, SkinLimit lim) {
     double4_32a v = A.vel[i], p = A.pos[i];
     const double4_32a f = A.force[i], q3 = A.g3[i];
     const double h2 = 0.5 * dt * dt;
@@ -161,37 +200,24 @@ __device__ __forceinline__ void predict_pc3(const Atoms &A, const Box *boxes, in
     A.g2[i] = make_double4_32a(__dadd_rn(ax, bx), __dadd_rn(ay, by), __dadd_rn(az, bz), 0.0);
     A.vel[i] = v;
     A.pos[i] = p;
-    const double4_32a r = A.ref[i];
-    const double ex = __dsub_rn(p.x, r.x), ey = __dsub_rn(p.y, r.y), ez = __dsub_rn(p.z, r.z);
-    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
-    if (d2 > lim2 || !(d2 == d2)) {
-        A.flags->need_rebuild = 1;
-        A.flags->skin_exceeded = 1;
-    }
-    A.posf[i] = build_image(p, r, boxes[replica_of(A, i)], A.spec[i]);
-    if (A.posd) {
-        const Box &B = boxes[replica_of(A, i)];
-        const double4_32a q = build_image64(p, r, B);
-        A.posd[i] = q;
-        if (A.posx) store_dfpos(A, i, q, B);
-    }
+    place(A, boxes, i, p, lim);
 }
 
 // What opens a step: the half kick and drift of velocity Verlet, or the predictor.
 __device__ __forceinline__ void open_step(const Atoms &A, const Box *boxes, int i, int motion, double half_dt,
-                                          double dt, double s, bool strain, double lim2, const Thermo *th = nullptr) {
-    if (motion == kMotionPC3) predict_pc3(A, boxes, i, dt, lim2);
-    else kick_drift(A, boxes, i, half_dt, dt, s, strain, lim2, th);
+                                          double dt, double s, bool strain, SkinLimit lim, const Thermo *th = nullptr) {
+    if (motion == kMotionPC3) predict_pc3(A, boxes, i, dt, lim);
+    else kick_drift(A, boxes, i, half_dt, dt, s, strain, lim, th);
 }
 
-__device__ __forceinline__ void check_displacement(const Atoms &A, int i, double lim2) {
-    const double4_32a p = A.pos[i], r = A.ref[i];
-    const double ex = __dsub_rn(p.x, r.x), ey = __dsub_rn(p.y, r.y), ez = __dsub_rn(p.z, r.z);
-    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
-    if (d2 > lim2 || !(d2 == d2)) {
-        A.flags->need_rebuild = 1;
-        A.flags->skin_exceeded = 1;
+// The displacement check of positions already placed (posf current: not after a corrector).
+__device__ __forceinline__ void check_displacement(const Atoms &A, int i, SkinLimit lim) {
+    if (A.image_fixed && !A.g3) {
+        const float4 f = A.posf[i], rf = A.reff[i];
+        const float ex = f.x - rf.x, ey = f.y - rf.y, ez = f.z - rf.z;
+        if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) <= lim.d2f) return;
     }
+    check_exact(A, A.pos[i], A.ref[i], lim.d2);
 }
 
 // ---------------------------------------------------------------- rebuild (§3.2.1, §3.2.2)
@@ -339,10 +365,14 @@ __device__ __forceinline__ void copyback_atom(const Atoms &A, const Box *boxes, 
         A.g2[k] = A.g2_tmp[k];
         A.g3[k] = A.g3_tmp[k];
     }
-    A.posf[k] = wrapped(p, boxes[replica_of(A, k)], sp);
+    // wrapped into the box: p - L floor(p / L), its FP32 rounding, and the floors for place()
+    const Box &B = boxes[replica_of(A, k)];
+    const double fx = floor(p.x * B.invL[0]), fy = floor(p.y * B.invL[1]), fz = floor(p.z * B.invL[2]);
+    const double4_32a q = make_double4_32a(fma(-B.L[0], fx, p.x), fma(-B.L[1], fy, p.y), fma(-B.L[2], fz, p.z), p.w);
+    const float4 f = make_float4(eam::f32_rn(q.x), eam::f32_rn(q.y), eam::f32_rn(q.z), __int_as_float(sp));
+    A.posf[k] = f;
+    A.reff[k] = make_float4(f.x, f.y, f.z, __int_as_float(pack_image(fx, fy, fz)));
     if (A.posd) {
-        const Box &B = boxes[replica_of(A, k)];
-        const double4_32a q = wrapped64(p, B);
         A.posd[k] = q;
         if (A.posx) store_dfpos(A, k, q, B);
     }

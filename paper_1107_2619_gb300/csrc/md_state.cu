@@ -9,10 +9,10 @@ namespace mdk {
 
 namespace {
 
-__global__ void k_check_displacement(Atoms A, double lim2) {
+__global__ void k_check_displacement(Atoms A, SkinLimit lim) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= A.n) return;
-    ph::check_displacement(A, i, lim2);
+    ph::check_displacement(A, i, lim);
 }
 
 __global__ void k_wrap(Atoms A) {
@@ -178,9 +178,9 @@ cudaError_t launch_replica_sums(const Atoms &A, const int32_t *off, int n_rep, d
     return cudaGetLastError();
 }
 
-cudaError_t launch_check_displacement(const Atoms &A, double lim2, cudaStream_t s) {
+cudaError_t launch_check_displacement(const Atoms &A, SkinLimit lim, cudaStream_t s) {
     if (A.n == 0) return cudaSuccess;
-    k_check_displacement<<<blocks_for(A.n, kThreads), kThreads, 0, s>>>(A, lim2);
+    k_check_displacement<<<blocks_for(A.n, kThreads), kThreads, 0, s>>>(A, lim);
     return cudaGetLastError();
 }
 

@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
             MD_SYNC();
         }
         for (long long i = tid; i < A.n; i += stride) {
-            ph::open_step(A, boxes, (int)i, sp.motion, sp.half_dt, sp.dt, sp.strain_scale, strain, sp.lim2,
+            ph::open_step(A, boxes, (int)i, sp.motion, sp.half_dt, sp.dt, sp.strain_scale, strain, sp.lim,
                           thermo ? sp.thermo : nullptr);
             if constexpr (WALK == kWalkHalf) A.rho_acc[i] = 0.0;
         }
@@ -408,14 +408,20 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
             }
         }
         const bool energy_step = s == sp.n_steps - 1 && sp.energy_last;
+        // the per-atom results (rho, F', energies) are stored on the call's last step only
         if constexpr (WALK == kWalkPairs) {   // each pair once, then F(rho) once every share is in
             for (long long g = tid; g < items; g += stride)
                 ps::density64_pairs<T, KIND>(A, P, boxes, g, energy_step, psum);
             MD_SYNC();
-            for (long long i = tid; i < A.n; i += stride) ps::pairs_embed64(A, P, (int)i);
+            if (s == sp.n_steps - 1)
+                for (long long i = tid; i < A.n; i += stride) ps::pairs_embed64<true>(A, P, (int)i);
+            else
+                for (long long i = tid; i < A.n; i += stride) ps::pairs_embed64<false>(A, P, (int)i);
         } else if (!tiled) {
-            for (long long g = tid; g < items; g += stride)
-                ps::density_item<PREC, T, KIND, MULTI, SMT>(A, P, boxes, g, energy_step);
+            if (s == sp.n_steps - 1)
+                ps::density_walk<PREC, T, KIND, MULTI, SMT, true>(A, P, boxes, tid, stride, items, energy_step);
+            else
+                ps::density_walk<PREC, T, KIND, MULTI, SMT, false>(A, P, boxes, tid, stride, items, false);
         }
         MD_SYNC();
         MD_STAMP(10);
@@ -446,7 +452,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
                                 for (int c = tl::claim(pipe, b, 1); c < G.h1 - G.h0; c = tl::claim(pipe, b, 1))
                                     tl::force_cell_atom<KIND, true, SMT>(A, P, boxes, st, pipe.loc[b], C.gx + 2, G,
                                                                          G.h0 + c, cells_q[threadIdx.x >> 5], sp.half_dt,
-                                                                         sp.dt, sp.lim2, false, part);
+                                                                         sp.dt, sp.lim, false, part);
                             } else {
                                 const int gi = ((G.h1 - G.h0) * T + 31) & ~31;
                                 for (int c = tl::claim(pipe, b, 32); c < gi; c = tl::claim(pipe, b, 32)) {
@@ -473,10 +479,9 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
                 for (long long g = tid; g < items; g += stride)
                     ps::force64_pairs<T, KIND, true>(A, P, boxes, g, part, psum);
                 MD_SYNC();
-                for (long long i = tid; i < A.n; i += stride) ps::pairs_kick64<true>(A, (int)i, sp.half_dt, sp.motion, part);
+                for (long long i = tid; i < A.n; i += stride) ps::pairs_close64<true>(A, boxes, sp, (int)i, false, part);
             } else if (!tiled) {
-                for (long long g = tid; g < items; g += stride)
-                    ps::force_item<PREC, T, KIND, MULTI, true, SMT>(A, P, boxes, g, sp.half_dt, sp.motion, part);
+                ps::force_walk<PREC, T, KIND, MULTI, SMT, true>(A, P, boxes, sp, tid, stride, items, false, part);
             }
             eam::block_partials<NT>(part, A.partials, A.part_stride);
         } else {
@@ -494,7 +499,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
                                 for (int c = tl::claim(pipe, b, 1); c < G.h1 - G.h0; c = tl::claim(pipe, b, 1))
                                     tl::force_cell_atom<KIND, false, SMT>(A, P, boxes, st, pipe.loc[b], C.gx + 2, G,
                                                                          G.h0 + c, cells_q[threadIdx.x >> 5], sp.half_dt,
-                                                                         sp.dt, sp.lim2, fuse, part);
+                                                                         sp.dt, sp.lim, fuse, part);
                             } else {
                                 const int gi = ((G.h1 - G.h0) * T + 31) & ~31;
                                 for (int c = tl::claim(pipe, b, 32); c < gi; c = tl::claim(pipe, b, 32)) {
@@ -504,7 +509,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
                                             A, P, st, G.h1, G.h0 + it / T, it & (T - 1), sp.half_dt, true, part);
                                         if (fuse && i >= 0)
                                             ph::kick_drift(A, boxes, i, sp.half_dt, sp.dt, sp.strain_scale, false,
-                                                           sp.lim2);
+                                                           sp.lim);
                                     } else {
                                         tl::force_half_item<T, KIND, false, SMT>(A, P, st, half_acc + (size_t)b * C.cap,
                                                                                  G.h1, G.h0 + it / T, it & (T - 1), part);
@@ -519,7 +524,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
                         MD_SYNC();
                         for (long long i = tid; i < A.n; i += stride) {
                             tl::half_kick<false>(A, (int)i, sp.half_dt, part);
-                            if (fuse) ph::kick_drift(A, boxes, (int)i, sp.half_dt, sp.dt, sp.strain_scale, false, sp.lim2);
+                            if (fuse) ph::kick_drift(A, boxes, (int)i, sp.half_dt, sp.dt, sp.strain_scale, false, sp.lim);
                         }
                     }
                 }
@@ -528,17 +533,9 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
                 for (long long g = tid; g < items; g += stride)
                     ps::force64_pairs<T, KIND, false>(A, P, boxes, g, part, psum);
                 MD_SYNC();
-                for (long long i = tid; i < A.n; i += stride) {
-                    ps::pairs_kick64<false>(A, (int)i, sp.half_dt, sp.motion, part);
-                    if (fuse) ph::open_step(A, boxes, (int)i, sp.motion, sp.half_dt, sp.dt, sp.strain_scale, false, sp.lim2);
-                }
+                for (long long i = tid; i < A.n; i += stride) ps::pairs_close64<false>(A, boxes, sp, (int)i, fuse, part);
             } else if (!tiled) {
-                for (long long g = tid; g < items; g += stride) {
-                    const int i = ps::force_item<PREC, T, KIND, MULTI, false, SMT>(A, P, boxes, g, sp.half_dt,
-                                                                                   sp.motion, part);
-                    if (fuse && i >= 0)
-                        ph::open_step(A, boxes, i, sp.motion, sp.half_dt, sp.dt, sp.strain_scale, false, sp.lim2);
-                }
+                ps::force_walk<PREC, T, KIND, MULTI, SMT, false>(A, P, boxes, sp, tid, stride, items, fuse, part);
             }
         }
         MD_SYNC();
@@ -555,7 +552,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
             MD_SYNC();
             if (!last) {
                 for (long long i = tid; i < A.n; i += stride)
-                    ph::kick_drift(A, boxes, (int)i, sp.half_dt, sp.dt, sp.strain_scale, strain, sp.lim2, sp.thermo);
+                    ph::kick_drift(A, boxes, (int)i, sp.half_dt, sp.dt, sp.strain_scale, strain, sp.lim, sp.thermo);
                 MD_SYNC();
             } else {
                 for (long long i = tid; i < A.n; i += stride) {
@@ -574,7 +571,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
             }
             MD_SYNC();
             for (long long i = tid; i < A.n; i += stride)
-                ph::kick_drift(A, boxes, (int)i, sp.half_dt, sp.dt, sp.strain_scale, true, sp.lim2);
+                ph::kick_drift(A, boxes, (int)i, sp.half_dt, sp.dt, sp.strain_scale, true, sp.lim);
             MD_SYNC();
         }
     }

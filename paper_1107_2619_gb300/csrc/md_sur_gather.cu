@@ -293,10 +293,10 @@ __global__ void k_sur_stats(Atoms A, SurNet S, double *part) {
     }
 }
 
-__global__ void k_sur_kick_drift(Atoms A, double half_dt, double dt, double lim2) {
+__global__ void k_sur_kick_drift(Atoms A, double half_dt, double dt, SkinLimit lim) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= A.n) return;
-    ph::kick_drift(A, A.boxes, i, half_dt, dt, 1.0, false, lim2);
+    ph::kick_drift(A, A.boxes, i, half_dt, dt, 1.0, false, lim);
 }
 
 // Rows of 32 floats from cell order back to the caller's order.
@@ -313,9 +313,9 @@ int gather_blocks(int n_atoms) { return std::max(1, std::min(blocks_for(n_atoms,
 
 int sur_force_blocks(int n_atoms) { return gather_blocks(n_atoms); }
 
-cudaError_t launch_sur_kick_drift(const Atoms &A, double half_dt, double dt, double lim2, cudaStream_t s) {
+cudaError_t launch_sur_kick_drift(const Atoms &A, double half_dt, double dt, SkinLimit lim, cudaStream_t s) {
     if (A.n == 0) return cudaSuccess;
-    k_sur_kick_drift<<<blocks_for(A.n, kThreads), kThreads, 0, s>>>(A, half_dt, dt, lim2);
+    k_sur_kick_drift<<<blocks_for(A.n, kThreads), kThreads, 0, s>>>(A, half_dt, dt, lim);
     return cudaGetLastError();
 }
 

@@ -488,7 +488,7 @@ __device__ __forceinline__ void density_cell_atom(const Atoms &A, const Pot &P, 
 template <int KIND, bool ENERGY, bool SMT>
 __device__ __forceinline__ void force_cell_atom(const Atoms &A, const Pot &P, const Box *boxes, const float4 *st,
                                                 const int *loc, int W, const Group &G, int i, uint16_t *q,
-                                                double half_dt, double dt, double lim2, bool fuse,
+                                                double half_dt, double dt, SkinLimit lim, bool fuse,
                                                 double (&part)[kPartials]) {
     const int lane = threadIdx.x & 31;
     const int si = loc[4 * W + 1] + (i - G.h0);
@@ -502,7 +502,7 @@ __device__ __forceinline__ void force_cell_atom(const Atoms &A, const Pot &P, co
     ps::lane_sum_acc<32, ENERGY>(a);
     if (lane == 0) {
         ps::force32_finish<ENERGY>(A, i, a, half_dt, true, part);
-        if (fuse) ph::kick_drift(A, boxes, i, half_dt, dt, 1.0, false, lim2);
+        if (fuse) ph::kick_drift(A, boxes, i, half_dt, dt, 1.0, false, lim);
     }
 }
 
