@@ -410,7 +410,6 @@ cudaError_t launch_sur_pack(const float *theta, unsigned char *img, cudaStream_t
 cudaError_t launch_sur_stats(const Atoms &A, const SurNet &S, double *part, int blocks, cudaStream_t s);
 cudaError_t launch_sur_unsort_rows(const Atoms &A, const float *src, float *dst, cudaStream_t s);
 int sur_net32_blocks(int n_atoms);
-int sur_force_blocks(int n_atoms);
 
 inline int blocks_for(long long n, int threads) { return (int)((n + threads - 1) / threads); }
 

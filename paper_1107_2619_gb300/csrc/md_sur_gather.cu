@@ -2,8 +2,9 @@
 // descriptor tangent used by the force term of the training loss.  One warp per atom, lane k
 // = radial-basis channel k (32 channels = 32 lanes).  The lanes first evaluate the geometry of
 // 32 list entries at once (lane q: entry q), stage it in shared memory, and then all lanes walk
-// the entries inside the descriptor cutoff, each adding its own channel.  The per-channel
-// quantities of neighbour j (its gradient row g_j) are then one coalesced 128-byte row read.
+// the entries inside the descriptor cutoff two at a time (packed FP32 operations), each adding its
+// own channel.  The per-channel quantities of neighbour j (its gradient row g_j) are then one
+// coalesced 128-byte row read.
 //
 //   descriptors  G_ik = sum_j b_k(r_ij)
 //   forces       F_i  = sum_j [ sum_k (g_ik + g_jk) b_k'(r_ij) ] (r_j - r_i) / r_ij
@@ -22,21 +23,102 @@ namespace {
 
 constexpr int kWarps = kThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
+constexpr float kLog2e = 1.4426950408889634f;
 
 __device__ __forceinline__ float mi(float d, float L, float iL) { return d - L * rintf(d * iL); }
 
-// Per-pair constants of one chunk of list entries, compacted: the pairs inside rd occupy
-// slots 0 .. n-1 in list order.  P0 = (r, fc, fc', j bits), P1 = (unit vector, fc / w^2).
+// Two FP32 values in one 64-bit register pair and the packed operations on them (PTX f32x2: each
+// half rounded as the scalar operation), which halve the issue slots of the channel loops: those
+// bound these kernels.  The halves are two consecutive pairs of the row.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pack(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack(F2 x, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v)); }
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ float both(F2 x) {
+    float a, b;
+    unpack(x, a, b);
+    return a + b;
+}
+
+// 2^x (PTX ex2.approx.ftz: relative error < 2^-22).
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ F2 ex2_2(F2 x) {
+    float a, b;
+    unpack(x, a, b);
+    return pack(ex2(a), ex2(b));
+}
+
+__device__ __forceinline__ float warp_sum(float x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+    return x;
+}
+
+// The warp sums of four values with six shuffles instead of twenty: each of the first two rounds
+// halves the values a lane carries; lane l ends with the sum of value l & 3.
+__device__ __forceinline__ float warp_sum4(float a, float b, float c, float d) {
+    const int lane = threadIdx.x & 31;
+    const bool o1 = lane & 1, o2 = lane & 2;
+    float x = o1 ? b : a, y = o1 ? d : c;
+    x += __shfl_xor_sync(kFull, o1 ? a : b, 1);
+    y += __shfl_xor_sync(kFull, o1 ? c : d, 1);
+    float z = o2 ? y : x;
+    z += __shfl_xor_sync(kFull, o2 ? x : y, 2);
+    z += __shfl_xor_sync(kFull, z, 4);
+    z += __shfl_xor_sync(kFull, z, 8);
+    z += __shfl_xor_sync(kFull, z, 16);
+    return z;
+}
+
+// Per-pair constants of one chunk of 32 list entries, compacted: the pairs inside rd take slots
+// 0 .. n-1 in list order, two slots to a block whose words lie in the order the packed loops read
+// them (value f of slot s at word (s / 2) kBlk + 2 f + (s & 1); kBlk = 4 (2 m + 1) words keeps the
+// 16-byte reads aligned and the scattered stores two to a bank).  An odd n is filled up with a
+// slot of zeros.
+template <int NF>
 struct Stage {
-    float4 P0[kWarps][32];
-    float4 P1[kWarps][32];
+    static constexpr int kBlk = (NF + 1) / 2 * 4 % 8 ? (NF + 1) / 2 * 4 : (NF + 1) / 2 * 4 + 4;
+    float4 w[16 * kBlk / 4];
+    __device__ __forceinline__ void put(int s, int f, float v) {
+        reinterpret_cast<float *>(w)[(s >> 1) * kBlk + 2 * f + (s & 1)] = v;
+    }
+    // values f and f + 1 (f even) of block b, each as its two slots
+    __device__ __forceinline__ void get2(int b, int f, F2 &x, F2 &y) const {
+        const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(&w[(b * kBlk + 2 * f) / 4]);
+        x.v = q.x;
+        y.v = q.y;
+    }
 };
 
-// Geometry of list entries [base, base + 32) of atom i into the compacted slots; returns the
-// number of pairs inside rd.
+// Geometry of list entries [base, base + 32) of an atom at pi: lane q takes entry base + q; inside
+// rd, fn(slot, r, 1/r, d, j) with the compacted slot.  Returns the number of pairs inside.
+template <typename Fn>
 __device__ __forceinline__ int stage_chunk(const Atoms &A, const SurNet &S, const float4 &pi, const Box &B,
-                                           const NbrRow &row, int cnt, int base, int lane, float4 *P0,
-                                           float4 *P1) {
+                                           const NbrRow &row, int cnt, int base, int lane, Fn &&fn) {
     const int q = base + lane;
     const bool valid = q < cnt;
     const int j = valid ? __ldg(row.ptr(q)) : 0;
@@ -49,31 +131,24 @@ __device__ __forceinline__ int stage_chunk(const Atoms &A, const SurNet &S, cons
     const unsigned m = __ballot_sync(kFull, inside);
     if (inside) {
         const float rinv = rsqrtf(r2);
-        const float r = r2 * rinv;
-        float sn, cs;
-        __sincosf(S.pi_rd * r, &sn, &cs);
-        const float fc = 0.5f * (cs + 1.f);
-        const int slot = __popc(m & ((1u << lane) - 1u));
-        P0[slot] = make_float4(r, fc, -0.5f * S.pi_rd * sn, __int_as_float(j));
-        P1[slot] = make_float4(dx * rinv, dy * rinv, dz * rinv, fc * S.invw2);
+        fn(__popc(m & ((1u << lane) - 1u)), r2 * rinv, rinv, dx, dy, dz, j);
     }
-    __syncwarp();
     return __popc(m);
 }
-
-// 2^x (PTX ex2.approx.ftz: relative error < 2^-22).
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
+// The cutoff function fc = (cos(pi r / rd) + 1) / 2 and its derivative.
+__device__ __forceinline__ void cutoff(const SurNet &S, float r, float &fc, float &dfc) {
+    float sn, cs;
+    __sincosf(S.pi_rd * r, &sn, &cs);
+    fc = 0.5f * (cs + 1.f);
+    dfc = -0.5f * S.pi_rd * sn;
 }
 
-constexpr float kLog2e = 1.4426950408889634f;
-
-__device__ __forceinline__ float warp_sum(float x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-    return x;
+// A block's atoms: a contiguous range (its warps' neighbourhoods overlap, so the gathered rows stay
+// in L1), dealt to the warps in turn.
+__device__ __forceinline__ void block_range(int a0, int a1, int &b0, int &b1) {
+    const long long n = a1 - a0;
+    b0 = a0 + (int)(n * blockIdx.x / gridDim.x);
+    b1 = a0 + (int)(n * (blockIdx.x + 1) / gridDim.x);
 }
 
 // ---------------------------------------------------------------- descriptors
@@ -81,39 +156,44 @@ __device__ __forceinline__ float warp_sum(float x) {
 // x = (G - gmu) ginv rounded to bf16 in the 128-atom tile layout the MMA reads (S.Gt):
 // tile t = i / 128, row r = i % 128, column k at byte t*8192 + (r/8)*512 + (k/8)*128 + (r%8)*16 + (k%8)*2.
 __global__ void __launch_bounds__(kThreads) k_sur_desc(Atoms A, SurNet S, int a0, int a1, int bf16) {
-    __shared__ Stage st;
+    __shared__ Stage<2> stage[kWarps];   // r, fc
     __shared__ __align__(16) __nv_bfloat16 out[kWarps][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    Stage<2> &st = stage[w];
     const float mu = S.mu0 + S.dmu * (float)lane;
     const float kx = -S.inv2w2 * kLog2e;   // b = 2^(kx a^2) fc
+    const F2 nmu = pack(-mu, -mu), kx2 = pack(kx, kx);
     const float gm = S.gmu[lane], gi = S.ginv[lane];
-    for (long long i0 = a0 + (long long)blockIdx.x * kWarps + w; i0 < a1; i0 += (long long)gridDim.x * kWarps) {
-        const int i = (int)i0;
+    int b0, b1;
+    block_range(a0, a1, b0, b1);
+    for (int i = b0 + w; i < b1; i += kWarps) {
         const Box &B = A.boxes[ph::replica_of(A, i)];
         const float4 pi = A.posf[i];
         const int cnt = min(A.count[i], A.k_max);
         const NbrRow row = nbr_row(A, i);
-        float G = 0.f, G2 = 0.f;
+        F2 G = pack(0.f, 0.f);
         for (int base = 0; base < cnt; base += 32) {
-            const int np = stage_chunk(A, S, pi, B, row, cnt, base, lane, st.P0[w], st.P1[w]);
-            int q = 0;
-            for (; q + 1 < np; q += 2) {
-                const float2 p0 = *reinterpret_cast<const float2 *>(&st.P0[w][q]);
-                const float2 p1 = *reinterpret_cast<const float2 *>(&st.P0[w][q + 1]);
-                const float a0_ = p0.x - mu, a1_ = p1.x - mu;
-                G = fmaf(ex2(kx * a0_ * a0_), p0.y, G);
-                G2 = fmaf(ex2(kx * a1_ * a1_), p1.y, G2);
-            }
-            if (q < np) {
-                const float2 p0 = *reinterpret_cast<const float2 *>(&st.P0[w][q]);
-                const float a0_ = p0.x - mu;
-                G = fmaf(ex2(kx * a0_ * a0_), p0.y, G);
+            const int np = stage_chunk(A, S, pi, B, row, cnt, base, lane,
+                                       [&](int s, float r, float, float, float, float, int) {
+                float fc, dfc;
+                cutoff(S, r, fc, dfc);
+                st.put(s, 0, r);
+                st.put(s, 1, fc);
+            });
+            if (lane < 2 && (np & 1)) st.put(np, lane, 0.f);
+            __syncwarp();
+#pragma unroll 4
+            for (int b = 0; b < (np + 1) >> 1; b++) {
+                F2 r, fc;
+                st.get2(b, 0, r, fc);
+                const F2 a = add2(r, nmu);
+                G = fma2(ex2_2(mul2(mul2(kx2, a), a)), fc, G);
             }
             __syncwarp();
         }
-        G += G2;
+        const float g = both(G);
         if (bf16) {
-            out[w][lane] = __float2bfloat16_rn((G - gm) * gi);
+            out[w][lane] = __float2bfloat16_rn((g - gm) * gi);
             __syncwarp();
             if (lane < 4) {
                 const int r = i & (kSurTile - 1);
@@ -122,78 +202,128 @@ __global__ void __launch_bounds__(kThreads) k_sur_desc(Atoms A, SurNet S, int a0
             }
             __syncwarp();
         } else {
-            S.G[(size_t)i * kSurNb + lane] = G;
+            S.G[(size_t)i * kSurNb + lane] = g;
         }
     }
 }
 
 // ---------------------------------------------------------------- forces (+ kick, partials)
+// Eight lanes take one pair, four channels a lane, so that a warp walks four staged pairs at a time:
+// with a lane per channel the pair's seven constants went to all 32 lanes of every pair, and
+// returning them from shared memory (128 bytes a cycle) bounded the kernel (83 % of the L1's
+// throughput, 0.35 ms for 524,288 bcc Fe atoms); here one read serves four pairs, and four rows g_j
+// come with one 16-byte load a lane.
 // phi_scale > 0 (training): also phi_i = phi_scale (F_i - Fref_i) and part[0] = sum |F_i - Fref_i|^2.
+// What follows an atom's force is FP64 work, which takes the FP64 pipe the same time for one active
+// lane as for 32 (md_bits.cuh): a warp keeps the forces of up to 32 atoms, one per lane, and then
+// finishes them together.
 template <bool ENERGY, bool TRAIN>
-__global__ void __launch_bounds__(kThreads) k_sur_force(Atoms A, SurNet S, int a0, int a1, int kick, double half_dt,
-                                                        float phi_scale) {
-    __shared__ Stage st;
+__global__ void __launch_bounds__(kThreads, 8) k_sur_force(Atoms A, SurNet S, int a0, int a1, int kick, double half_dt,
+                                                           float phi_scale) {
+    constexpr bool VIRIAL = ENERGY && !TRAIN;
+    __shared__ float4 P0[kWarps][32], P1[kWarps][32];   // (r, fc', -fc/w^2, u_x), (u_y, u_z, j bits, 0)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const float mu = S.mu0 + S.dmu * (float)lane;
+    const int k0 = 4 * (lane & 7), grp = lane >> 3;   // this lane's channels k0 .. k0 + 3, its pair of the four
+    const float mu = S.mu0 + S.dmu * (float)k0;
+    const F2 nmu01 = pack(-mu, -(S.mu0 + S.dmu * (float)(k0 + 1)));
+    const F2 nmu23 = pack(-(S.mu0 + S.dmu * (float)(k0 + 2)), -(S.mu0 + S.dmu * (float)(k0 + 3)));
     const float kx = -S.inv2w2 * kLog2e;
+    const F2 kx2 = pack(kx, kx);
     double part[kPartials];
 #pragma unroll
     for (int q = 0; q < kPartials; q++) part[q] = 0.0;
-    for (long long i0 = a0 + (long long)blockIdx.x * kWarps + w; i0 < a1; i0 += (long long)gridDim.x * kWarps) {
-        const int i = (int)i0;
-        const Box &B = A.boxes[ph::replica_of(A, i)];
-        const float4 pi = A.posf[i];
-        const int cnt = min(A.count[i], A.k_max);
-        const NbrRow row = nbr_row(A, i);
-        const float gi = S.g[(size_t)i * kSurNb + lane];
+    int b0, b1;
+    block_range(a0, a1, b0, b1);
+    for (int i0 = b0 + w; i0 < b1; i0 += kWarps * 32) {   // up to 32 atoms i0 + kWarps q, q = 0 .. 31
         float fx = 0.f, fy = 0.f, fz = 0.f;
-        float wxx = 0.f, wyy = 0.f, wzz = 0.f, wyz = 0.f, wxz = 0.f, wxy = 0.f;
-        // one pair: c = (g_ik + g_jk) b_k'(r) (this lane's channel), f += c * unit vector;
-        // on the energy step the virial -1/2 c r u (x) u
-        auto pair = [&](const float4 &p0, const float4 &p1, float gj) {
-            const float a = p0.x - mu;
-            const float bp = ex2(kx * a * a) * fmaf(-a, p1.w, p0.z);   // b_k'(r)
-            const float c = (gi + gj) * bp;
-            fx = fmaf(c, p1.x, fx);
-            fy = fmaf(c, p1.y, fy);
-            fz = fmaf(c, p1.z, fz);
-            if (ENERGY && !TRAIN) {
-                const float h = -0.5f * c * p0.x;
-                wxx = fmaf(h * p1.x, p1.x, wxx);
-                wyy = fmaf(h * p1.y, p1.y, wyy);
-                wzz = fmaf(h * p1.z, p1.z, wzz);
-                wyz = fmaf(h * p1.y, p1.z, wyz);
-                wxz = fmaf(h * p1.x, p1.z, wxz);
-                wxy = fmaf(h * p1.x, p1.y, wxy);
-            }
-        };
-        // the g_j rows of 8 pairs are loaded before any of them is used (8 independent loads in
-        // flight per lane), then the 8 pairs are added
-        constexpr int kBatch = 8;
-        for (int base = 0; base < cnt; base += 32) {
-            const int np = stage_chunk(A, S, pi, B, row, cnt, base, lane, st.P0[w], st.P1[w]);
-            for (int q0 = 0; q0 < np; q0 += kBatch) {
-                float gj[kBatch];
+        float wv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        const int na = min(32, (b1 - i0 + kWarps - 1) / kWarps);
+        for (int q = 0; q < na; q++) {
+            const int i = i0 + kWarps * q;
+            const Box &B = A.boxes[ph::replica_of(A, i)];
+            const float4 pi = A.posf[i];
+            const int cnt = min(A.count[i], A.k_max);
+            const NbrRow row = nbr_row(A, i);
+            const float4 g = __ldg(reinterpret_cast<const float4 *>(S.g + (size_t)i * kSurNb + k0));
+            const F2 gi01 = pack(g.x, g.y), gi23 = pack(g.z, g.w);
+            float sx = 0.f, sy = 0.f, sz = 0.f;
+            float sw[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            for (int base = 0; base < cnt; base += 32) {
+                const int np = stage_chunk(A, S, pi, B, row, cnt, base, lane,
+                                           [&](int s, float r, float rinv, float dx, float dy, float dz, int j) {
+                    float fc, dfc;
+                    cutoff(S, r, fc, dfc);
+                    P0[w][s] = make_float4(r, dfc, -fc * S.invw2, dx * rinv);
+                    P1[w][s] = make_float4(dy * rinv, dz * rinv, __int_as_float(j), 0.f);
+                });
+                const int ng = (np + 3) >> 2;
+                if (lane >= np && lane < 4 * ng) {   // fill the last four up with nothing
+                    P0[w][lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    P1[w][lane] = make_float4(0.f, 0.f, __int_as_float(i), 0.f);
+                }
+                __syncwarp();
+                // c = sum over this lane's channels of (g_ik + g_jk) b_k'(r); f += c u; the g_j rows
+                // of kBatch fours are loaded before any of them is used
+                constexpr int kBatch = 4;
+                for (int q0 = 0; q0 < ng; q0 += kBatch) {
+                    float4 gj[kBatch];
 #pragma unroll
-                for (int u = 0; u < kBatch; u++) {
-                    const int q = min(q0 + u, np - 1);
-                    gj[u] = __ldg(S.g + (size_t)__float_as_int(st.P0[w][q].w) * kSurNb + lane);
+                    for (int u = 0; u < kBatch; u++) {
+                        const int j = __float_as_int(P1[w][4 * min(q0 + u, ng - 1) + grp].z);
+                        gj[u] = __ldg(reinterpret_cast<const float4 *>(S.g + (size_t)j * kSurNb + k0));
+                    }
+#pragma unroll
+                    for (int u = 0; u < kBatch; u++) {
+                        if (q0 + u < ng) {
+                            const float4 p0 = P0[w][4 * (q0 + u) + grp], p1 = P1[w][4 * (q0 + u) + grp];
+                            const F2 r = pack(p0.x, p0.x), dfc = pack(p0.y, p0.y), nw = pack(p0.z, p0.z);
+                            const F2 a01 = add2(r, nmu01), a23 = add2(r, nmu23);
+                            const F2 b01 = mul2(ex2_2(mul2(mul2(kx2, a01), a01)), fma2(a01, nw, dfc));   // b_k'(r)
+                            const F2 b23 = mul2(ex2_2(mul2(mul2(kx2, a23), a23)), fma2(a23, nw, dfc));
+                            const F2 g01 = add2(gi01, pack(gj[u].x, gj[u].y)), g23 = add2(gi23, pack(gj[u].z, gj[u].w));
+                            const float c = both(fma2(g01, b01, mul2(g23, b23)));
+                            sx = fmaf(c, p0.w, sx);
+                            sy = fmaf(c, p1.x, sy);
+                            sz = fmaf(c, p1.y, sz);
+                            if constexpr (VIRIAL) {   // -1/2 c r u (x) u
+                                const float h = -0.5f * c * p0.x, hx = h * p0.w, hy = h * p1.x;
+                                sw[0] = fmaf(hx, p0.w, sw[0]);
+                                sw[1] = fmaf(hy, p1.x, sw[1]);
+                                sw[2] = fmaf(h * p1.y, p1.y, sw[2]);
+                                sw[3] = fmaf(hy, p1.y, sw[3]);
+                                sw[4] = fmaf(hx, p1.y, sw[4]);
+                                sw[5] = fmaf(hx, p1.x, sw[5]);
+                            }
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+            const float t = warp_sum4(sx, sy, sz, VIRIAL ? sw[0] : 0.f);   // lanes 0, 1, 2, 3: x, y, z, xx
+            const float tx = __shfl_sync(kFull, t, 0), ty = __shfl_sync(kFull, t, 1), tz = __shfl_sync(kFull, t, 2);
+            if (lane == q) {
+                fx = tx;
+                fy = ty;
+                fz = tz;
+            }
+            if constexpr (VIRIAL) {
+                const float t1 = warp_sum4(sw[1], sw[2], sw[3], sw[4]), t2 = warp_sum(sw[5]);
+                const float x0 = __shfl_sync(kFull, t, 3);
+                if (lane == q) {
+                    wv[0] = x0;
+                    wv[5] = t2;
                 }
 #pragma unroll
-                for (int u = 0; u < kBatch; u++)
-                    if (q0 + u < np) pair(st.P0[w][q0 + u], st.P1[w][q0 + u], gj[u]);
+                for (int v = 0; v < 4; v++) {
+                    const float x = __shfl_sync(kFull, t1, v);
+                    if (lane == q) wv[1 + v] = x;
+                }
             }
-            __syncwarp();
         }
-        fx = warp_sum(fx);
-        fy = warp_sum(fy);
-        fz = warp_sum(fz);
-        if (ENERGY && !TRAIN) {
-            wxx = warp_sum(wxx); wyy = warp_sum(wyy); wzz = warp_sum(wzz);
-            wyz = warp_sum(wyz); wxz = warp_sum(wxz); wxy = warp_sum(wxy);
-        }
-        if (lane == 0) {
-            A.force[i] = make_double4_32a(fx, fy, fz, 0.0);
+        if (lane < na) {
+            const int i = i0 + kWarps * lane;
+            const double dx = fx, dy = fy, dz = fz;
+            A.force[i] = make_double4_32a(dx, dy, dz, 0.0);
             if (!isfinite(fx + fy + fz)) atomicOr(&A.flags->error, FLAG_NONFINITE);
             if (TRAIN) {
                 const double4_32a fr = S.fref[i];
@@ -202,14 +332,14 @@ __global__ void __launch_bounds__(kThreads) k_sur_force(Atoms A, SurNet S, int a
                 part[0] += (double)ex * ex + (double)ey * ey + (double)ez * ez;
             } else {
                 double4_32a v = A.vel[i];
-                eam::kick_and_partials(v, fx, fy, fz, half_dt, kick != 0);
+                eam::kick_and_partials(v, dx, dy, dz, half_dt, kick != 0);
                 if (kick) A.vel[i] = v;
                 if (ENERGY) {
                     const double m = 1.0 / (kMvv2e * v.w);
                     part[0] += A.e_atom[i];
                     part[1] += m * fma(v.x, v.x, fma(v.y, v.y, v.z * v.z));
-                    part[2] += wxx; part[3] += wyy; part[4] += wzz;
-                    part[5] += wyz; part[6] += wxz; part[7] += wxy;
+#pragma unroll
+                    for (int q = 0; q < 6; q++) part[2 + q] += wv[q];
                     part[8] += m * v.x; part[9] += m * v.y; part[10] += m * v.z;
                 }
             }
@@ -219,33 +349,49 @@ __global__ void __launch_bounds__(kThreads) k_sur_force(Atoms A, SurNet S, int a
 }
 
 // ---------------------------------------------------------------- tangent of the descriptors
-// u_ik (standardised: times ginv_k) for the force term of the loss gradient.
+// u_ik (standardised: times ginv_k) for the force term of the loss gradient.  The pair's projection
+// t = u_ij . (phi_j - phi_i) is the same for every channel: the staging lane folds it into b'.
 __global__ void __launch_bounds__(kThreads) k_sur_u(Atoms A, SurNet S, int a0, int a1) {
-    __shared__ Stage st;
+    __shared__ Stage<4> stage[kWarps];   // r, t fc', -t fc/w^2
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    Stage<4> &st = stage[w];
     const float mu = S.mu0 + S.dmu * (float)lane;
     const float kx = -S.inv2w2 * kLog2e;
+    const F2 nmu = pack(-mu, -mu), kx2 = pack(kx, kx);
     const float gi = S.ginv[lane];
-    for (long long i0 = a0 + (long long)blockIdx.x * kWarps + w; i0 < a1; i0 += (long long)gridDim.x * kWarps) {
-        const int i = (int)i0;
+    int b0, b1;
+    block_range(a0, a1, b0, b1);
+    for (int i = b0 + w; i < b1; i += kWarps) {
         const Box &B = A.boxes[ph::replica_of(A, i)];
         const float4 pi = A.posf[i];
         const float4 fi = S.phi[i];
         const int cnt = min(A.count[i], A.k_max);
         const NbrRow row = nbr_row(A, i);
-        float u = 0.f;
+        F2 u = pack(0.f, 0.f);
         for (int base = 0; base < cnt; base += 32) {
-            const int np = stage_chunk(A, S, pi, B, row, cnt, base, lane, st.P0[w], st.P1[w]);
-            for (int q = 0; q < np; q++) {
-                const float4 p0 = st.P0[w][q], p1 = st.P1[w][q];
-                const float4 fj = __ldg(S.phi + __float_as_int(p0.w));
-                const float t = p1.x * (fj.x - fi.x) + p1.y * (fj.y - fi.y) + p1.z * (fj.z - fi.z);
-                const float a = p0.x - mu;
-                u = fmaf(ex2(kx * a * a) * fmaf(-a, p1.w, p0.z), t, u);
+            const int np = stage_chunk(A, S, pi, B, row, cnt, base, lane,
+                                       [&](int s, float r, float rinv, float dx, float dy, float dz, int j) {
+                float fc, dfc;
+                cutoff(S, r, fc, dfc);
+                const float4 fj = __ldg(S.phi + j);
+                const float t = dx * rinv * (fj.x - fi.x) + dy * rinv * (fj.y - fi.y) + dz * rinv * (fj.z - fi.z);
+                st.put(s, 0, r);
+                st.put(s, 1, t * dfc);
+                st.put(s, 2, -t * (fc * S.invw2));
+            });
+            if (lane < 3 && (np & 1)) st.put(np, lane, 0.f);
+            __syncwarp();
+#pragma unroll 4
+            for (int b = 0; b < (np + 1) >> 1; b++) {
+                F2 r, td, tw, unused;
+                st.get2(b, 0, r, td);
+                st.get2(b, 2, tw, unused);
+                const F2 a = add2(r, nmu);
+                u = fma2(ex2_2(mul2(mul2(kx2, a), a)), fma2(a, tw, td), u);
             }
             __syncwarp();
         }
-        S.u[(size_t)i * kSurNb + lane] = u * gi;
+        S.u[(size_t)i * kSurNb + lane] = both(u) * gi;
     }
 }
 
@@ -307,11 +453,32 @@ __global__ void k_sur_unsort_rows(Atoms A, const float *src, float *dst) {
     dst[(size_t)A.id[i] * kSurNb + k] = src[t];
 }
 
-int gather_blocks(int n_atoms) { return std::max(1, std::min(blocks_for(n_atoms, kWarps), 8192)); }
+// Blocks of a gather: as many as stay resident at once (blocks_per_sm of this kernel, fewer for few
+// atoms), so that each warp has the most atoms to finish together; at most one block per kWarps atoms.
+template <auto Kernel>
+int gather_blocks(int n_atoms) {
+    static int resident = 0;
+    if (!resident) {
+        int dev = 0, n_sm = 0, per_sm = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kernel, kThreads, 0);
+        resident = std::min(8192, std::max(1, n_sm * per_sm));
+    }
+    return std::max(1, std::min(blocks_for(n_atoms, kWarps), resident));
+}
+
+template <bool ENERGY, bool TRAIN>
+cudaError_t force_t(const Atoms &A, const SurNet &S, int a0, int a1, int kick, double half_dt, float phi_scale,
+                    int *rows_out, cudaStream_t s) {
+    const int nb = gather_blocks<k_sur_force<ENERGY, TRAIN>>(a1 - a0);
+    if (rows_out) *rows_out = nb;
+    if (a1 <= a0) return cudaSuccess;
+    k_sur_force<ENERGY, TRAIN><<<nb, kThreads, 0, s>>>(A, S, a0, a1, kick, half_dt, phi_scale);
+    return cudaGetLastError();
+}
 
 }  // namespace
-
-int sur_force_blocks(int n_atoms) { return gather_blocks(n_atoms); }
 
 cudaError_t launch_sur_kick_drift(const Atoms &A, double half_dt, double dt, SkinLimit lim, cudaStream_t s) {
     if (A.n == 0) return cudaSuccess;
@@ -321,27 +488,20 @@ cudaError_t launch_sur_kick_drift(const Atoms &A, double half_dt, double dt, Ski
 
 cudaError_t launch_sur_descriptors(const Atoms &A, const SurNet &S, int a0, int a1, cudaStream_t s) {
     if (a1 <= a0) return cudaSuccess;
-    k_sur_desc<<<gather_blocks(a1 - a0), kThreads, 0, s>>>(A, S, a0, a1, S.bf16);
+    k_sur_desc<<<gather_blocks<k_sur_desc>(a1 - a0), kThreads, 0, s>>>(A, S, a0, a1, S.bf16);
     return cudaGetLastError();
 }
 
 cudaError_t launch_sur_force(const Atoms &A, const SurNet &S, int a0, int a1, bool kick, bool energy,
                              double half_dt, double phi_scale, int *rows_out, cudaStream_t s) {
-    const int nb = gather_blocks(a1 - a0);
-    if (rows_out) *rows_out = nb;
-    if (a1 <= a0) return cudaSuccess;
-    if (phi_scale > 0.0)
-        k_sur_force<true, true><<<nb, kThreads, 0, s>>>(A, S, a0, a1, 0, 0.0, (float)phi_scale);
-    else if (energy)
-        k_sur_force<true, false><<<nb, kThreads, 0, s>>>(A, S, a0, a1, kick, half_dt, 0.f);
-    else
-        k_sur_force<false, false><<<nb, kThreads, 0, s>>>(A, S, a0, a1, kick, half_dt, 0.f);
-    return cudaGetLastError();
+    if (phi_scale > 0.0) return force_t<true, true>(A, S, a0, a1, 0, 0.0, (float)phi_scale, rows_out, s);
+    return energy ? force_t<true, false>(A, S, a0, a1, kick, half_dt, 0.f, rows_out, s)
+                  : force_t<false, false>(A, S, a0, a1, kick, half_dt, 0.f, rows_out, s);
 }
 
 cudaError_t launch_sur_u(const Atoms &A, const SurNet &S, int a0, int a1, cudaStream_t s) {
     if (a1 <= a0) return cudaSuccess;
-    k_sur_u<<<gather_blocks(a1 - a0), kThreads, 0, s>>>(A, S, a0, a1);
+    k_sur_u<<<gather_blocks<k_sur_u>(a1 - a0), kThreads, 0, s>>>(A, S, a0, a1);
     return cudaGetLastError();
 }
 
