@@ -11,8 +11,9 @@
 //                (group walks)
 //   k_cell_sort  stable order inside a cell: ascending caller atom id (deterministic)
 //   k_gather / k_copyback   renumber every per-atom array into cell order
-//   k_build_list full list: the 27 cells around each cell, |r_ij|^2 < r_list^2, a group of
-//                lanes per cell (for the staged and half walks also as 16-bit stencil slots)
+//   k_build_list full list: the 27 cells around each cell, |r_ij|^2 < r_list^2, 32 candidates at a
+//                time (k_build_local: a group of lanes per cell, for the staged and half walks,
+//                which take 16-bit stencil slots)
 // Link cells are fixed in fractional coordinates and at least r_list wide, so every pair
 // closer than r_list lies in adjacent cells (the hybrid NL-LCM of §3.2.1).
 #include <cuda_runtime.h>
@@ -89,11 +90,20 @@ __global__ void k_copyback(Atoms A) {
     for (long long k = gtid(); k < A.n; k += gstride()) ph::copyback_atom(A, A.boxes, (int)k);
 }
 
+// Local rows (group walks; LOCAL as in ph::build_cell_group).
 template <int G, int LOCAL>
-__global__ void __launch_bounds__(kThreads, 8) k_build_list(Atoms A, Cells C, double rl2, float band_lo,
-                                                         float band_hi) {
+__global__ void __launch_bounds__(kThreads, 8) k_build_local(Atoms A, Cells C, double rl2, float band_lo,
+                                                          float band_hi) {
     if (!ph::rebuild_requested(A.flags)) return;
     int m = ph::build_cells<G, LOCAL>(A, C, A.boxes, gtid() >> 5, gstride() >> 5, threadIdx.x & 31, rl2, band_lo, band_hi);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(&A.flags->max_count, m);
+}
+
+template <bool MARK>
+__global__ void __launch_bounds__(kThreads, 8) k_build_list(Atoms A, Cells C, double rl2, float band_lo, float band_hi) {
+    if (!ph::rebuild_requested(A.flags)) return;
+    int m = ph::build_slices<MARK>(A, C, A.boxes, gtid() >> 5, gstride() >> 5, threadIdx.x & 31, rl2, band_lo, band_hi);
     m = __reduce_max_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(&A.flags->max_count, m);
 }
@@ -101,10 +111,10 @@ __global__ void __launch_bounds__(kThreads, 8) k_build_list(Atoms A, Cells C, do
 template <int LOCAL>
 void launch_build(const Atoms &A, const Cells &C, double rl2, float band_lo, float band_hi, int list_group, int nbl,
                   cudaStream_t s) {
-    if (list_group == 4) k_build_list<4, LOCAL><<<nbl, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
-    else if (list_group == 8) k_build_list<8, LOCAL><<<nbl, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
-    else if (list_group == 16) k_build_list<16, LOCAL><<<nbl, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
-    else k_build_list<32, LOCAL><<<nbl, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
+    if (list_group == 4) k_build_local<4, LOCAL><<<nbl, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
+    else if (list_group == 8) k_build_local<8, LOCAL><<<nbl, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
+    else if (list_group == 16) k_build_local<16, LOCAL><<<nbl, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
+    else k_build_local<32, LOCAL><<<nbl, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
 }
 
 int capped_blocks(long long items, int threads) {
@@ -130,10 +140,10 @@ cudaError_t launch_clear_rebuild(Flags *f, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// FP64 pair walk: each row's entries j > i first (one warp per atom).
+// FP64 pair walk: each row's entries j > i first (one warp per atom), after a build only.
 __global__ void k_partition_rows(Atoms A) {
-    const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w < A.n) ph::partition_row_warp(A, A.boxes, (int)w, threadIdx.x & 31);
+    if (!ph::rebuild_requested(A.flags)) return;
+    for (long long w = gtid() >> 5; w < A.n; w += gstride() >> 5) ph::partition_row_warp(A, (int)w, threadIdx.x & 31);
 }
 
 cudaError_t launch_rebuild(const Atoms &A, const Cells &C, double rl2, float band_lo, float band_hi,
@@ -150,10 +160,13 @@ cudaError_t launch_rebuild(const Atoms &A, const Cells &C, double rl2, float ban
         k_gather<<<nb, kThreads, 0, s>>>(A);
         k_copyback<<<nb, kThreads, 0, s>>>(A);
         const int nbl = capped_blocks((long long)C.ncell * list_group, kThreads);
+        // a warp per link cell, and up to 8 blocks per SM of slices of it where there are fewer cells
+        const int nbs = capped_blocks((long long)A.n * 32, kThreads);
         if (C.tile == kWalkStaged) launch_build<1>(A, C, rl2, band_lo, band_hi, list_group, nbl, s);
         else if (C.tile == kWalkHalf) launch_build<2>(A, C, rl2, band_lo, band_hi, list_group, nbl, s);
-        else launch_build<0>(A, C, rl2, band_lo, band_hi, list_group, nbl, s);
-        if (A.pairs) k_partition_rows<<<(int)(((long long)A.n * 32 + kThreads - 1) / kThreads), kThreads, 0, s>>>(A);
+        else if (A.pairs) k_build_list<true><<<nbs, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
+        else k_build_list<false><<<nbs, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
+        if (A.pairs) k_partition_rows<<<nbs, kThreads, 0, s>>>(A);
     }
     return cudaGetLastError();
 }

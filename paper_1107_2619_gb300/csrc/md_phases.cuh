@@ -378,30 +378,28 @@ __device__ __forceinline__ void copyback_atom(const Atoms &A, const Box *boxes, 
     }
 }
 
-// The FP64 pair walk's row order (one warp per atom): the entries j > i first, those inside
-// r_cut at this build's FP32 positions (cin[i] of them) ahead of the others, then the entries
-// j < i, each group in its order; cup[i] = the number of entries j > i.  The order only steers
-// the walk (its flattened rows take the inside entries first, so that lanes rarely idle on a
-// pair beyond r_cut); which entries count is still decided by every pass's own FP64 test.  The
-// whole row (k_max <= kPairsKMax) is read into registers before any entry is written back.
-__device__ __forceinline__ void partition_row_warp(const Atoms &A, const Box *boxes, int i, int lane) {
+// The FP64 pair walk's row order (one warp per atom): the entries j > i first, those the build
+// marked as inside r_cut at its FP32 positions (kInsideMark; cin[i] of them) ahead of the others,
+// then the entries j < i, each group in its order; cup[i] = the number of entries j > i.  The marks
+// are taken off.  The order only steers the walk (its flattened rows take the inside entries first,
+// so that lanes rarely idle on a pair beyond r_cut); which entries count is still decided by every
+// pass's own FP64 test.  The whole row (k_max <= kPairsKMax) is read into registers before any
+// entry is written back.  (With the marks the row's neighbours need not be gathered again: 430 of
+// the 1,480 us of a rebuild of fcc Cu 500,000 atoms before.)
+constexpr int32_t kInsideMark = (int32_t)0x80000000;
+__device__ __forceinline__ void partition_row_warp(const Atoms &A, int i, int lane) {
     const int cnt = min(A.count[i], A.k_max);
     const NbrRow row = nbr_row(A, i);
-    const Box &B = boxes[replica_of(A, i)];
-    const float4 pi = A.posf[i];
     int v[kPairsKMax / 32];
-    unsigned in = 0;   // bit c: entry 32 c + lane lies inside r_cut
+    unsigned in = 0;   // bit c: entry 32 c + lane is marked
 #pragma unroll
     for (int c = 0; c < kPairsKMax / 32; c++) {
         const int k = 32 * c + lane;
-        v[c] = k < cnt ? *row.ptr(k) : -1;
-        if (v[c] > i) {
-            const float4 pj = A.posf[v[c]];
-            float dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
-            dx = fmaf(-B.Lf[0], rintf(dx * B.invLf[0]), dx);
-            dy = fmaf(-B.Lf[1], rintf(dy * B.invLf[1]), dy);
-            dz = fmaf(-B.Lf[2], rintf(dz * B.invLf[2]), dz);
-            if (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < A.pair_rc2f) in |= 1u << c;
+        v[c] = -1;
+        if (k < cnt) {
+            const int e = *row.ptr(k);
+            if (e & kInsideMark) in |= 1u << c;
+            v[c] = e & ~kInsideMark;
         }
     }
     __syncwarp();
@@ -459,29 +457,6 @@ static __device__ __noinline__ bool within_exact_band(const double4_32a *pos, in
 #ifndef MD_BUILD_UNROLL
 #define MD_BUILD_UNROLL 4
 #endif
-// Smallest lane group whose last atoms take several lanes each: a warp-wide group only.  In the
-// 4-lane groups of bcc Fe cells (eight cells per warp, about five atoms each) it built the lists
-// 20 % slower on GB300 (0.78 against 0.63 ms per rebuild at 1.02M atoms).
-#ifndef MD_BUILD_SLICE_MIN_G
-#define MD_BUILD_SLICE_MIN_G 32
-#endif
-
-// Full list rows of the atoms of link cell c (§3.2.1: candidates from the cells around it, 27 for
-// cells r_list wide, 125 for cells r_list / 2 wide) by a group of G lanes (G = 4, 8, 16 or 32;
-// 32 / G cells per warp): lane a of the group takes atoms s + a, s + a + G, ... of the cell.  All
-// lanes of the group walk the same neighbour cells and the same candidates in the same order,
-// so a candidate is one broadcast load for the group and
-// the control flow is uniform inside it.  Candidates are screened with FP32 wrapped coordinates,
-// shifted by whole box edges for neighbour cells across the periodic boundary (no rounding to the
-// nearest image per candidate).  Only a candidate whose FP32 r^2 lies in [band_lo, band_hi] (a band
-// wider than the proven FP32 error) is decided by the exact FP64 test, so each row is the exact
-// FP64 set, listed by cell in (dz, dy, dx) order and by ascending slot inside a cell.  Rows are cut
-// at k_max (the count is kept).  Returns the longest row of this lane's atoms.  The stencil of
-// +-reach cells along each edge needs >= 2 reach + 1 cells per edge (no cell visited twice).
-// LOCAL (group walks, one system, reach 1): 1, every entry is also written to the 16-bit local
-// list as the slot of the candidate in its cell group's stage (grp_loc of the stencil cell plus
-// the candidate's rank inside its cell); 2, only the entries j > i are, as the half row of the
-// half walk (lcount of them).
 // The cells of the stencil of link cell (cx, cy, cz) of a replica (+-R cells along each edge), in
 // (dz, dy, dx) order: fn(js, je, sx, sy, sz, dz, dy, dx) with the cell's slot range and the shift
 // by whole box edges that puts a cell across the periodic boundary next to the home cell.
@@ -524,15 +499,11 @@ __device__ __forceinline__ void for_stencil(const Cells &C, const RepCells &g, i
 // FP64 set, listed by cell in (dz, dy, dx) order and by ascending slot inside a cell.  Rows are cut
 // at k_max (the count is kept).  Returns the longest row of this lane's atoms.  The stencil of
 // +-reach cells along each edge needs >= 2 reach + 1 cells per edge (no cell visited twice).
-// In a warp-wide group (G = 32), the last atoms of a cell, when they fill at most half the warp (the
-// 4 atoms after the first 32 of a 36-atom fcc Cu cell), take L = 2, 4, ... lanes each:
-// lane l of an atom tests candidates js + l, js + l + L, ... of every stencil cell, and a ballot
-// over the atom's L lanes places the accepted ones in slot order, so the rows are the same.
 // LOCAL (group walks, one system, reach 1): 1, every entry is also written to the 16-bit local
 // list as the slot of the candidate in its cell group's stage (grp_loc of the stencil cell plus
 // the candidate's rank inside its cell); 2, only the entries j > i are, as the half row of the
-// half walk (lcount of them).  Those builds keep one lane per atom, and write the global rows
-// (A.nbr) only when `rows` is set (the counts always): the step kernel's group walks read the
+// half walk (lcount of them).  (Builds without local rows: build_slice.)  The global rows
+// (A.nbr) are written only when `rows` is set (the counts always): the step kernel's group walks read the
 // local rows alone while every group fits its stage.
 template <int G, int LOCAL>
 __device__ __forceinline__ int build_cell_group(const Atoms &A, const Cells &C, const Box *boxes, int c, int gl,
@@ -552,60 +523,12 @@ __device__ __forceinline__ int build_cell_group(const Atoms &A, const Cells &C, 
     const bool edge = cx < R || cx >= nx - R || cy < R || cy >= ny - R || cz < R || cz >= nz - R;
     int longest = 0;
     for (int a0 = s; a0 < e; a0 += G) {
-        if constexpr (LOCAL == 0 && G >= MD_BUILD_SLICE_MIN_G) {
-            if (2 * (e - a0) <= G) {   // the last atoms of the cell: L lanes each
-                const int rem = e - a0;
-                int lg = 1;
-                while ((rem << (lg + 1)) <= G) lg++;
-                const int L = 1 << lg;
-                const int a = gl >> lg, sl = gl & (L - 1);
-                const bool act = a < rem;
-                const int i = a0 + a, ii = act ? i : s;
-                const float4 fi = A.posf[ii];
-                const int gbase = (int)(threadIdx.x & 31) & ~(G - 1);
-                const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << gbase;
-                const unsigned lmask = L == 32 ? 0xffffffffu : (1u << L) - 1u;
-                const int sh = gbase + (a << lg);
-                int32_t *const row = A.nbr + 4 * (size_t)ii;
-                int cnt = 0;
-                for_stencil(C, g, R, cx, cy, cz, Lx, Ly, Lz,
-                            [&](int js, int je, float sx, float sy, float sz, int, int, int) {
-                    const float ox = sx - fi.x, oy = sy - fi.y, oz = sz - fi.z;
-                    for (int j0 = js; j0 < je; j0 += L) {   // the same trip count on every lane of the group
-                        const int j = j0 + sl;
-                        bool in = false;
-                        if (j < je) {
-                            const float4 f = A.posf[j];
-                            const float dx = f.x + ox, dy = f.y + oy, dz = f.z + oz;
-                            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                            if (r2 <= band_hi)
-                                in = (r2 < band_lo || within_exact_band(A.pos, ii, j, B, rl2)) && act && j != i;
-                        }
-                        const unsigned sub = (__ballot_sync(gmask, in) >> sh) & lmask;
-                        if (in) {
-                            const int k = cnt + __popc(sub & ((1u << sl) - 1u));
-                            if (k < kmax) row[(long long)(k >> 2) * plane + (k & 3)] = j;
-                        }
-                        cnt += __popc(sub);
-                    }
-                });
-                if (act) {
-                    if (sl == 0) {
-                        A.count[i] = cnt;
-                        A.wrap[i] = edge ? 1 : 0;
-                        if (cnt > kmax) atomicOr(&A.flags->error, FLAG_OVERFLOW);
-                    }
-                    longest = max(longest, cnt);
-                }
-                break;
-            }
-        }
         const int i = a0 + gl;
         const bool act = i < e;
         const int ii = act ? i : s;
         const float4 fi = A.posf[ii];
         int32_t *wp = A.nbr + 4 * (size_t)ii;   // entry cnt of the row (planes of 4 entries)
-        uint16_t *lwp = LOCAL ? A.lnbr + 4 * (size_t)ii : nullptr;   // the same entry of the local list
+        uint16_t *lwp = A.lnbr + 4 * (size_t)ii;   // the same entry of the local list
         int cnt = 0, lcnt = 0;
         int lbase = 0;   // staged slot of the first atom of the current candidate cell (local list)
         // one candidate: append j to the row if it is a neighbour
@@ -614,7 +537,7 @@ __device__ __forceinline__ int build_cell_group(const Atoms &A, const Cells &C, 
                 const bool in = r2 < band_lo || within_exact_band(A.pos, ii, j, B, rl2);
                 if (in && act && j != i) {
                     if (cnt < kmax) {
-                        if (LOCAL == 0 || rows) *wp = j;
+                        if (rows) *wp = j;
                         if constexpr (LOCAL == 1) *lwp = (uint16_t)(lbase + (j - js));
                         if constexpr (LOCAL == 2) {
                             if (j > i) {
@@ -685,6 +608,134 @@ __device__ __forceinline__ int build_cell_group(const Atoms &A, const Cells &C, 
         }
     }
     return longest;
+}
+
+// Full list rows of a slice of the atoms of link cell c by one warp: atoms s + slice, s + slice + S, ...
+// of the cell's range (S slices per cell; list walks, no local rows).  The candidates, the atoms of
+// the (2 reach + 1)^3 cells around c in (dz, dy, dx) order, are numbered through, and the lanes take 32
+// consecutive ones at a time, empty cells and cell boundaries costing no lane; every home atom of
+// the slice then tests the 32 at once, and a ballot places the accepted ones behind each other in
+// candidate order, so that the rows are the exact FP64 set in the same order as build_cell_group's.
+// A lane per home atom (build_cell_group) appended candidate by candidate with most lanes idle,
+// and the appends' address chain bounded it.  Per rebuild, list phase, before -> after (us): 32 bcc
+// Fe replicas of 623,572 atoms 473 -> 350, Fe-C 250,250 221 -> 129, bcc Fe 2,000 65 -> 29, fcc Cu
+// 500,000 994 -> 984 (57 instructions per home atom and 32 candidates; issue slots 75 % busy).
+// MARK: entries inside r_cut (FP32) get kInsideMark, for partition_row_warp.
+template <bool MARK>
+__device__ __forceinline__ int build_slice(const Atoms &A, const Cells &C, const Box *boxes, int c, int slice, int S,
+                                           int lane, double rl2, float band_lo, float band_hi) {
+    const int s = C.cell_start[c] + slice, e = C.cell_start[c + 1];
+    if (s >= e) return 0;
+    const int r = replica_of(A, s);
+    const Box &B = boxes[r];
+    const RepCells g = C.rc[r];
+    const int nx = g.nc[0], ny = g.nc[1], nz = g.nc[2];
+    const int local = c - g.base;
+    const int cx = local % nx, cy = (local / nx) % ny, cz = local / (nx * ny);
+    const int R = C.reach, W = 2 * R + 1, nst = W * W * W;
+    const int kmax = A.k_max;
+    const bool edge = cx < R || cx >= nx - R || cy < R || cy >= ny - R || cz < R || cz >= nz - R;
+    const unsigned full = 0xffffffffu, below = (1u << lane) - 1u;
+    const int homes = (e - s + S - 1) / S;
+    int longest = 0;
+    for (int h0 = 0; h0 < homes; h0 += 32) {
+        const int nh = min(32, homes - h0);
+        const int mine = s + S * (h0 + min(lane, nh - 1));   // this lane's home atom
+        const float4 fh = A.posf[mine];
+        int cnt = 0;
+        for (int q0 = 0; q0 < nst; q0 += 32) {   // (one round for reach 1)
+            // this lane's stencil cell: its first atom, length and shift by whole box edges
+            const int q = q0 + lane;
+            int first = 0, len = 0;
+            float sx = 0.f, sy = 0.f, sz = 0.f;
+            if (q < nst) {
+                int x = cx + q % W - R, y = cy + (q / W) % W - R, z = cz + q / (W * W) - R;
+                if (x < 0) { x += nx; sx = -B.Lf[0]; }
+                if (x >= nx) { x -= nx; sx = B.Lf[0]; }
+                if (y < 0) { y += ny; sy = -B.Lf[1]; }
+                if (y >= ny) { y -= ny; sy = B.Lf[1]; }
+                if (z < 0) { z += nz; sz = -B.Lf[2]; }
+                if (z >= nz) { z -= nz; sz = B.Lf[2]; }
+                const int cc = g.base + (z * ny + y) * nx + x;
+                first = C.cell_start[cc];
+                len = C.cell_start[cc + 1] - first;
+            }
+            // the non-empty cells moved to the first lanes (lane t: the t-th set bit of ne)
+            const unsigned ne = __ballot_sync(full, len > 0);
+            const int nne = __popc(ne);
+            int src = 0;
+#pragma unroll
+            for (int b = 16; b > 0; b >>= 1)
+                if (__popc(ne & ((1u << (src + b)) - 1u)) <= lane) src += b;
+            first = __shfl_sync(full, first, src & 31);
+            len = __shfl_sync(full, len, src & 31);
+            sx = __shfl_sync(full, sx, src & 31);
+            sy = __shfl_sync(full, sy, src & 31);
+            sz = __shfl_sync(full, sz, src & 31);
+            if (lane >= nne) len = 0;
+            int off = len;   // candidates before this lane's cell
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(full, off, o);
+                if (lane >= o) off += y;
+            }
+            const int total = __shfl_sync(full, off, 31);
+            off -= len;
+            for (int p0 = 0; p0 < total; p0 += 32) {
+                // candidate p0 + lane: the cell it lies in, its slot and shifted position
+                const bool cell = lane < nne;
+                const int base = __popc(__ballot_sync(full, cell && off <= p0)) - 1;
+                const unsigned starts =
+                    __reduce_or_sync(full, cell && off > p0 && off < p0 + 32 ? 1u << (off - p0) : 0u);
+                const int t = base + __popc(starts & (below | (1u << lane)));
+                const int j = __shfl_sync(full, first, t) + p0 + lane - __shfl_sync(full, off, t);
+                const float ox = __shfl_sync(full, sx, t), oy = __shfl_sync(full, sy, t), oz = __shfl_sync(full, sz, t);
+                const bool live = p0 + lane < total;
+                float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (live) f = A.posf[j];
+                for (int a = 0; a < nh; a++) {
+                    const float dx = f.x + (ox - __shfl_sync(full, fh.x, a)), dy = f.y + (oy - __shfl_sync(full, fh.y, a)),
+                                dz = f.z + (oz - __shfl_sync(full, fh.z, a));
+                    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                    const int i = s + S * (h0 + a);
+                    bool in = live && r2 <= band_hi && j != i;
+                    if (__any_sync(full, in && r2 >= band_lo)) {   // the band: the exact test decides
+                        if (in && r2 >= band_lo) in = within_exact_band(A.pos, i, j, B, rl2);
+                    }
+                    const unsigned m = __ballot_sync(full, in);
+                    if (m == 0u) continue;
+                    const int k = __shfl_sync(full, cnt, a) + __popc(m & below);
+                    if (in && k < kmax)
+                        A.nbr[4 * ((long long)(k >> 2) * A.n + i) + (k & 3)] = MARK && r2 < A.pair_rc2f ? j | kInsideMark : j;
+                    if (lane == a) cnt += __popc(m);
+                }
+            }
+        }
+        if (lane < nh) {
+            A.count[mine] = cnt;
+            A.wrap[mine] = edge ? 1 : 0;
+            if (cnt > kmax) atomicOr(&A.flags->error, FLAG_OVERFLOW);
+            longest = max(longest, cnt);
+        }
+    }
+    return longest;
+}
+
+// Slices per link cell: enough that every warp of the launch has one, at most a home atom each.
+__host__ __device__ inline int list_slices(long long ncell, long long nwarps) {
+    const long long q = ncell > 0 ? nwarps / ncell : 1;
+    return (int)(q < 1 ? 1 : (q > 32 ? 32 : q));
+}
+
+// The list phase over all cells and slices.
+template <bool MARK>
+__device__ __forceinline__ int build_slices(const Atoms &A, const Cells &C, const Box *boxes, long long warp,
+                                            long long nwarps, int lane, double rl2, float band_lo, float band_hi) {
+    const int S = list_slices(C.ncell, nwarps);
+    int m = 0;
+    for (long long q = warp; q < (long long)C.ncell * S; q += nwarps)
+        m = max(m, build_slice<MARK>(A, C, boxes, (int)(q / S), (int)(q % S), S, lane, rl2, band_lo, band_hi));
+    return m;
 }
 
 // The list phase over all cells: warp w of nwarps takes cell groups w, w + nwarps, ...; every

@@ -158,10 +158,8 @@ constexpr bool kGroupWalk = WALK == kWalkStaged || WALK == kWalkCells || WALK ==
 // The list rebuild (§3.2.1: bin, counting sort, Verlet list; and for the walks that need them the
 // group tables, local rows or the half-list row order), every block of a cooperative launch
 // taking part, with grid barriers between the phases.  srow: the step's profiling stamps (1..9)
-// or NULL.  False once the launch is aborted (a barrier gave up).  G: the lanes per link cell of
-// the list build as a compile-time constant (one build variant in the kernel: fewer registers),
-// or 0 for sp.list_group at run time.
-template <int WALK, int G = 0>
+// or NULL.  False once the launch is aborted (a barrier gave up).
+template <int WALK>
 __device__ __forceinline__ bool rebuild_phases(const Atoms &A, const Cells &C, Box *boxes, const StepParams &sp,
                                                GridBarrier *bar, int *ws, unsigned long long *srow) {
     const unsigned nb = gridDim.x;
@@ -215,20 +213,19 @@ __device__ __forceinline__ bool rebuild_phases(const Atoms &A, const Cells &C, B
     // the group walks need the global rows only when some group does not fit its stage
     const bool rows = !kGroupWalk<WALK> || *reinterpret_cast<volatile int32_t *>(&A.flags->tile_bad);
     if (WALK != kWalkCells || rows) {
-        constexpr int LOCAL = WALK == kWalkStaged ? 1 : (WALK == kWalkHalf ? 2 : 0);
         int m;
-        if constexpr (G > 0)
-            m = ph::build_cells<G, LOCAL>(A, C, boxes, tid >> 5, stride >> 5, threadIdx.x & 31, sp.rl2, sp.band_lo,
-                                          sp.band_hi, rows);
+        if constexpr (WALK == kWalkStaged || WALK == kWalkHalf)
+            m = ph::build_cells_any<WALK == kWalkStaged ? 1 : 2>(sp.list_group, A, C, boxes, tid >> 5, stride >> 5,
+                                                                 threadIdx.x & 31, sp.rl2, sp.band_lo, sp.band_hi, rows);
         else
-            m = ph::build_cells_any<LOCAL>(sp.list_group, A, C, boxes, tid >> 5, stride >> 5, threadIdx.x & 31, sp.rl2,
-                                           sp.band_lo, sp.band_hi, rows);
+            m = ph::build_slices<WALK == kWalkPairs>(A, C, boxes, tid >> 5, stride >> 5, threadIdx.x & 31, sp.rl2,
+                                                     sp.band_lo, sp.band_hi);
         m = __reduce_max_sync(0xffffffffu, m);
         if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(&A.flags->max_count, m);
     }
     if constexpr (WALK == kWalkPairs) {   // each row's entries j > i first
         RB_SYNC();
-        for (long long i = tid >> 5; i < A.n; i += stride >> 5) ph::partition_row_warp(A, boxes, (int)i, threadIdx.x & 31);
+        for (long long i = tid >> 5; i < A.n; i += stride >> 5) ph::partition_row_warp(A, (int)i, threadIdx.x & 31);
     }
     RB_SYNC();
     MD_STAMP(9);
@@ -636,7 +633,7 @@ constexpr int kRebuildThreads = 256;
 #define MD_REBUILD_MIN_BLOCKS 4
 #endif
 
-template <int WALK, int G>
+template <int WALK>
 __global__ void __launch_bounds__(kRebuildThreads, MD_REBUILD_MIN_BLOCKS)
     k_rebuild(Atoms A, Cells C, StepParams sp, GridBarrier *bar, unsigned long long *stamps) {
     __shared__ int ws[32];
@@ -647,15 +644,15 @@ __global__ void __launch_bounds__(kRebuildThreads, MD_REBUILD_MIN_BLOCKS)
         return;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     unsigned long long *srow = stamps && lead ? stamps + kStampsPerStep * (s + 1) : nullptr;
-    if (!rebuild_phases<WALK, G>(A, C, A.boxes, sp, bar, ws, srow)) return;
+    if (!rebuild_phases<WALK>(A, C, A.boxes, sp, bar, ws, srow)) return;
     if (lead) {   // every block has passed the rebuild decision (the barriers above)
         A.flags->n_rebuilds++;
         A.flags->need_rebuild = 0;
     }
 }
 
-template <int WALK, int G>
-cudaError_t launch_rebuild_g(const Atoms &A, const Cells &C, const StepParams &sp, GridBarrier *bar,
+template <int WALK>
+cudaError_t launch_rebuild_t(const Atoms &A, const Cells &C, const StepParams &sp, GridBarrier *bar,
                              unsigned long long *stamps, cudaStream_t s) {
     static int grid = 0;
     if (grid == 0) {
@@ -663,7 +660,7 @@ cudaError_t launch_rebuild_g(const Atoms &A, const Cells &C, const StepParams &s
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rebuild<WALK, G>, kRebuildThreads, 0);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rebuild<WALK>, kRebuildThreads, 0);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
         grid = per_sm * n_sm;
@@ -674,19 +671,8 @@ cudaError_t launch_rebuild_g(const Atoms &A, const Cells &C, const StepParams &s
     Cells c = C;
     StepParams q = sp;
     void *args[] = {&a, &c, &q, &bar, &stamps};
-    return cudaLaunchCooperativeKernel((const void *)k_rebuild<WALK, G>, dim3(grid), dim3(kRebuildThreads), args, 0,
+    return cudaLaunchCooperativeKernel((const void *)k_rebuild<WALK>, dim3(grid), dim3(kRebuildThreads), args, 0,
                                        s);
-}
-
-template <int WALK>
-cudaError_t launch_rebuild_t(const Atoms &A, const Cells &C, const StepParams &sp, GridBarrier *bar,
-                             unsigned long long *stamps, cudaStream_t s) {
-    switch (sp.list_group) {
-        case 4: return launch_rebuild_g<WALK, 4>(A, C, sp, bar, stamps, s);
-        case 8: return launch_rebuild_g<WALK, 8>(A, C, sp, bar, stamps, s);
-        case 16: return launch_rebuild_g<WALK, 16>(A, C, sp, bar, stamps, s);
-        default: return launch_rebuild_g<WALK, 32>(A, C, sp, bar, stamps, s);
-    }
 }
 
 template <int PREC, int T>

@@ -36,13 +36,9 @@ int step_walk(const Atoms &A, const Cells &C, const Pot &P, int precision, int l
 
 cudaError_t launch_rebuild_step(const Atoms &A, const Cells &C, const Pot &P, int precision, int lanes,
                                 const StepParams &sp, GridBarrier *bar, unsigned long long *stamps, cudaStream_t s) {
-    switch (step_walk(A, C, P, precision, lanes)) {
-        case kWalkStaged: return st::launch_rebuild_t<kWalkStaged>(A, C, sp, bar, stamps, s);
-        case kWalkCells: return st::launch_rebuild_t<kWalkCells>(A, C, sp, bar, stamps, s);
-        case kWalkHalf: return st::launch_rebuild_t<kWalkHalf>(A, C, sp, bar, stamps, s);
-        case kWalkPairs: return st::launch_rebuild_t<kWalkPairs>(A, C, sp, bar, stamps, s);
-        default: return st::launch_rebuild_t<kWalkList>(A, C, sp, bar, stamps, s);
-    }
+    // (segments are an FP64 matter: the list walk, or the pairs of the half list)
+    return step_walk(A, C, P, precision, lanes) == kWalkPairs ? st::launch_rebuild_t<kWalkPairs>(A, C, sp, bar, stamps, s)
+                                                              : st::launch_rebuild_t<kWalkList>(A, C, sp, bar, stamps, s);
 }
 
 }  // namespace mdk
