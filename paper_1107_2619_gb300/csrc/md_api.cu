@@ -16,6 +16,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 #include <cstring>
 #include <map>
@@ -77,8 +78,6 @@ struct md_ctx {
     // Nose-Hoover thermostat (md_set_thermostat)
     bool thermo_on = false;
     Thermo *d_thermo = nullptr;
-    int2 *d_ke_chunks = nullptr;
-    int n_ke_chunks = 0;
     std::vector<double> h_rep;           // [5 n_rep] replica sums after the last thermostatted md_step
     // learned surrogate (kind MD_POT_SURROGATE)
     bool sur = false;          // context kind
@@ -250,11 +249,11 @@ md_status sync_and_check(md_ctx *ctx, bool strict_skin) {
     return MD_OK;
 }
 
-// Clear the sticky device error bits (called at the start of every compute call).
+// Clear the grid barrier and the sticky device error bits, which lie behind each other (called at
+// the start of every compute call).
 cudaError_t reset_errors(md_ctx *ctx) {
-    cudaError_t e = cudaMemsetAsync(&ctx->d_flags->error, 0, sizeof(int32_t), ctx->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&ctx->d_flags->skin_exceeded, 0, sizeof(int32_t), ctx->stream);
-    return e;
+    static_assert(offsetof(Flags, error) == 0 && offsetof(Flags, skin_exceeded) == sizeof(int32_t), "cleared together");
+    return cudaMemsetAsync(ctx->d_bar, 0, sizeof(GridBarrier) + 2 * sizeof(int32_t), ctx->stream);
 }
 
 cudaError_t enqueue_rebuild(md_ctx *ctx) {
@@ -388,9 +387,6 @@ StepParams step_params(md_ctx *ctx, int n_steps) {
     sp.list_group = ph_list_group(ctx);
     if (ctx->thermo_on) {
         sp.thermo = ctx->d_thermo;
-        sp.ke_chunks = ctx->d_ke_chunks;
-        sp.n_ke_chunks = ctx->n_ke_chunks;
-        sp.rep_off = ctx->d_rep_off;
     }
     sp.spin_limit = kSpinLimit;
     sp.motion = ctx->cfg.integrator == MD_INTEGRATOR_PC3 ? kMotionPC3 : kMotionVerlet;
@@ -695,8 +691,11 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
     chk(dalloc(ctx, &ctx->d_rc, n_rep));
     chk(dalloc(ctx, &ctx->d_rep_off, n_rep + 1));
     chk(dalloc(ctx, &ctx->d_rep_sums, (size_t)n_rep * 5));
-    chk(dalloc(ctx, &ctx->d_flags, 1));
-    chk(dalloc(ctx, &ctx->d_bar, 1));
+    unsigned char *bar_flags = nullptr;   // the barrier, then the flags
+    chk(dalloc(ctx, &bar_flags, sizeof(GridBarrier) + sizeof(Flags)));
+    if (e == cudaSuccess) e = cudaMemset(bar_flags, 0, sizeof(GridBarrier) + sizeof(Flags));
+    ctx->d_bar = reinterpret_cast<GridBarrier *>(bar_flags);
+    ctx->d_flags = reinterpret_cast<Flags *>(bar_flags + sizeof(GridBarrier));
     chk(dalloc(ctx, &ctx->d_reduce, kPartials));
     Cells &C = ctx->C;
     C.ncell = (int)ncell;
@@ -1658,7 +1657,8 @@ md_status md_tune(md_ctx *ctx, int32_t *lanes_out) {
         sp.rebuild_every = 0;
         sp.strain_scale = 1.0;
         cudaEvent_t e0 = nullptr, e1 = nullptr;
-        cudaError_t e = copy(true);
+        cudaError_t e = reset_errors(ctx);
+        if (e == cudaSuccess) e = copy(true);
         if (e == cudaSuccess) e = cudaEventCreate(&e0);
         if (e == cudaSuccess) e = cudaEventCreate(&e1);
         float best = 1e30f;
@@ -1996,9 +1996,6 @@ md_status md_set_thermostat(md_ctx *ctx, int32_t on, const double *t_kelvin, con
     for (int r = 0; r < nr; r++)
         if (!(t_kelvin[r] > 0.0) || !std::isfinite(t_kelvin[r]) || !(tau_fs[r] > 0.0) || !std::isfinite(tau_fs[r]))
             return fail(ctx, MD_ERR_ARG, "thermostat: T > 0 and tau > 0 for every replica");
-    std::vector<int2> chunks;
-    for (int r = 0; r < nr; r++)
-        for (int64_t a = ctx->rep_off[r]; a < ctx->rep_off[r + 1]; a += kKeChunk) chunks.push_back(make_int2(r, (int)a));
     std::vector<Thermo> th(nr);
     for (int r = 0; r < nr; r++) {
         const int64_t m = ctx->rep_off[r + 1] - ctx->rep_off[r];
@@ -2011,11 +2008,7 @@ md_status md_set_thermostat(md_ctx *ctx, int32_t on, const double *t_kelvin, con
         th[r].s_b = th[r].s_a = 1.0;
     }
     if (!ctx->d_thermo) MD_CK(dalloc(ctx, &ctx->d_thermo, nr));
-    if (ctx->n_ke_chunks < (int)chunks.size()) MD_CK(dalloc(ctx, &ctx->d_ke_chunks, chunks.size()));
-    ctx->n_ke_chunks = (int)chunks.size();
     MD_CK(cudaMemcpy(ctx->d_thermo, th.data(), nr * sizeof(Thermo), cudaMemcpyHostToDevice));
-    if (!chunks.empty())
-        MD_CK(cudaMemcpy(ctx->d_ke_chunks, chunks.data(), chunks.size() * sizeof(int2), cudaMemcpyHostToDevice));
     ctx->thermo_on = true;
     ctx->h_rep.clear();
     drop_graphs(ctx);   // graphs hold the step parameters by value

@@ -44,10 +44,10 @@ struct Box {
 
 // Device-side status, read by the host after each synchronising call.
 struct Flags {
-    int32_t need_rebuild;   // set by the displacement check or the schedule; cleared by pass 1
-    int32_t error;          // FLAG_* bits
-    int32_t max_count;      // longest list at the last build
+    int32_t error;          // FLAG_* bits (this word and the next are cleared at the start of every call)
     int32_t skin_exceeded;  // an atom moved more than skin/2 since the last build
+    int32_t need_rebuild;   // set by the displacement check or the schedule; cleared by pass 1
+    int32_t max_count;      // longest list at the last build
     unsigned long long n_rebuilds;
     unsigned long long range_violations;
     long long step;         // steps taken (the rebuild schedule counts from here)
@@ -118,12 +118,25 @@ struct RepCells {
     int base;
 };
 
-// Grid barrier of the persistent step kernel (see md_step.cu).
+// Grid barrier of the cooperative kernels (st::grid_sync): blocks arrive at their group's counter
+// and the last of a group at the launch's; the counters return to zero at every barrier, the
+// generations run on.  Words that are polled lie in lines of their own.  Zeroed at the start of
+// every call (an aborted barrier leaves its counts behind).
+constexpr int kBarFlat = 256;    // up to this many blocks: one group
+constexpr int kBarGroup = 64;    // else blocks per group
+constexpr int kBarGroups = 40;
+constexpr int kGridMax = kBarGroup * kBarGroups;
 struct GridBarrier {
     unsigned int count;
-    unsigned int gen;
+    unsigned int pad0[31];
     int abort;
-    int pad;
+    int pad1[31];
+    struct Group {
+        unsigned int count;
+        unsigned int pad0[31];
+        unsigned int gen;
+        unsigned int pad1[31];
+    } group[kBarGroups];
 };
 
 // Device view of the per-atom state (cell order).  A batch of replicas is stored as one
@@ -320,7 +333,6 @@ struct Thermo {
     unsigned long long pad;
 };
 constexpr double kKeFix = 1099511627776.0;   // 2^40
-constexpr int kKeChunk = 1024;               // atoms per chunk of the kinetic-energy sums
 
 // Persistent step kernel (md_step.cu): n_steps velocity-Verlet steps in one cooperative
 // launch; grid barriers between phases; per-phase %globaltimer stamps when stamps != NULL.
@@ -334,9 +346,6 @@ struct StepParams {
     float band_lo, band_hi;
     int list_group;       // lanes per link cell in the list build (4, 8, 16 or 32)
     Thermo *thermo;       // [n_rep] Nose-Hoover state, or NULL (NVE)
-    const int2 *ke_chunks;  // (replica, first atom) of each chunk of <= kKeChunk atoms
-    int n_ke_chunks;
-    const int32_t *rep_off;  // [n_rep + 1]
     unsigned long long spin_limit;
     int withhold_arrival;  // self-test of the bounded waits: 1, block 0 skips its first grid-barrier
                            // arrival; 2 (group walks), block 0's staging producer releases no group

@@ -1233,6 +1233,25 @@ __device__ __forceinline__ double4_32a close_step(const Atoms &A, const Box *box
     return v;
 }
 
+// Kinetic energy of the atoms i of a warp's lanes (i < 0: none; v: the velocity records) into their
+// replicas' fixed-point accumulators, whose sum does not depend on the order: one atomic add per
+// warp where its atoms are of one replica.  Every lane of the warp calls.
+__device__ __forceinline__ void add_kinetic(const Atoms &A, Thermo *th, int i, const double4_32a &v) {
+    const int r = i >= 0 ? ph::replica_of(A, i) : -1;
+    const unsigned live = __ballot_sync(0xffffffffu, i >= 0);
+    if (live == 0u) return;
+    unsigned long long ke = 0;   // v.w = 1 / (m mvv2e): KE_i = |v|^2 / (2 v.w)
+    if (i >= 0) ke = (unsigned long long)llrint(0.5 * fma(v.x, v.x, fma(v.y, v.y, v.z * v.z)) / v.w * kKeFix);
+    const int r0 = __shfl_sync(0xffffffffu, r, __ffs(live) - 1);
+    if (__all_sync(0xffffffffu, i < 0 || r == r0)) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ke += __shfl_down_sync(0xffffffffu, ke, o);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&th[r0].ke_fix, ke);
+    } else if (i >= 0) {
+        atomicAdd(&th[r].ke_fix, ke);
+    }
+}
+
 // After the pair force pass, per atom: the force = own share + the neighbours' shares, then what
 // follows it; on the energy step the atom's energy and partial sums (v: the velocity after it).
 template <bool ENERGY>
@@ -1266,14 +1285,22 @@ __device__ __forceinline__ void pairs_kick64(const Atoms &A, int i, double half_
     pairs_partials64<ENERGY>(A, i, fx, fy, fz, v, part);
 }
 
-// The same inside the step kernel.
+// The same inside the step kernel, over all atoms (whole warps; th as in force_walk).
 template <bool ENERGY>
-__device__ __forceinline__ void pairs_close64(const Atoms &A, const Box *boxes, const StepParams &sp, int i, bool open,
-                                              double (&part)[kPartials]) {
-    const double4_32a own = A.force[i], acc = A.f_acc[i];
-    const double fx = own.x + acc.x, fy = own.y + acc.y, fz = own.z + acc.z;
-    const double4_32a v = close_step(A, boxes, sp, i, fx, fy, fz, open);
-    pairs_partials64<ENERGY>(A, i, fx, fy, fz, v, part);
+__device__ __forceinline__ void pairs_close64(const Atoms &A, const Box *boxes, const StepParams &sp, long long tid,
+                                              long long stride, bool open, Thermo *th, double (&part)[kPartials]) {
+    const int lane = threadIdx.x & 31;
+    for (long long i0 = tid - lane; i0 < A.n; i0 += stride) {
+        const int i = i0 + lane < A.n ? (int)(i0 + lane) : -1;
+        double4_32a v = make_double4_32a(0.0, 0.0, 0.0, 1.0);
+        if (i >= 0) {
+            const double4_32a own = A.force[i], acc = A.f_acc[i];
+            const double fx = own.x + acc.x, fy = own.y + acc.y, fz = own.z + acc.z;
+            v = close_step(A, boxes, sp, i, fx, fy, fz, open);
+            pairs_partials64<ENERGY>(A, i, fx, fy, fz, v, part);
+        }
+        if (th) add_kinetic(A, th, i, v);
+    }
 }
 
 // ======================================================================= double-float (MD_PREC_DF)
@@ -1572,11 +1599,12 @@ __device__ __forceinline__ void density_walk(const Atoms &A, const Pot &P, const
     }
 }
 
-// open: see close_step.
+// open: see close_step.  th: the thermostats whose kinetic-energy sums the atoms are added to (NULL:
+// none).
 template <int PREC, int T, int KIND, bool MULTI, bool SMT, bool ENERGY>
 __device__ __forceinline__ void force_walk(const Atoms &A, const Pot &P, const Box *boxes, const StepParams &sp,
                                            long long tid, long long stride, long long items, bool open,
-                                           double (&part)[kPartials]) {
+                                           Thermo *th, double (&part)[kPartials]) {
     for (long long g0 = tid; g0 < items; g0 += stride * T) {
         const Batch<T> b(g0);
         if constexpr (PREC == MD_PREC_MIXED) {
@@ -1595,15 +1623,17 @@ __device__ __forceinline__ void force_walk(const Atoms &A, const Pot &P, const B
                 }
             }
             const int i = b.atom(stride, items, A.n);
+            double4_32a v = make_double4_32a(0.0, 0.0, 0.0, 1.0);
             if (i >= 0) {
                 // (an infinite sum becomes NaN here: not finite either way)
-                const double4_32a v = close_step(A, boxes, sp, i, f64_of_f32(k.fx), f64_of_f32(k.fy), f64_of_f32(k.fz), open);
+                v = close_step(A, boxes, sp, i, f64_of_f32(k.fx), f64_of_f32(k.fy), f64_of_f32(k.fz), open);
                 if (ENERGY) {
                     const double e = A.e_atom[i] + (double)k.ep;
                     A.e_atom[i] = e;
                     add_partials(part, e, v, k);
                 }
             }
+            if (th) add_kinetic(A, th, i, v);
         } else {
             Acc64 k;
 #pragma unroll 1
@@ -1621,14 +1651,16 @@ __device__ __forceinline__ void force_walk(const Atoms &A, const Pot &P, const B
                 }
             }
             const int i = b.atom(stride, items, A.n);
+            double4_32a v = make_double4_32a(0.0, 0.0, 0.0, 1.0);
             if (i >= 0) {
-                const double4_32a v = close_step(A, boxes, sp, i, k.fx, k.fy, k.fz, open);
+                v = close_step(A, boxes, sp, i, k.fx, k.fy, k.fz, open);
                 if (ENERGY) {
                     const double e = A.e_atom[i] + k.ep;
                     A.e_atom[i] = e;
                     add_partials(part, e, v, k);
                 }
             }
+            if (th) add_kinetic(A, th, i, v);
         }
     }
 }

@@ -24,6 +24,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
+#include <type_traits>
 
 #include "md_passes.cuh"
 #include "md_tile.cuh"
@@ -37,34 +39,78 @@ __device__ __forceinline__ unsigned long long globaltimer() {
     return t;
 }
 
-// Generation barrier over all blocks of a cooperative launch (all co-resident).
-__device__ __forceinline__ bool grid_sync(GridBarrier *b, unsigned nblocks, unsigned long long limit, Flags *f) {
+// Barrier over all blocks of a cooperative launch (all co-resident), in two levels above kBarFlat
+// blocks: with one counter, 1,216 blocks took 8.5 us a barrier on GB300 (152: 4.5), each arrival and
+// each poll queueing for the same word.  Thread 0 of a block arrives; the last block runs then() (every
+// thread of it, after all other blocks have arrived and before any leaves) and releases the groups.
+// Polls are relaxed loads, so that waiting blocks do not invalidate the L1 of the blocks still at work
+// on their SM; one fence follows.
+__device__ __forceinline__ unsigned bar_arrive_gpu(unsigned *p) {
+    unsigned old;
+    asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
+    return old;
+}
+__device__ __forceinline__ unsigned bar_peek(const unsigned *p) {
+    unsigned v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void bar_zero(unsigned *p) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(p) : "memory");
+}
+__device__ __forceinline__ void bar_bump(unsigned *p) {
+    asm volatile("red.add.relaxed.gpu.global.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+
+template <typename Then>
+__device__ __forceinline__ bool grid_sync(GridBarrier *b, unsigned nblocks, unsigned long long limit, Flags *f,
+                                          Then &&then) {
+    constexpr bool kThen = !std::is_same_v<std::decay_t<Then>, std::nullptr_t>;
+    const unsigned size = nblocks <= kBarFlat ? kBarFlat : kBarGroup;
+    const unsigned g = blockIdx.x / size, ng = (nblocks + size - 1) / size;
+    GridBarrier::Group *grp = &b->group[g];
+    unsigned gen = 0;
+    bool last = false;
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile unsigned *vgen = &b->gen;
-        const unsigned gen = *vgen;
-        __threadfence();
-        const unsigned arrived = atomicAdd(&b->count, 1u) + 1u;
-        if (arrived == nblocks) {
-            atomicExch(&b->count, 0u);
+        gen = bar_peek(&grp->gen);
+        if (bar_arrive_gpu(&grp->count) == min(size, nblocks - g * size) - 1u) {
+            bar_zero(&grp->count);
+            if (ng > 1u) __threadfence();   // what the group's blocks released, before passing it on
+            last = ng == 1u || bar_arrive_gpu(&b->count) == ng - 1u;
+        }
+    }
+    if constexpr (kThen) {
+        if (__syncthreads_or(last)) {
             __threadfence();
-            atomicAdd(&b->gen, 1u);
+            then();
+            __syncthreads();
+        }
+    }
+    if (threadIdx.x == 0) {
+        if (last) {
+            bar_zero(&b->count);
+            __threadfence();   // (once: the bumps are relaxed)
+            for (unsigned q = 0; q < ng; q++) bar_bump(&b->group[q].gen);
         } else {
             unsigned long long polls = 0;
-            while (*vgen == gen) {
-                if (*reinterpret_cast<volatile int *>(&b->abort)) break;
-                if (++polls > limit) {
+            while (bar_peek(&grp->gen) == gen) {
+                if ((++polls & 15) == 0 && *reinterpret_cast<volatile int *>(&b->abort)) break;
+                if (polls > limit) {
                     atomicExch(&b->abort, 1);
                     atomicOr(&f->error, FLAG_TIMEOUT);
                     break;
                 }
-                __nanosleep(100);
+                if (polls > 32) __nanosleep(64);
             }
         }
         __threadfence();
     }
     __syncthreads();
     return *reinterpret_cast<volatile int *>(&b->abort) == 0;
+}
+__device__ __forceinline__ bool grid_sync(GridBarrier *b, unsigned nblocks, unsigned long long limit, Flags *f) {
+    return grid_sync(b, nblocks, limit, f, nullptr);
 }
 
 // Box matrix times the strain matrix diag(1, 1, s) (§2.2), every replica.
@@ -82,22 +128,15 @@ __device__ __forceinline__ void strain_boxes(Box *boxes, int n_rep, double s) {
 }
 
 // ---- Nose-Hoover thermostat (§2.1.2), one per replica ----
-// Kinetic energy of every replica into its fixed-point accumulator: one warp per chunk of at most
-// kKeChunk atoms of one replica, one integer atomic per chunk (the sum does not depend on order).
+// Kinetic energy of every replica into its fixed-point accumulator (the opening of a call; inside it
+// the force pass adds each atom's as it finishes it, ps::add_kinetic).
 __device__ __forceinline__ void ke_sums(const Atoms &A, const StepParams &sp, long long tid, long long stride) {
     const int lane = threadIdx.x & 31;
-    for (long long c = tid >> 5; c < sp.n_ke_chunks; c += stride >> 5) {
-        const int2 ch = sp.ke_chunks[c];
-        const int end = min(ch.y + kKeChunk, sp.rep_off[ch.x + 1]);
-        unsigned long long acc = 0;
-        for (int i = ch.y + lane; i < end; i += 32) {
-            const double4_32a v = A.vel[i];   // v.w = 1 / (m mvv2e): KE_i = |v|^2 / (2 v.w)
-            const double ke = 0.5 * fma(v.x, v.x, fma(v.y, v.y, v.z * v.z)) / v.w;
-            acc += (unsigned long long)llrint(ke * kKeFix);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (lane == 0) atomicAdd(&sp.thermo[ch.x].ke_fix, acc);
+    for (long long i0 = tid - lane; i0 < A.n; i0 += stride) {
+        const long long i = i0 + lane;
+        double4_32a v = make_double4_32a(0.0, 0.0, 0.0, 1.0);
+        if (i < A.n) v = A.vel[i];
+        ps::add_kinetic(A, sp.thermo, i < A.n ? (int)i : -1, v);
     }
 }
 
@@ -267,6 +306,11 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
     const unsigned nb = gridDim.x;
     const long long tid = (long long)blockIdx.x * NT + threadIdx.x;
     const long long stride = (long long)nb * NT;
+    int s0 = 0;
+    if (sp.resume) {   // the step was opened by the launch that stopped at its rebuild request
+        s0 = *reinterpret_cast<volatile int32_t *>(&A.flags->seg_done);
+        if (s0 >= sp.n_steps || (*reinterpret_cast<volatile int32_t *>(&A.flags->error) & FLAG_TIMEOUT)) return;
+    }
     if (SMT && !kSplitTable) {
         const float4 *src = reinterpret_cast<const float4 *>(P.VP32);
         if constexpr (!MULTI && MD_DTABLE) {   // derivative rows, then the phi rows
@@ -299,11 +343,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
     } while (0)
 
     const bool thermo = sp.thermo != nullptr;
-    int s0 = 0;
-    if (sp.resume) {   // the step was opened by the launch that stopped at its rebuild request
-        s0 = *reinterpret_cast<volatile int32_t *>(&A.flags->seg_done);
-        if (s0 >= sp.n_steps || (*reinterpret_cast<volatile int32_t *>(&A.flags->error) & FLAG_TIMEOUT)) return;
-    } else {
+    if (!sp.resume) {
         if (stamps && lead) stamps[0] = globaltimer();
         // first half kick + drift of the first step
         if (strain) {
@@ -313,9 +353,8 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
         if (lead && sp.rebuild_every > 0 && (step + 1) % sp.rebuild_every == 0) A.flags->need_rebuild = 1;
         if (thermo) {  // the thermostat half step that opens the first step
             ke_sums(A, sp, tid, stride);
-            MD_SYNC();
-            thermo_update(sp, A.n_rep, tid, stride, false, true);
-            MD_SYNC();
+            if (!grid_sync(bar, nb, sp.spin_limit, A.flags, [&] { thermo_update(sp, A.n_rep, threadIdx.x, NT, false, true); }))
+                return;
         }
         for (long long i = tid; i < A.n; i += stride) {
             ph::open_step(A, boxes, (int)i, sp.motion, sp.half_dt, sp.dt, sp.strain_scale, strain, sp.lim,
@@ -431,6 +470,8 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
         const bool fuse = !last && !strain && !thermo;
         if (fuse && lead && sp.rebuild_every > 0 && (step + s + 2) % sp.rebuild_every == 0)
             A.flags->need_rebuild = 1;
+        // (the group walks' own passes do not add the kinetic energies: a pass of their own does)
+        Thermo *const ke = kGroupWalk<WALK> ? nullptr : sp.thermo;
         double part[kPartials];
 #pragma unroll
         for (int q = 0; q < kPartials; q++) part[q] = 0.0;
@@ -476,9 +517,9 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
                 for (long long g = tid; g < items; g += stride)
                     ps::force64_pairs<T, KIND, true>(A, P, boxes, g, part, psum);
                 MD_SYNC();
-                for (long long i = tid; i < A.n; i += stride) ps::pairs_close64<true>(A, boxes, sp, (int)i, false, part);
+                ps::pairs_close64<true>(A, boxes, sp, tid, stride, false, sp.thermo, part);
             } else if (!tiled) {
-                ps::force_walk<PREC, T, KIND, MULTI, SMT, true>(A, P, boxes, sp, tid, stride, items, false, part);
+                ps::force_walk<PREC, T, KIND, MULTI, SMT, true>(A, P, boxes, sp, tid, stride, items, false, ke, part);
             }
             eam::block_partials<NT>(part, A.partials, A.part_stride);
         } else {
@@ -530,23 +571,32 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
                 for (long long g = tid; g < items; g += stride)
                     ps::force64_pairs<T, KIND, false>(A, P, boxes, g, part, psum);
                 MD_SYNC();
-                for (long long i = tid; i < A.n; i += stride) ps::pairs_close64<false>(A, boxes, sp, (int)i, fuse, part);
+                ps::pairs_close64<false>(A, boxes, sp, tid, stride, fuse, sp.thermo, part);
             } else if (!tiled) {
-                ps::force_walk<PREC, T, KIND, MULTI, SMT, false>(A, P, boxes, sp, tid, stride, items, fuse, part);
+                ps::force_walk<PREC, T, KIND, MULTI, SMT, false>(A, P, boxes, sp, tid, stride, items, fuse, ke, part);
             }
         }
-        MD_SYNC();
+        if constexpr (kGroupWalk<WALK>) {
+            if (thermo) {
+                MD_SYNC();
+                ke_sums(A, sp, tid, stride);
+            }
+        }
+        if (thermo) {   // the last block closes this step and opens the next with thermostat half steps
+            if (!grid_sync(bar, nb, sp.spin_limit, A.flags, [&] {
+                    thermo_update(sp, A.n_rep, threadIdx.x, NT, true, !last);
+                    if (!last && threadIdx.x == 0) {
+                        if (strain) strain_boxes(boxes, A.n_rep, sp.strain_scale);
+                        if (sp.rebuild_every > 0 && (A.flags->step + s + 2) % sp.rebuild_every == 0)
+                            A.flags->need_rebuild = 1;
+                    }
+                }))
+                return;
+        } else {
+            MD_SYNC();
+        }
         MD_STAMP(11);
         if (thermo) {
-            // close this step and open the next with thermostat half steps
-            ke_sums(A, sp, tid, stride);
-            MD_SYNC();
-            thermo_update(sp, A.n_rep, tid, stride, true, !last);
-            if (!last && lead) {
-                if (strain) strain_boxes(boxes, A.n_rep, sp.strain_scale);
-                if (sp.rebuild_every > 0 && (step + s + 2) % sp.rebuild_every == 0) A.flags->need_rebuild = 1;
-            }
-            MD_SYNC();
             if (!last) {
                 for (long long i = tid; i < A.n; i += stride)
                     ph::kick_drift(A, boxes, (int)i, sp.half_dt, sp.dt, sp.strain_scale, strain, sp.lim, sp.thermo);
@@ -612,11 +662,9 @@ cudaError_t launch_t(const Atoms &A, const Cells &C, const Pot &P, const StepPar
     }
     const long long work = std::max<long long>((long long)A.n * T, (long long)C.ncell);
     const int need = (int)std::max<long long>(1, (work + NT - 1) / NT);
-    const int grid = std::max(1, std::min(per_sm * n_sm, need));
+    const int grid = std::max(1, std::min(std::min(per_sm * n_sm, kGridMax), need));
     if (grid_out) *grid_out = grid;
     if (sp.n_steps <= 0) return cudaSuccess;  // preparation only (attributes, occupancy): no launch
-    cudaError_t e = cudaMemsetAsync(bar, 0, sizeof(GridBarrier), s);
-    if (e != cudaSuccess) return e;
     Atoms a = A;
     Cells c = C;
     Pot p = P;
@@ -663,10 +711,8 @@ cudaError_t launch_rebuild_t(const Atoms &A, const Cells &C, const StepParams &s
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rebuild<WALK>, kRebuildThreads, 0);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        grid = per_sm * n_sm;
+        grid = std::min(per_sm * n_sm, kGridMax);
     }
-    cudaError_t e = cudaMemsetAsync(bar, 0, sizeof(GridBarrier), s);
-    if (e != cudaSuccess) return e;
     Atoms a = A;
     Cells c = C;
     StepParams q = sp;
