@@ -603,7 +603,14 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
         ncell += (long long)ctx->rc[r].nc[0] * ctx->rc[r].nc[1] * ctx->rc[r].nc[2];
         if (ncell > INT32_MAX / 2) return MD_ERR_BOX;
     }
-    // lanes per atom: given, or from the expected neighbour count (4/3 pi r_list^3 x density)
+    // lanes per atom: given, or from the expected neighbour count (4/3 pi r_list^3 x density) and the
+    // number of atoms, measured on GB300, us a step at 1 / 2 / 4 / 8 lanes.  About 20 entries a lane (24
+    // for the FP32 terms): bcc Fe mixed 624,000 atoms 135 / 149 / 175 / 220, 35,000 22.7 / 24.2 / 27.8 /
+    // 30.2; fcc Cu FP64 83,000 - / 1319 / 1040 / 906, half list 88,000 - / 919 / 687 / 658, mixed 88,000 - /
+    // 176 / 148 / 136.  Half of that once the mixed lanes fill the chip 16 times, where fewer, longer walks
+    // gather better: fcc Cu 500,000 682 / 592 / 575 / 626.  A system that does not fill the chip takes
+    // more lanes, up to 8 (the group walks' most) and one for every other entry: bcc Fe FP64 2,000
+    // - / 33.9 / 24.3 / 18.2, mixed 3,456 21.2 / 18.2 / 16.6 / 16.2 but 11,664 21.1 / 19.5 / 22.3 / 24.9.
     {
         const int want = cfg->lanes_per_atom;
         if (want != 0 && want != 1 && want != 2 && want != 4 && want != 8 && want != 16 && want != 32)
@@ -614,8 +621,15 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
             double vol = 0.0;
             for (int r = 0; r < n_rep; r++) vol += L[3 * r] * L[3 * r + 1] * L[3 * r + 2];
             const double k_est = 4.18879020478639 * ctx->r_list * ctx->r_list * ctx->r_list * (double)n / vol;
-            int t = 1;
-            while (t < 8 && t * 12 < k_est) t *= 2;
+            const bool mixed = cfg->precision == MD_PREC_MIXED;
+            int t = 1, dev = 0, n_sm = 0;
+            while (t < 8 && t * (mixed ? 24 : 20) < k_est) t *= 2;
+            if (cudaGetDevice(&dev) != cudaSuccess ||
+                cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+                return MD_ERR_CUDA;
+            if (mixed && t > 1 && n * t > 16 * (int64_t)n_sm * 1024) t /= 2;
+            const int64_t fill = (int64_t)n_sm * (mixed ? 192 : 512);
+            while (t < 8 && 2 * n * t <= fill && 4 * t <= k_est) t *= 2;
             ctx->lanes = t;
         }
     }
