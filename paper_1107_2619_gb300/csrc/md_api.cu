@@ -24,6 +24,7 @@
 #include <string>
 #include <vector>
 
+#include "md_bits.cuh"
 #include "md_df.cuh"
 #include "md_internal.cuh"
 
@@ -197,7 +198,7 @@ int cells_along(double L, double r_list) {
 // skin: the double-float offset xoff = 2 (L + skin) + 1 keeps every image coordinate plus xoff
 // within a factor of two of every other (image coordinates lie in [-skin/2, L + skin/2)), also
 // while a strain ramp shrinks the box, so that differences of their FP32 high parts are exact.
-Box make_box(const double *L, double skin) {
+Box make_box(const double *L, double skin, int qfb) {
     Box b;
     for (int k = 0; k < 3; k++) {
         b.L[k] = L[k];
@@ -207,6 +208,7 @@ Box make_box(const double *L, double skin) {
         b.Lh[k] = (float)L[k];
         b.Ll[k] = (float)(L[k] - (double)b.Lh[k]);
         b.xoff[k] = 2.0 * (L[k] + skin) + 1.0;
+        b.Lq[k] = eam::fix64(L[k], qfb);
     }
     return b;
 }
@@ -917,6 +919,76 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
         for (size_t k = 0; k < F64.size(); k++)
             FD64[k] = make_double4_32a(F64[k].y * P.inv_drho, 2.0 * F64[k].z * P.inv_drho, 3.0 * F64[k].w * P.inv_drho, 0.0);
         P.xmax_rho = nk - 1;
+        // FP64, one species: the pair terms from FP32 pieces (ps::pair_terms_q), where every coefficient
+        // is well inside FP32's range, relative to the largest of its function, and the fixed-point
+        // numbers hold the list's separations, the knots and the box; else FP64 arithmetic throughout
+        std::vector<float4> TQ;
+        if (ns == 1 && cfg->precision == MD_PREC_FP64) {
+            double Lmax = 0.0;
+            for (double l : L) Lmax = std::fmax(Lmax, l);
+            // |separation| < 2^(53 - fb) for every pair of the list, twice the skin and a tenth to spare
+            const int fb = std::min(53 - (int)std::ceil(std::log2(1.1 * (ctx->r_list + 2.0 * cfg->skin))),
+                                    61 - (int)std::ceil(std::log2(2.0 * Lmax + 2.0 * cfg->skin)));
+            const int U = 2 * fb - 42;
+            const float hrf = (float)hr, rmf = (float)pot->r_min;
+            // r^2 - rho^2 within a row and a half of rho_k: 24 bits in the high part, the rest below
+            const int dbits = (int)std::ceil(std::log2(3.0 * pot->r_cut * hr)) + U;
+            auto fits = [](double m) { return m == 0.0 || (m >= std::ldexp(1.0, -60) && m <= std::ldexp(1.0, 60)); };
+            double mv = 0.0, mp = 0.0, mf = 0.0;
+            for (int k = 0; k < nk; k++) {
+                const double4_32a &v = VP64[2 * k], &p = VP64[2 * k + 1];
+                mv = std::max({mv, std::fabs(v.x), std::fabs(v.y), std::fabs(v.z), std::fabs(v.w)});
+                mp = std::max({mp, std::fabs(p.x), std::fabs(p.y), std::fabs(p.z), std::fabs(p.w)});
+                mf = std::max({mf, std::fabs(FD64[k].x), std::fabs(FD64[k].y), std::fabs(FD64[k].z)});
+            }
+            // (rho_0^2 a whole number of the units; rho_k within 1e-3 of a row of its knot)
+            const int whole = rmf > 0.f ? U - 300 + 2 * (std::ilogb(rmf) + 127) : -1;
+            if (fb >= 45 && fb <= 51 && nk <= 20000 && whole >= 0 && dbits >= 25 && dbits <= 55 && fits(mv) &&
+                fits(mp) && fits(mf) && fits(P.inv_dr)) {
+                A.qfb = fb;
+                P.hr_f = hrf;
+                P.r_min_f = rmf;
+                P.rc2q = (unsigned long long)std::ceil(std::ldexp((long double)P.rc2, U));
+                P.qs1 = (float)std::ldexp(1.0, 29 - fb);
+                P.qe1 = (unsigned)(127 + 23 + 14 - fb) << 23;
+                P.qe0 = (unsigned)(127 + 23 - fb) << 23;
+                P.q2h = (float)std::ldexp(1.0, 40 - U);
+                P.q2l = (float)std::ldexp(1.0, 8 - U);
+                P.q2e = U - 300;
+                P.dsh = dbits - 24;
+                P.dsc1 = (float)std::ldexp(1.0, P.dsh - U);
+                P.dsc0 = (float)std::ldexp(1.0, -U);
+                const df::F2 idr = df::from_double(P.inv_dr), x0 = df::from_double(pot->r_min * P.inv_dr);
+                P.idr_h = idr.h;
+                P.idr_l = idr.l;
+                P.x0_h = x0.h;
+                P.x0_l = x0.l;
+                TQ.resize(4 * (size_t)nk);
+                for (int k = 0; k < nk; k++) {
+                    // the row's cubics about rho_k, s rows beyond its knot
+                    const long double s = ((long double)std::fma((float)k, hrf, rmf) - pot->r_min) * P.inv_dr - k;
+                    auto about = [s](const double4_32a &c) {
+                        return make_double4_32a((double)(c.x + s * (c.y + s * (c.z + s * c.w))),
+                                                (double)(c.y + s * (2 * c.z + 3 * s * c.w)), (double)(c.z + 3 * s * c.w), c.w);
+                    };
+                    const double4_32a v = about(VP64[2 * k]), p = about(VP64[2 * k + 1]);
+                    auto two = [](double x, double y) {
+                        const df::F2 a = df::from_double(x), b = df::from_double(y);
+                        return make_float4(a.h, a.l, b.h, b.l);
+                    };
+                    TQ[4 * k] = two(p.x, p.y);
+                    TQ[4 * k + 1] = two(p.z, p.w);
+                    TQ[4 * k + 2] = two(v.y, v.z);
+                    TQ[4 * k + 3] = two(v.w, v.x);
+                }
+                float4 *dTQ;
+                chk(dalloc(ctx, &A.posq, n));
+                chk(dalloc(ctx, &dTQ, TQ.size()));
+                if (e != cudaSuccess) return fail(ctx, MD_ERR_OOM, "table allocation", e);
+                chk(cudaMemcpy(dTQ, TQ.data(), TQ.size() * sizeof(float4), cudaMemcpyHostToDevice));
+                P.TQ = dTQ;
+            }
+        }
         double4_32a *dVP64, *dVP32, *dF64, *dFD64;
         chk(dalloc(ctx, &dVP64, VP64.size()));
         chk(dalloc(ctx, &dVP32, VP32.size() / 8));
@@ -982,7 +1054,7 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
     }
     // initial state (caller order = cell order until the first build)
     std::vector<Box> boxes(n_rep);
-    for (int r = 0; r < n_rep; r++) boxes[r] = make_box(&L[3 * r], cfg->skin);
+    for (int r = 0; r < n_rep; r++) boxes[r] = make_box(&L[3 * r], cfg->skin, A.qfb);
     std::vector<int32_t> off32(n_rep + 1);
     for (int r = 0; r <= n_rep; r++) off32[r] = (int32_t)ctx->rep_off[r];
     Flags flags{};
@@ -1642,13 +1714,11 @@ md_status md_tune(md_ctx *ctx, int32_t *lanes_out) {
         // atom is renumbered; the state the steps change is saved first and put back after
         // every trial.
         const size_t n = (size_t)ctx->n;
-        const size_t bytes = n * (4 * sizeof(double4_32a) + sizeof(float4)) + sizeof(Flags);
+        const size_t bytes = n * 3 * sizeof(double4_32a) + sizeof(Flags);
         unsigned char *snap = nullptr;
         MD_CK(cudaMalloc(&snap, bytes));
         double4_32a *s_pos = reinterpret_cast<double4_32a *>(snap), *s_vel = s_pos + n, *s_force = s_vel + n;
-        double4_32a *s_posd = s_force + n;
-        float4 *s_posf = reinterpret_cast<float4 *>(s_posd + n);
-        Flags *s_flags = reinterpret_cast<Flags *>(s_posf + n);
+        Flags *s_flags = reinterpret_cast<Flags *>(s_force + n);
         Atoms &A = ctx->A;
         auto copy = [&](bool save) {
             const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
@@ -1656,9 +1726,7 @@ md_status md_tune(md_ctx *ctx, int32_t *lanes_out) {
             if (e == cudaSuccess) e = cudaMemcpyAsync(save ? s_vel : A.vel, save ? A.vel : s_vel, n * 32, k, ctx->stream);
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(save ? s_force : A.force, save ? A.force : s_force, n * 32, k, ctx->stream);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(save ? s_posf : A.posf, save ? A.posf : s_posf, n * 16, k, ctx->stream);
-            if (e == cudaSuccess && A.posd)
-                e = cudaMemcpyAsync(save ? s_posd : A.posd, save ? A.posd : s_posd, n * 32, k, ctx->stream);
+            if (e == cudaSuccess && !save) e = launch_wrap(A, ctx->stream);   // the copies that the passes read
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(save ? s_flags : ctx->d_flags, save ? ctx->d_flags : s_flags, sizeof(Flags), k,
                                     ctx->stream);

@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <string.h>
 
 namespace mdk {
 namespace eam {
@@ -52,6 +53,23 @@ __device__ __forceinline__ float f32_rn(double x) {
     if (mag >= (1151u << 20)) m = (mag > 0x7ff00000u || (mag == 0x7ff00000u && lo)) ? 0x7fc00000u : 0x7f800000u;
     return __uint_as_float(sgn | m);
 }
+// x in units of 2^-fb as a whole number, rounded to nearest (0 <= fb <= 60), saturated to 62 bits.
+__host__ __device__ __forceinline__ long long fix64(double x, int fb) {
+#ifdef __CUDA_ARCH__
+    const long long b = __double_as_longlong(x);
+#else
+    long long b;
+    memcpy(&b, &x, sizeof b);
+#endif
+    const int e = (int)((b >> 52) & 0x7ff) - 1023;
+    const long long m = (b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;
+    const int s = e - 52 + fb;   // x = m 2^(e - 52)
+    long long v;
+    if (s >= 0) v = s <= 9 ? m << s : (1LL << 62);
+    else v = s > -54 ? (m + (1LL << (-s - 1))) >> -s : 0;
+    return b < 0 ? -v : v;
+}
+
 // Whether v is finite.
 __device__ __forceinline__ bool finite64(double v) {
     return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;

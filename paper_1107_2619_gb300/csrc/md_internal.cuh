@@ -40,6 +40,7 @@ struct Box {
     // two of each other and their differences are exact
     float Lh[3], Ll[3];
     double xoff[3];
+    long long Lq[3];   // fixed-point copies (Atoms::qfb): L in units of 2^-qfb
 };
 
 // Device-side status, read by the host after each synchronising call.
@@ -94,6 +95,19 @@ struct Pot {
     // (c2, c3, 0, 0) for the energy
     const float4 *TX;
     const float4 *TVx;
+    // one species, FP64 path: the cubics of V and phi of an interval about rho_k (ps::pair_terms_q),
+    // each coefficient as hi + lo: [4k]: phi (c0, c1), [4k + 1]: phi (c2, c3), [4k + 2]: V (c1, c2),
+    // [4k + 3]: V (c3, c0).  rho_k = fma(k, hr_f, r_min_f)
+    const float4 *TQ;
+    float hr_f, r_min_f;
+    // fixed-point coordinates in units of 2^-qfb (Atoms::qfb), r^2 in units of 2^-U, U = 2 qfb - 42
+    unsigned long long rc2q;  // r_cut^2
+    float qs1;                // 2^(29 - qfb)
+    unsigned qe1, qe0;        // the FP32 numbers whose last bit is worth 2^(14 - qfb), 2^-qfb
+    float q2h, q2l;           // 2^(40 - U), 2^(8 - U)
+    int q2e;                  // U - 300: rho^2 = significand^2 2^(q2e + 2 exponent field)
+    int dsh;                  // low bits of r^2 - rho^2 taken as the low part
+    float dsc1, dsc0;         // 2^(dsh - U), 2^-U
     float idr_h, idr_l;       // inv_dr as hi + lo
     float x0_h, x0_l;         // r_min inv_dr as hi + lo
     float dsv, dsp;
@@ -148,6 +162,11 @@ struct Atoms {
     double4_32a *posd;                           // FP64 path: pos in the periodic image of the last
                                                  // build (as posf; NULL on the mixed path)
     double4_32a *pos_tmp, *vel_tmp, *force_tmp;  // renumbering scratch
+    // FP64, one species with knot tables: fixed-point copies of the image coordinates, the bits of whole
+    // numbers in units of 2^-qfb in x, y, z (qfb 0: not kept, the pair terms are FP64 arithmetic
+    // throughout); p2d then holds the same, and F'(rho) as two FP32 numbers in w
+    double4_32a *posq;
+    int qfb;
     float4 *posf;                            // FP32 wrapped position, w = species bits
     float4 *reff;                            // posf at the last build (ph::place's skin screen); w = the
                                              // box edges wrapped off there (ph::pack_image)

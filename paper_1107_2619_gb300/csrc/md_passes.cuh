@@ -447,6 +447,175 @@ __device__ __forceinline__ void force32_item(const Atoms &A, const Pot &P, const
     if (i < A.n && (g & (T - 1)) == 0) force32_finish<ENERGY>(A, i, a, half_dt, motion, part);
 }
 
+// ======================================================================= FP64 pair terms from FP32 pieces
+// One species with knot tables.  GB300's FP64 pipe runs at 1/64 of the FP32 rate, so the terms of a
+// pair are formed as unevaluated sums of two FP32 numbers (md_df.cuh) and enter the FP64 sums with one
+// FP64 addition each; sums, F(rho), integration and reductions are FP64 as before.
+//  - Separations are exact whole-number differences of fixed-point coordinates (Atoms::posq, 2^-50 Å
+//    for r_list up to 6.6 Å, 2^-49 Å up to 13.9 Å), and r^2 their sum of squares in 64 bits, rounded to
+//    about 2^-58 Å^2; the cut is a comparison of whole numbers.
+//  - 1/r by Newton's step from the FP32 estimate with its second-order term, as hi + lo.
+//  - The knot coordinate t = (r - rho_k) / h from r^2 - rho_k^2, an exact whole-number difference, over
+//    r + rho_k: rho_k, the knot rounded to FP32, has an exact square, and the rows are cubics about it
+//    (the difference r - r_k itself, at 5,000 knots, would cost t twelve bits).
+//  - The cubic of phi and the slopes of V and phi with every coefficient as hi + lo.
+// Against 64-bit arithmetic the forces are closer than those of the FP64 evaluation they replace,
+// whose 1/r took one Newton step without the second-order term (on thermal fcc Cu 3e-14 of the RMS
+// force from the pair terms, 1.1e-13 before).  About 250 FP32 and whole-number operations a pair stand
+// in place of 16 on the FP64 pipe, each of which takes the time of 75.
+
+struct PairQ {
+    df::F2 phi, gphi, gV, V;   // phi(r), phi'(r) / r, V'(r) / r, V(r) (energy only)
+};
+
+// Product and sum of double-floats, not renormalised.
+__device__ __forceinline__ df::F2 mul_raw(df::F2 a, df::F2 b) {
+    df::F2 p = df::two_prod(a.h, b.h);
+    p.l = __fmaf_rn(a.h, b.l, p.l);
+    p.l = __fmaf_rn(a.l, b.h, p.l);
+    return p;
+}
+__device__ __forceinline__ df::F2 add_raw(df::F2 a, df::F2 b) {
+    const df::F2 s = df::two_sum(a.h, b.h);
+    return df::make(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+
+// x_j - x_i of fixed-point coordinates (minimum image with WRAP; s: the whole box edges taken off, in
+// the same units).
+template <typename WRAP>
+__device__ __forceinline__ long long sep_fixed(double xj, double xi, long long Lq, long long &s) {
+    const long long D = __double_as_longlong(xj) - __double_as_longlong(xi);
+    s = 0;
+    if (!WRAP::value) return D;
+    const long long half = Lq >> 1;
+    s = D > half ? Lq : (D < -half ? -Lq : 0);
+    return D - s;
+}
+// A separation as a double-float in Å, to 2^-48 of itself: 24 bits and a sign, then 15 and 14 bits
+// (each exact, through the significand of a number of the right exponent).
+__device__ __forceinline__ df::F2 sep_df64(const Pot &P, long long D) {
+    const float a = __fmul_rn(__int2float_rn((int)(D >> 29)), P.qs1);
+    const unsigned lo = (unsigned)D & 0x1fffffffu;
+    const float b = __fsub_rn(__uint_as_float(P.qe1 | (lo >> 14)), __uint_as_float(P.qe1));
+    const float c = __fsub_rn(__uint_as_float(P.qe0 | (lo & 0x3fffu)), __uint_as_float(P.qe0));
+    const df::F2 d = df::two_sum(a, b);
+    return df::make(d.h, __fadd_rn(d.l, c));
+}
+// r^2 in units of 2^-(2 qfb - 42) Å^2 (64 bits hold it for any pair of the list).
+template <typename WRAP>
+__device__ __forceinline__ unsigned long long r2_fixed(const double4_32a &xj, const double4_32a &xi, const Box &B) {
+    long long s;
+    auto sq = [](long long D) {
+        const unsigned long long u = (unsigned long long)(D < 0 ? -D : D) << 11;
+        return __umul64hi(u, u);
+    };
+    return sq(sep_fixed<WRAP>(xj.x, xi.x, B.Lq[0], s)) + sq(sep_fixed<WRAP>(xj.y, xi.y, B.Lq[1], s)) +
+           sq(sep_fixed<WRAP>(xj.z, xi.z, B.Lq[2], s));
+}
+
+// The terms of a pair at r2 = r^2 (r2_fixed), inside r_cut.
+__device__ __forceinline__ void pair_terms_q(const Pot &P, unsigned long long r2, bool energy, PairQ &o, Flags *flags) {
+    const df::F2 x2 = df::make(__fmul_rn(__uint2float_rn((unsigned)(r2 >> 40)), P.q2h),
+                               __fmul_rn(__uint2float_rn((unsigned)(r2 >> 8)), P.q2l));
+    // 1/r: estimate y, e = 1 - r^2 y^2 as hi + lo, 1/r = y + y (e/2 + 3 e^2/8)
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x2.h));
+    const df::F2 yy = df::two_prod(y, y), m = df::two_prod(x2.h, yy.h);
+    const df::F2 e = df::two_sum(__fsub_rn(1.f, m.h), -__fmaf_rn(x2.h, yy.l, __fmaf_rn(x2.l, yy.h, m.l)));
+    const float hy = 0.5f * y;
+    const df::F2 c = df::two_prod(hy, e.h);
+    df::F2 rinv = df::fast_two_sum(y, c.h);
+    rinv.l = __fadd_rn(rinv.l, __fmaf_rn(hy, __fmaf_rn(0.75f * e.h, e.h, e.l), c.l));
+    const df::F2 r = mul_raw(x2, rinv);
+    // the row: its knot by rounding x - 1/2, to a few 1e-4 of a row (corrected below)
+    const df::F2 idr = df::make(P.idr_h, P.idr_l);
+    const float x = __fmaf_rn(r.h, P.idr_h, -P.x0_h), last = (float)(P.nk - 1);
+    float kf = __fsub_rn(__fadd_rn(__fsub_rn(x, 0.5f), 12582912.f), 12582912.f);
+    kf = fminf(fmaxf(kf, 0.f), last);   // (a NaN x: row 0, and t carries it on)
+    const float4 *row = P.TQ + 4 * (size_t)(int)kf;
+    float4 p0 = __ldg(row), p1 = __ldg(row + 1), v0 = __ldg(row + 2), v1 = __ldg(row + 3);
+    const bool below = x < 0.f;   // linear continuation below the first knot, any distance from it
+    if (below) atomicAdd(&flags->range_violations, 1ull);
+    // t = (r^2 - rho^2) / (r + rho) / h
+    auto coord = [&](float k) {
+        const float rho = __fmaf_rn(k, P.hr_f, P.r_min_f);
+        const unsigned rb = __float_as_uint(rho), sg = (rb & 0x7fffffu) | 0x800000u;
+        const unsigned long long rho2 = ((unsigned long long)sg * sg) << (P.q2e + 2 * (int)(rb >> 23));
+        const long long del = (long long)(r2 - rho2);
+        df::F2 dd = df::make(__fmul_rn(__int2float_rn((int)(del >> P.dsh)), P.dsc1),
+                             __fmul_rn(__uint2float_rn((unsigned)del & ((1u << P.dsh) - 1u)), P.dsc0));
+        if (below) {
+            const float f = __ll2float_rn(del);
+            dd = df::make(__fmul_rn(f, P.dsc0), __fmul_rn(__ll2float_rn(del - (long long)f), P.dsc0));
+        }
+        df::F2 sum = df::two_sum(r.h, rho);
+        sum.l = __fadd_rn(sum.l, r.l);
+        float w;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(sum.h));
+        const float we = __fmaf_rn(-sum.l, w, __fmaf_rn(-sum.h, w, 1.f));
+        const df::F2 tr = mul_raw(mul_raw(dd, df::make(w, __fmul_rn(w, __fmaf_rn(we, we, we)))), idr);
+        return df::fast_two_sum(tr.h, tr.l);
+    };
+    df::F2 t = coord(kf);
+    // The neighbouring row where t lies outside [0, 1): beside its interval by 1e-4 of a row a cubic's
+    // slope is off by about 1e-12 (its second derivative jumps at the knots), which such rows, one in
+    // some thousand, would make the largest error of all.
+    const float move = t.h < 0.f ? -1.f : (t.h > 1.f || (t.h == 1.f && t.l >= 0.f) ? 1.f : 0.f);
+    if (move != 0.f && !below && kf + move >= 0.f && kf + move <= last) {
+        kf += move;
+        row = P.TQ + 4 * (size_t)(int)kf;
+        p0 = __ldg(row);
+        p1 = __ldg(row + 1);
+        v0 = __ldg(row + 2);
+        v1 = __ldg(row + 3);
+        t = coord(kf);
+    }
+    const float on = below ? 0.f : 1.f;
+    const df::F2 c2 = df::make(p1.x * on, p1.y * on), c3 = df::make(p1.z * on, p1.w * on);
+    const df::F2 w2 = df::make(v0.z * on, v0.w * on), w3 = df::make(v1.x * on, v1.y * on);
+    // q = c3 t, then c2 + q for the value and 2 c2 + 3 q for the slope
+    const df::F2 q = mul_raw(t, c3), u = add_raw(c2, q);
+    const df::F2 du = add_raw(df::make(2.f * u.h, 2.f * u.l), q);
+    const df::F2 srinv = mul_raw(rinv, idr);   // the slopes are in t: phi' = inv_dr d/dt
+    o.phi = add_raw(df::make(p0.x, p0.y), mul_raw(t, add_raw(df::make(p0.z, p0.w), mul_raw(t, u))));
+    o.gphi = mul_raw(add_raw(df::make(p0.z, p0.w), mul_raw(t, du)), srinv);
+    const df::F2 wq = mul_raw(t, w3), wu = add_raw(w2, wq);
+    const df::F2 dwu = add_raw(df::make(2.f * wu.h, 2.f * wu.l), wq);
+    o.gV = mul_raw(add_raw(df::make(v0.x, v0.y), mul_raw(t, dwu)), srinv);
+    if (energy) o.V = add_raw(df::make(v1.z, v1.w), mul_raw(t, add_raw(df::make(v0.x, v0.y), mul_raw(t, wu))));
+}
+
+// A double-float as FP64: one FP64 addition, the conversions on the bit fields.
+__device__ __forceinline__ double to64(df::F2 a) { return f64_of_f32(a.h) + f64_of_f32(a.l); }
+
+// The entry of the derivative cache: (gV, gphi), negated for the half list.
+__device__ __forceinline__ float4 cache_q(const PairQ &o, bool negate) {
+    return negate ? make_float4(-o.gV.h, -o.gV.l, -o.gphi.h, -o.gphi.l) : make_float4(o.gV.h, o.gV.l, o.gphi.h, o.gphi.l);
+}
+// The pair's radial factor g = gV + (F'_i + F'_j) gphi from the cache entry and F' as kept in p2d.w.
+__device__ __forceinline__ df::F2 fprime_q(double w) {
+    const long long b = __double_as_longlong(w);
+    return df::make(__int_as_float((int)(b >> 32)), __int_as_float((int)b));
+}
+__device__ __forceinline__ double pack_fprime(double dF) {
+    const float h = f32_rn(dF);
+    const float l = f32_rn(dF - f64_of_f32(h));
+    return __longlong_as_double(((long long)__float_as_int(h) << 32) | (unsigned)__float_as_int(l));
+}
+__device__ __forceinline__ df::F2 radial_q(const float4 &e, df::F2 Fi, df::F2 Fj) {
+    return df::add(df::make(e.x, e.y), mul_raw(df::add(Fi, Fj), df::make(e.z, e.w)));
+}
+// The pass-2 copy of atom i in its p2d record.
+__device__ __forceinline__ void store_pass2(const Atoms &A, int i, double dF) {
+    if (A.qfb) {
+        const double4_32a p = ld_phase(A.posq + i);
+        A.p2d[i] = make_double4_32a(p.x, p.y, p.z, pack_fprime(dF));
+    } else {
+        const double4_32a p = ld_phase(A.posd + i);
+        A.p2d[i] = make_double4_32a(p.x, p.y, p.z, dF);
+    }
+}
+
 // ======================================================================= FP64
 // Per-atom sums of the FP64 force pass (and of the double-float pass, converted).
 struct Acc64 {
@@ -512,6 +681,31 @@ __device__ __forceinline__ void density64_sum(const Atoms &A, const Pot &P, cons
         // one species: keep (V'/r, phi'/r) of every entry for the force passes without energies
         const bool keep = !MULTI && A.dcache != nullptr;
         const DRow drow = dcache_row(A, i);
+        auto walk_q = [&](auto wrapt) {   // the pair terms from FP32 pieces
+            using W = decltype(wrapt);
+            const double4_32a qi = ld_phase(A.posq + i);
+            for (int k = lane; k < cnt; k += T) {
+                const int j = ld_phase(row.ptr(k));
+                const double4_32a qj = ld_phase(A.posq + j);
+                float4 *dc = reinterpret_cast<float4 *>(drow.ptr(k));
+                const unsigned long long r2 = r2_fixed<W>(qj, qi, B);
+                if (r2 >= P.rc2q) {
+                    *dc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    continue;
+                }
+                PairQ o;
+                pair_terms_q(P, r2, energy, o, A.flags);
+                rho += to64(o.phi);
+                if (energy) ep = fma(0.5, to64(o.V), ep);
+                *dc = cache_q(o, false);
+            }
+        };
+        if constexpr (KIND == MD_POT_TABLES && !MULTI) {
+            if (A.qfb) {
+                if (wrap) walk_q(std::true_type{});
+                else walk_q(std::false_type{});
+            }
+        }
         auto walk = [&](auto wrapt) {
             using W = decltype(wrapt);
             for (int k = lane; k < cnt; k += T) {
@@ -568,8 +762,10 @@ __device__ __forceinline__ void density64_sum(const Atoms &A, const Pot &P, cons
                 }
             }
         };
-        if (wrap) walk(std::true_type{});
-        else walk(std::false_type{});
+        if (!A.qfb) {
+            if (wrap) walk(std::true_type{});
+            else walk(std::false_type{});
+        }
     }
     rho = lane_sum<T>(rho);
     if (energy) ep = lane_sum<T>(ep);
@@ -585,8 +781,7 @@ __device__ __forceinline__ void density64_finish(const Atoms &A, const Pot &P, i
         A.dF[i] = dF;
         A.e_atom[i] = F + ep;
     }
-    const double4_32a p = ld_phase(A.posd + i);
-    A.p2d[i] = make_double4_32a(p.x, p.y, p.z, dF);
+    store_pass2(A, i, dF);
 }
 
 template <int T, int KIND, bool MULTI>
@@ -616,6 +811,41 @@ __device__ __forceinline__ void force64_cached_sum(const Atoms &A, const Pot &P,
         const int cnt = min(A.count[i], A.k_max);
         const NbrRow row = nbr_row(A, i);
         const DRow drow = dcache_row(A, i);
+        auto walk_q = [&](auto wrapt) {   // the pair terms from FP32 pieces
+            using W = decltype(wrapt);
+            const df::F2 Fi = fprime_q(pi.w);
+            for (int k = lane; k < cnt; k += T) {
+                const float4 e = ld_phase(reinterpret_cast<const float4 *>(drow.ptr(k)));
+                const int j = ld_phase(row.ptr(k));
+                if (((__float_as_uint(e.x) | __float_as_uint(e.z)) << 1) == 0u) continue;   // beyond r_cut
+                const double4_32a pj = ld_phase(A.p2d + j);
+                long long s;
+                const df::F2 dx = sep_df64(P, sep_fixed<W>(pj.x, pi.x, B.Lq[0], s)),
+                             dy = sep_df64(P, sep_fixed<W>(pj.y, pi.y, B.Lq[1], s)),
+                             dz = sep_df64(P, sep_fixed<W>(pj.z, pi.z, B.Lq[2], s));
+                const df::F2 g = radial_q(e, Fi, fprime_q(pj.w));
+                const df::F2 gx = mul_raw(g, dx), gy = mul_raw(g, dy), gz = mul_raw(g, dz);
+                fx += to64(gx);
+                fy += to64(gy);
+                fz += to64(gz);
+                if (ENERGY) {   // -1/2 g d (x) d (the pair energies are in E_i: density pass)
+                    const df::F2 hx = df::make(-0.5f * gx.h, -0.5f * gx.l), hy = df::make(-0.5f * gy.h, -0.5f * gy.l);
+                    wxx += to64(mul_raw(hx, dx));
+                    wyy += to64(mul_raw(hy, dy));
+                    wzz += to64(mul_raw(df::make(-0.5f * gz.h, -0.5f * gz.l), dz));
+                    wyz += to64(mul_raw(hy, dz));
+                    wxz += to64(mul_raw(hx, dz));
+                    wxy += to64(mul_raw(hx, dy));
+                }
+            }
+        };
+        if constexpr (KIND == MD_POT_TABLES) {
+            if (A.qfb) {
+                if (wrap) walk_q(std::true_type{});
+                else walk_q(std::false_type{});
+                return;
+            }
+        }
         auto walk = [&](auto wrapt) {
             using W = decltype(wrapt);
             for (int k = lane; k < cnt; k += T) {
@@ -776,6 +1006,37 @@ __device__ __forceinline__ void density64_pairs_item(const Atoms &A, const Pot &
         const int cnt = ld_phase(A.cup + i);
         const NbrRow row = nbr_row(A, i);
         const DRow drow = dcache_row(A, i);
+        auto walk_q = [&](auto wrapt) {   // the pair terms from FP32 pieces
+            using W = decltype(wrapt);
+            const double4_32a qi = ld_phase(A.posq + i);
+            for (int k = lane; k < cnt; k += T) {
+                const int j = ld_phase(row.ptr(k));
+                const double4_32a qj = ld_phase(A.posq + j);
+                float4 *dc = reinterpret_cast<float4 *>(drow.ptr(k));
+                const unsigned long long r2 = r2_fixed<W>(qj, qi, B);
+                if (r2 >= P.rc2q) {
+                    *dc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    continue;
+                }
+                PairQ o;
+                pair_terms_q(P, r2, energy, o, A.flags);
+                const double phi = to64(o.phi);
+                rho += phi;
+                atomicAdd(A.rho_acc + j, phi);
+                if (energy) {   // each atom of the pair gets half its pair energy
+                    const double hV = half64(to64(o.V));
+                    ep += hV;
+                    atomicAdd(A.e_acc + j, hV);
+                }
+                *dc = cache_q(o, true);
+            }
+        };
+        if constexpr (KIND == MD_POT_TABLES) {
+            if (A.qfb) {
+                if (wrap) walk_q(std::true_type{});
+                else walk_q(std::false_type{});
+            }
+        }
         auto walk = [&](auto wrapt) {
             using W = decltype(wrapt);
             for (int k = lane; k < cnt; k += T) {
@@ -821,8 +1082,10 @@ __device__ __forceinline__ void density64_pairs_item(const Atoms &A, const Pot &
                 *drow.ptr(k) = make_double2(-dV * rinv, -dphi * rinv);   // negated (the force pass needs -g)
             }
         };
-        if (wrap) walk(std::true_type{});
-        else walk(std::false_type{});
+        if (!A.qfb) {
+            if (wrap) walk(std::true_type{});
+            else walk(std::false_type{});
+        }
     }
     rho = lane_sum<T>(rho);
     if (energy) ep = lane_sum<T>(ep);
@@ -846,10 +1109,46 @@ __device__ __forceinline__ void pairs_embed64(const Atoms &A, const Pot &P, int 
         A.e_atom[i] = F + A.e_acc[i];
         A.e_acc[i] = 0.0;
     }
-    const double4_32a p = A.posd[i];
-    A.p2d[i] = make_double4_32a(p.x, p.y, p.z, dF);
+    store_pass2(A, i, dF);
     A.rho_acc[i] = 0.0;
     A.f_acc[i] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+}
+
+// The neighbour's share -g d of a pair's force (from the negated radial factors: no negation), and
+// the image shift s = d_raw - d of the pair for the virial.
+template <int KIND, typename W>
+__device__ __forceinline__ void pair_share(const Atoms &A, const Pot &P, const Box &B, const double4_32a &pi,
+                                           const double4_32a &pj, const double2 &e, double &ngx, double &ngy,
+                                           double &ngz, double &sx, double &sy, double &sz) {
+    sx = sy = sz = 0.0;
+    if constexpr (KIND == MD_POT_TABLES) {
+        if (A.qfb) {   // from FP32 pieces
+            long long qx, qy, qz;
+            const df::F2 dx = sep_df64(P, sep_fixed<W>(pj.x, pi.x, B.Lq[0], qx)),
+                         dy = sep_df64(P, sep_fixed<W>(pj.y, pi.y, B.Lq[1], qy)),
+                         dz = sep_df64(P, sep_fixed<W>(pj.z, pi.z, B.Lq[2], qz));
+            const long long f = __double_as_longlong(e.x), p = __double_as_longlong(e.y);
+            const float4 c = make_float4(__int_as_float((int)f), __int_as_float((int)(f >> 32)), __int_as_float((int)p),
+                                         __int_as_float((int)(p >> 32)));
+            const df::F2 g = radial_q(c, fprime_q(pi.w), fprime_q(pj.w));
+            ngx = to64(mul_raw(g, dx));
+            ngy = to64(mul_raw(g, dy));
+            ngz = to64(mul_raw(g, dz));
+            if (W::value) {
+                sx = qx > 0 ? B.L[0] : (qx < 0 ? -B.L[0] : 0.0);
+                sy = qy > 0 ? B.L[1] : (qy < 0 ? -B.L[1] : 0.0);
+                sz = qz > 0 ? B.L[2] : (qz < 0 ? -B.L[2] : 0.0);
+            }
+            return;
+        }
+    }
+    const double dx = sep64s<W>(pj.x - pi.x, B.L[0], sx);
+    const double dy = sep64s<W>(pj.y - pi.y, B.L[1], sy);
+    const double dz = sep64s<W>(pj.z - pi.z, B.L[2], sz);
+    const double ngr = fma(pi.w + pj.w, e.y, e.x);
+    ngx = ngr * dx;
+    ngy = ngr * dy;
+    ngz = ngr * dz;
 }
 
 template <int T, int KIND, bool ENERGY>
@@ -874,13 +1173,8 @@ __device__ __forceinline__ void force64_pairs_item(const Atoms &A, const Pot &P,
                 if ((__double_as_longlong(e.x) | __double_as_longlong(e.y)) == 0) continue;
                 const int j = ld_phase(row.ptr(k));
                 const double4_32a pj = ld_phase(A.p2d + j);
-                double sx, sy, sz;
-                const double dx = sep64s<W>(pj.x - pi.x, B.L[0], sx);
-                const double dy = sep64s<W>(pj.y - pi.y, B.L[1], sy);
-                const double dz = sep64s<W>(pj.z - pi.z, B.L[2], sz);
-                // -g d, the neighbour's share, from the negated radial factors (no negation)
-                const double ngr = fma(pi.w + pj.w, e.y, e.x);
-                const double ngx = ngr * dx, ngy = ngr * dy, ngz = ngr * dz;
+                double ngx, ngy, ngz, sx, sy, sz;
+                pair_share<KIND, W>(A, P, B, pi, pj, e, ngx, ngy, ngz, sx, sy, sz);
                 fx -= ngx;
                 fy -= ngy;
                 fz -= ngz;
@@ -995,6 +1289,7 @@ __device__ __forceinline__ void density64_pairs_flat(const Atoms &A, const Pot &
     for (int q = 0; q < 2 * AW; q++) S[q * 32 + lane] = 0.0;
     auto walk = [&](auto wrapt) {
         using W = decltype(wrapt);
+        const double4_32a *const from = A.qfb ? A.posq : A.posd;
         for (int seg = 0; seg < 2; seg++) {
             const FlatRows<AW> R = flat_rows<AW>(c_in, c_up, seg);
             int cur = -1, i = 0;
@@ -1013,7 +1308,7 @@ __device__ __forceinline__ void density64_pairs_flat(const Atoms &A, const Pot &
                     cur = a;
                     rho = ep = 0.0;
                     i = i0 + a;
-                    pi = ld_phase(A.posd + i);
+                    pi = ld_phase(from + i);
                     row = nbr_row(A, i);
                     drow = dcache_row(A, i);
                 }
@@ -1036,7 +1331,28 @@ __device__ __forceinline__ void density64_pairs_flat(const Atoms &A, const Pot &
                         continue;
                     }
                 }
-                const double4_32a pj = ld_phase(A.posd + j);
+                const double4_32a pj = ld_phase(from + j);
+                if constexpr (KIND == MD_POT_TABLES) {
+                    if (A.qfb) {   // the pair terms from FP32 pieces
+                        const unsigned long long r2 = r2_fixed<W>(pj, pi, boxes[ph::replica_of(A, i)]);
+                        if (r2 >= P.rc2q) {
+                            *dc = make_double2(0.0, 0.0);
+                            continue;
+                        }
+                        PairQ o;
+                        pair_terms_q(P, r2, energy, o, A.flags);
+                        const double phi = to64(o.phi);
+                        rho += phi;
+                        atomicAdd(A.rho_acc + j, phi);
+                        if (energy) {
+                            const double hV = half64(to64(o.V));
+                            ep += hV;
+                            atomicAdd(A.e_acc + j, hV);
+                        }
+                        *reinterpret_cast<float4 *>(dc) = cache_q(o, true);
+                        continue;
+                    }
+                }
                 double dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
                 if (W::value) {
                     const Box &B = boxes[ph::replica_of(A, i)];
@@ -1142,16 +1458,8 @@ __device__ __forceinline__ void force64_pairs_flat(const Atoms &A, const Pot &P,
                     pi = ld_phase(A.p2d + i);
                 }
                 const double4_32a pj = ld_phase(A.p2d + j);
-                double dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z, sx = 0.0, sy = 0.0, sz = 0.0;
-                if (W::value) {
-                    const Box &B = boxes[ph::replica_of(A, i)];
-                    dx = mi64s(dx, B.L[0], sx);
-                    dy = mi64s(dy, B.L[1], sy);
-                    dz = mi64s(dz, B.L[2], sz);
-                }
-                // -g d, the neighbour's share, from the negated radial factors (no negation)
-                const double ngr = fma(pi.w + pj.w, d.y, d.x);
-                const double ngx = ngr * dx, ngy = ngr * dy, ngz = ngr * dz;
+                double ngx, ngy, ngz, sx, sy, sz;
+                pair_share<KIND, W>(A, P, boxes[ph::replica_of(A, i)], pi, pj, d, ngx, ngy, ngz, sx, sy, sz);
                 fx -= ngx;
                 fy -= ngy;
                 fz -= ngz;
@@ -1259,7 +1567,7 @@ __device__ __forceinline__ void pairs_partials64(const Atoms &A, int i, double f
                                                  const double4_32a &v, double (&part)[kPartials]) {
     if (!ENERGY) return;
     // the virial's per-atom part x_a F_b (virial_shift), x as the force pass took it
-    const double4_32a x = A.p2d[i];
+    const double4_32a x = A.posd[i];
     part[2] = fma(x.x, fx, part[2]);
     part[3] = fma(x.y, fy, part[3]);
     part[4] = fma(x.z, fz, part[4]);
@@ -1328,6 +1636,7 @@ __device__ __forceinline__ df::F2 sep_df(float xjh, float xih, float xjl, float 
     return df::make(dh, dl);
 }
 
+// r^2 of separations given as double-floats, not necessarily normalised.
 __device__ __forceinline__ df::F2 r2_df(df::F2 dx, df::F2 dy, df::F2 dz) {
     auto sq = [](df::F2 d) {   // d unnormalised: its low part may exceed ulp(d.h), so keep d.l^2
         df::F2 p = df::two_prod(d.h, d.h);

@@ -57,6 +57,14 @@ __device__ __forceinline__ void store_dfpos(const Atoms &A, int i, const double4
                                             eam::f32_rn(z - eam::f64_of_f32(zh)), 0.f);
 }
 
+// Fixed-point copy of an FP64 image coordinate q (Atoms::posq).  A coordinate that is not finite has
+// none: it is reported here, as it would otherwise be by the forces it leads to.
+__device__ __forceinline__ void store_fixed(const Atoms &A, int i, const double4_32a &q) {
+    if (!(eam::finite64(q.x) && eam::finite64(q.y) && eam::finite64(q.z))) atomicOr(&A.flags->error, FLAG_NONFINITE);
+    A.posq[i] = make_double4_32a(__longlong_as_double(eam::fix64(q.x, A.qfb)), __longlong_as_double(eam::fix64(q.y, A.qfb)),
+                                 __longlong_as_double(eam::fix64(q.z, A.qfb)), 0.0);
+}
+
 // The whole box edges to take off per axis, floor(r / L), as three signed 10-bit fields (0: none, as
 // for most atoms); kImageFar where one does not fit.
 constexpr int kImageFar = (int)0x80000000;
@@ -129,6 +137,7 @@ __device__ __forceinline__ void place(const Atoms &A, const Box *boxes, int i, c
             const double4_32a q = build_image64(p, r, B);
             A.posd[i] = q;
             if (A.posx) store_dfpos(A, i, q, B);
+            if (A.posq) store_fixed(A, i, q);
         }
         return;
     }
@@ -152,6 +161,7 @@ __device__ __forceinline__ void place(const Atoms &A, const Box *boxes, int i, c
     if (A.posd) {
         A.posd[i] = q;
         if (A.posx) store_dfpos(A, i, q, boxes[replica_of(A, i)]);
+        if (A.posq) store_fixed(A, i, q);
     }
 }
 
@@ -375,6 +385,7 @@ __device__ __forceinline__ void copyback_atom(const Atoms &A, const Box *boxes, 
     if (A.posd) {
         A.posd[k] = q;
         if (A.posx) store_dfpos(A, k, q, B);
+        if (A.posq) store_fixed(A, k, q);
     }
 }
 

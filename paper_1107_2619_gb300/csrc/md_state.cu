@@ -24,6 +24,7 @@ __global__ void k_wrap(Atoms A) {
         const double4_32a q = ph::build_image64(A.pos[i], A.ref[i], B);
         A.posd[i] = q;
         if (A.posx) ph::store_dfpos(A, i, q, B);
+        if (A.posq) ph::store_fixed(A, i, q);
     }
 }
 

@@ -114,7 +114,7 @@ __device__ __forceinline__ bool grid_sync(GridBarrier *b, unsigned nblocks, unsi
 }
 
 // Box matrix times the strain matrix diag(1, 1, s) (§2.2), every replica.
-__device__ __forceinline__ void strain_boxes(Box *boxes, int n_rep, double s) {
+__device__ __forceinline__ void strain_boxes(Box *boxes, int n_rep, double s, int qfb) {
     for (int r = 0; r < n_rep; r++) {
         Box b = boxes[r];
         b.L[2] = __dmul_rn(b.L[2], s);
@@ -123,6 +123,7 @@ __device__ __forceinline__ void strain_boxes(Box *boxes, int n_rep, double s) {
         b.invLf[2] = (float)b.invL[2];
         b.Lh[2] = (float)b.L[2];
         b.Ll[2] = (float)(b.L[2] - (double)b.Lh[2]);
+        b.Lq[2] = eam::fix64(b.L[2], qfb);
         boxes[r] = b;
     }
 }
@@ -347,7 +348,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
         if (stamps && lead) stamps[0] = globaltimer();
         // first half kick + drift of the first step
         if (strain) {
-            if (lead) strain_boxes(boxes, A.n_rep, sp.strain_scale);
+            if (lead) strain_boxes(boxes, A.n_rep, sp.strain_scale, A.qfb);
             MD_SYNC();
         }
         if (lead && sp.rebuild_every > 0 && (step + 1) % sp.rebuild_every == 0) A.flags->need_rebuild = 1;
@@ -586,7 +587,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
             if (!grid_sync(bar, nb, sp.spin_limit, A.flags, [&] {
                     thermo_update(sp, A.n_rep, threadIdx.x, NT, true, !last);
                     if (!last && threadIdx.x == 0) {
-                        if (strain) strain_boxes(boxes, A.n_rep, sp.strain_scale);
+                        if (strain) strain_boxes(boxes, A.n_rep, sp.strain_scale, A.qfb);
                         if (sp.rebuild_every > 0 && (A.flags->step + s + 2) % sp.rebuild_every == 0)
                             A.flags->need_rebuild = 1;
                     }
@@ -613,7 +614,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
             }
         } else if (!last && strain) {
             if (lead) {
-                strain_boxes(boxes, A.n_rep, sp.strain_scale);
+                strain_boxes(boxes, A.n_rep, sp.strain_scale, A.qfb);
                 if (sp.rebuild_every > 0 && (step + s + 2) % sp.rebuild_every == 0) A.flags->need_rebuild = 1;
             }
             MD_SYNC();
@@ -744,9 +745,9 @@ cudaError_t launch_kind(const Atoms &A, const Cells &C, const Pot &P, const Step
         if (P.kind == MD_POT_KNOTS)
             return P.ns == 1 ? launch_t<PREC, T, MD_POT_KNOTS, false>(A, C, P, sp, bar, stamps, grid_out, s)
                              : launch_t<PREC, T, MD_POT_KNOTS, true>(A, C, P, sp, bar, stamps, grid_out, s);
-        if (P.ns == 1) {
-            if (smem_table_bytes(P.kind, P.ns, PREC, P.nk) > 0) {
-                if constexpr (PREC == MD_PREC_MIXED && T <= 8) {
+        if constexpr (PREC == MD_PREC_MIXED) {   // the table of pair (0, 0) in shared memory where it fits
+            if (P.ns == 1 && smem_table_bytes(P.kind, P.ns, PREC, P.nk) > 0) {
+                if constexpr (T <= 8) {
                     if (C.tile == kWalkStaged)
                         return launch_t<PREC, T, MD_POT_TABLES, false, 1024, true, kWalkStaged>(A, C, P, sp, bar, stamps,
                                                                                                grid_out, s);
@@ -760,12 +761,12 @@ cudaError_t launch_kind(const Atoms &A, const Cells &C, const Pot &P, const Step
                 return launch_t<PREC, T, MD_POT_TABLES, false, MD_SMT_THREADS, true>(A, C, P, sp, bar, stamps, grid_out,
                                                                                     s);
             }
-            return launch_t<PREC, T, MD_POT_TABLES, false>(A, C, P, sp, bar, stamps, grid_out, s);
+            // several species: pair (0, 0) is the host species'
+            if (MD_SMEM_TABLE && P.ns > 1 && (size_t)P.nk * 32 <= kSmemTableMax)
+                return launch_t<PREC, T, MD_POT_TABLES, true, MD_SMT_THREADS, true>(A, C, P, sp, bar, stamps, grid_out, s);
         }
-        // several species: the table of pair (0, 0), the host species, in shared memory
-        if (MD_SMEM_TABLE && PREC == MD_PREC_MIXED && (size_t)P.nk * 32 <= kSmemTableMax)
-            return launch_t<PREC, T, MD_POT_TABLES, true, MD_SMT_THREADS, true>(A, C, P, sp, bar, stamps, grid_out, s);
-        return launch_t<PREC, T, MD_POT_TABLES, true>(A, C, P, sp, bar, stamps, grid_out, s);
+        return P.ns == 1 ? launch_t<PREC, T, MD_POT_TABLES, false>(A, C, P, sp, bar, stamps, grid_out, s)
+                         : launch_t<PREC, T, MD_POT_TABLES, true>(A, C, P, sp, bar, stamps, grid_out, s);
     }
 }
 
