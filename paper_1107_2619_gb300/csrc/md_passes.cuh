@@ -513,6 +513,18 @@ __device__ __forceinline__ unsigned long long r2_fixed(const double4_32a &xj, co
            sq(sep_fixed<WRAP>(xj.z, xi.z, B.Lq[2], s));
 }
 
+// Two float4 behind each other, 32-byte aligned, in one load.
+__device__ __forceinline__ void two_of(const double4_32a &d, float4 &a, float4 &b) {
+    unpack2(d.x, a.x, a.y); unpack2(d.y, a.z, a.w); unpack2(d.z, b.x, b.y); unpack2(d.w, b.z, b.w);
+}
+__device__ __forceinline__ void load2(const float4 *p, float4 &a, float4 &b) {
+    two_of(*reinterpret_cast<const double4_32a *>(p), a, b);
+}
+__device__ __forceinline__ void load_row_q(const Pot &P, int k, float4 &p0, float4 &p1, float4 &v0, float4 &v1) {
+    load2(P.TQ + 4 * (size_t)k, p0, p1);
+    load2(P.TQ + 4 * (size_t)k + 2, v0, v1);
+}
+
 // The terms of a pair at r2 = r^2 (r2_fixed), inside r_cut.
 __device__ __forceinline__ void pair_terms_q(const Pot &P, unsigned long long r2, bool energy, PairQ &o, Flags *flags) {
     const df::F2 x2 = df::make(__fmul_rn(__uint2float_rn((unsigned)(r2 >> 40)), P.q2h),
@@ -532,8 +544,9 @@ __device__ __forceinline__ void pair_terms_q(const Pot &P, unsigned long long r2
     const float x = __fmaf_rn(r.h, P.idr_h, -P.x0_h), last = (float)(P.nk - 1);
     float kf = __fsub_rn(__fadd_rn(__fsub_rn(x, 0.5f), 12582912.f), 12582912.f);
     kf = fminf(fmaxf(kf, 0.f), last);   // (a NaN x: row 0, and t carries it on)
-    const float4 *row = P.TQ + 4 * (size_t)(int)kf;
-    float4 p0 = __ldg(row), p1 = __ldg(row + 1), v0 = __ldg(row + 2), v1 = __ldg(row + 3);
+    // (two 32-byte loads: rows read at random cost the L1 a look-up per lane and load)
+    float4 p0, p1, v0, v1;
+    load_row_q(P, (int)kf, p0, p1, v0, v1);
     const bool below = x < 0.f;   // linear continuation below the first knot, any distance from it
     if (below) atomicAdd(&flags->range_violations, 1ull);
     // t = (r^2 - rho^2) / (r + rho) / h
@@ -563,11 +576,7 @@ __device__ __forceinline__ void pair_terms_q(const Pot &P, unsigned long long r2
     const float move = t.h < 0.f ? -1.f : (t.h > 1.f || (t.h == 1.f && t.l >= 0.f) ? 1.f : 0.f);
     if (move != 0.f && !below && kf + move >= 0.f && kf + move <= last) {
         kf += move;
-        row = P.TQ + 4 * (size_t)(int)kf;
-        p0 = __ldg(row);
-        p1 = __ldg(row + 1);
-        v0 = __ldg(row + 2);
-        v1 = __ldg(row + 3);
+        load_row_q(P, (int)kf, p0, p1, v0, v1);
         t = coord(kf);
     }
     const float on = below ? 0.f : 1.f;
@@ -1127,18 +1136,16 @@ __device__ __forceinline__ void pair_share(const Atoms &A, const Pot &P, const B
             const df::F2 dx = sep_df64(P, sep_fixed<W>(pj.x, pi.x, B.Lq[0], qx)),
                          dy = sep_df64(P, sep_fixed<W>(pj.y, pi.y, B.Lq[1], qy)),
                          dz = sep_df64(P, sep_fixed<W>(pj.z, pi.z, B.Lq[2], qz));
-            const long long f = __double_as_longlong(e.x), p = __double_as_longlong(e.y);
-            const float4 c = make_float4(__int_as_float((int)f), __int_as_float((int)(f >> 32)), __int_as_float((int)p),
-                                         __int_as_float((int)(p >> 32)));
+            float4 c;
+            unpack2(e.x, c.x, c.y);
+            unpack2(e.y, c.z, c.w);
             const df::F2 g = radial_q(c, fprime_q(pi.w), fprime_q(pj.w));
             ngx = to64(mul_raw(g, dx));
             ngy = to64(mul_raw(g, dy));
             ngz = to64(mul_raw(g, dz));
-            if (W::value) {
-                sx = qx > 0 ? B.L[0] : (qx < 0 ? -B.L[0] : 0.0);
-                sy = qy > 0 ? B.L[1] : (qy < 0 ? -B.L[1] : 0.0);
-                sz = qz > 0 ? B.L[2] : (qz < 0 ? -B.L[2] : 0.0);
-            }
+            sx = qx > 0 ? B.L[0] : (qx < 0 ? -B.L[0] : 0.0);
+            sy = qy > 0 ? B.L[1] : (qy < 0 ? -B.L[1] : 0.0);
+            sz = qz > 0 ? B.L[2] : (qz < 0 ? -B.L[2] : 0.0);
             return;
         }
     }
@@ -1248,7 +1255,7 @@ __device__ __forceinline__ FlatRows<AW> flat_rows(int c_in, int c_up, int seg) {
     return R;
 }
 
-__host__ __device__ constexpr int kPairSlots(int aw) { return 3 * aw * 32; }
+__host__ __device__ constexpr int kPairSlots(int aw) { return 3 * aw * 32 + 4 * aw; }   // and the atoms' records
 // The fewest lanes per atom that take the flattened walk (at most 32 / kFlatLanes atoms a warp).
 constexpr int kFlatLanes = 4;
 
@@ -1289,7 +1296,6 @@ __device__ __forceinline__ void density64_pairs_flat(const Atoms &A, const Pot &
     for (int q = 0; q < 2 * AW; q++) S[q * 32 + lane] = 0.0;
     auto walk = [&](auto wrapt) {
         using W = decltype(wrapt);
-        const double4_32a *const from = A.qfb ? A.posq : A.posd;
         for (int seg = 0; seg < 2; seg++) {
             const FlatRows<AW> R = flat_rows<AW>(c_in, c_up, seg);
             int cur = -1, i = 0;
@@ -1308,7 +1314,7 @@ __device__ __forceinline__ void density64_pairs_flat(const Atoms &A, const Pot &
                     cur = a;
                     rho = ep = 0.0;
                     i = i0 + a;
-                    pi = ld_phase(from + i);
+                    pi = ld_phase(A.posd + i);
                     row = nbr_row(A, i);
                     drow = dcache_row(A, i);
                 }
@@ -1331,28 +1337,7 @@ __device__ __forceinline__ void density64_pairs_flat(const Atoms &A, const Pot &
                         continue;
                     }
                 }
-                const double4_32a pj = ld_phase(from + j);
-                if constexpr (KIND == MD_POT_TABLES) {
-                    if (A.qfb) {   // the pair terms from FP32 pieces
-                        const unsigned long long r2 = r2_fixed<W>(pj, pi, boxes[ph::replica_of(A, i)]);
-                        if (r2 >= P.rc2q) {
-                            *dc = make_double2(0.0, 0.0);
-                            continue;
-                        }
-                        PairQ o;
-                        pair_terms_q(P, r2, energy, o, A.flags);
-                        const double phi = to64(o.phi);
-                        rho += phi;
-                        atomicAdd(A.rho_acc + j, phi);
-                        if (energy) {
-                            const double hV = half64(to64(o.V));
-                            ep += hV;
-                            atomicAdd(A.e_acc + j, hV);
-                        }
-                        *reinterpret_cast<float4 *>(dc) = cache_q(o, true);
-                        continue;
-                    }
-                }
+                const double4_32a pj = ld_phase(A.posd + j);
                 double dx = pj.x - pi.x, dy = pj.y - pi.y, dz = pj.z - pi.z;
                 if (W::value) {
                     const Box &B = boxes[ph::replica_of(A, i)];
@@ -1488,17 +1473,218 @@ __device__ __forceinline__ void force64_pairs_flat(const Atoms &A, const Pot &P,
     if (me < A.n && (lane & (T - 1)) == 0) A.force[me] = make_double4_32a(fx, fy, fz, 0.0);
 }
 
+// The flattened walks with the pair terms from FP32 pieces.  What is left of a pair is short enough
+// that the chain of loads before it (list entry, then the neighbour's record) bounds the pass, so
+// the chain runs ahead: while an entry is worked on, the neighbour's record of the next (and its
+// cached factors in the force pass) and the list entry after that are on their way.  The records of
+// the warp's own atoms wait in shared memory (after the slots of S).  fcc Cu 500,000 atoms, us per
+// step, before -> after: density 842 -> 800, force 926 -> 840 (of that, rows in two 32-byte loads
+// instead of four of 16 bytes: density 828 -> 800).  What bounds them now: density the L1's data pipe
+// (88 %: scattered rows and records), force the FP64 pipe (81 %: to64 and the sums) and the FP64
+// atomics (three a pair).  Double-float lane sums in place of the FP64 ones gained nothing.
+template <int AW>
+struct FlatEntry {
+    int a, k, j;
+    __device__ __forceinline__ void fetch(const Atoms &A, const FlatRows<AW> &R, int i0, int e) {
+        a = R.atom(e, k);
+        j = ld_phase(nbr_row(A, i0 + a).ptr(k));
+    }
+};
+template <int AW>
+__device__ __forceinline__ void stage_records(const Atoms &A, const double4_32a *from, int i0, int lane, double *rec) {
+    const double *src = reinterpret_cast<const double *>(from + i0);
+    for (int q = lane; q < 4 * AW; q += 32)
+        if (i0 + q / 4 < A.n) rec[q] = ld_phase(src + q);
+    __syncwarp();
+}
+__device__ __forceinline__ double4_32a record(const double *rec, int a) {
+    const double2 x = *reinterpret_cast<const double2 *>(rec + 4 * a), y = *reinterpret_cast<const double2 *>(rec + 4 * a + 2);
+    return make_double4_32a(x.x, x.y, y.x, y.y);
+}
+
+template <int T>
+__device__ __forceinline__ void density64_pairs_flat_q(const Atoms &A, const Pot &P, const Box *boxes, long long g,
+                                                       bool energy, double *S) {
+    constexpr int AW = 32 / T;
+    const int lane = (int)(g & 31);
+    const int i0 = (int)(g >> 5) * AW;
+    const int me = i0 + lane / T;
+    const bool wrap = needs_image(A, me, me < A.n);
+    int c_in = 0, c_up = 0;
+    if (lane < AW && i0 + lane < A.n) {
+        c_in = ld_phase(A.cin + i0 + lane);
+        c_up = ld_phase(A.cup + i0 + lane);
+    }
+#pragma unroll
+    for (int q = 0; q < 2 * AW; q++) S[q * 32 + lane] = 0.0;
+    double *const rec = S + 3 * AW * 32;
+    stage_records<AW>(A, A.posq, i0, lane, rec);
+    auto walk = [&](auto wrapt) {
+        using W = decltype(wrapt);
+        for (int seg = 0; seg < 2; seg++) {
+            const FlatRows<AW> R = flat_rows<AW>(c_in, c_up, seg);
+            const int end = R.off[AW];
+            int cur = -1;
+            double rho = 0.0, ep = 0.0;
+            FlatEntry<AW> n0{0, 0, 0}, n1{0, 0, 0};
+            double4_32a p0 = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+            if (lane < end) n0.fetch(A, R, i0, lane);
+            if (lane + 32 < end) n1.fetch(A, R, i0, lane + 32);
+            if (lane < end) p0 = ld_phase(A.posq + n0.j);
+            for (int e = lane; e < end; e += 32) {
+                const FlatEntry<AW> x = n0;
+                const double4_32a pj = p0;
+                n0 = n1;
+                if (e + 32 < end) p0 = ld_phase(A.posq + n1.j);
+                if (e + 64 < end) n1.fetch(A, R, i0, e + 64);
+                if (x.a != cur) {   // the next atom of this lane: flush the sums
+                    if (cur >= 0) {
+                        put_slot(S + cur * 32 + lane, rho, seg);
+                        if (energy) put_slot(S + (AW + cur) * 32 + lane, ep, seg);
+                    }
+                    cur = x.a;
+                    rho = ep = 0.0;
+                }
+                const int i = i0 + x.a;
+                float4 *dc = reinterpret_cast<float4 *>(dcache_row(A, i).ptr(x.k));
+                const unsigned long long r2 = r2_fixed<W>(pj, record(rec, x.a), boxes[W::value ? ph::replica_of(A, i) : 0]);
+                if (r2 >= P.rc2q) {
+                    *dc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    continue;
+                }
+                PairQ o;
+                pair_terms_q(P, r2, energy, o, A.flags);
+                const double phi = to64(o.phi);
+                rho += phi;
+                atomicAdd(A.rho_acc + x.j, phi);
+                if (energy) {   // each atom of the pair gets half its pair energy
+                    const double hV = half64(to64(o.V));
+                    ep += hV;
+                    atomicAdd(A.e_acc + x.j, hV);
+                }
+                *dc = cache_q(o, true);
+            }
+            if (cur >= 0) {
+                put_slot(S + cur * 32 + lane, rho, seg);
+                if (energy) put_slot(S + (AW + cur) * 32 + lane, ep, seg);
+            }
+        }
+    };
+    if (wrap) walk(std::true_type{});
+    else walk(std::false_type{});
+    __syncwarp();
+    const double rho = flat_sum<T>(S, 0);
+    const double ep = energy ? flat_sum<T>(S, 1) : 0.0;
+    __syncwarp();   // S is free for the next item of this warp
+    if (me < A.n && (lane & (T - 1)) == 0) {
+        A.rho[me] = rho;
+        if (energy) atomicAdd(A.e_acc + me, ep);
+    }
+}
+
+template <int T, bool ENERGY>
+__device__ __forceinline__ void force64_pairs_flat_q(const Atoms &A, const Pot &P, const Box *boxes, long long g,
+                                                     double (&part)[kPartials], double *S) {
+    constexpr int AW = 32 / T;
+    const int lane = (int)(g & 31);
+    const int i0 = (int)(g >> 5) * AW;
+    const int me = i0 + lane / T;
+    const bool wrap = needs_image(A, me, me < A.n);
+    int c_in = 0, c_up = 0;
+    if (lane < AW && i0 + lane < A.n) {
+        c_in = ld_phase(A.cin + i0 + lane);
+        c_up = ld_phase(A.cup + i0 + lane);
+    }
+#pragma unroll
+    for (int q = 0; q < 3 * AW; q++) S[q * 32 + lane] = 0.0;
+    double *const rec = S + 3 * AW * 32;
+    stage_records<AW>(A, A.p2d, i0, lane, rec);
+    double wxx = 0.0, wyy = 0.0, wzz = 0.0, wyz = 0.0, wxz = 0.0, wxy = 0.0;
+    auto walk = [&](auto wrapt) {
+        using W = decltype(wrapt);
+        for (int seg = 0; seg < 2; seg++) {
+            const FlatRows<AW> R = flat_rows<AW>(c_in, c_up, seg);
+            const int end = R.off[AW];
+            int cur = -1;
+            double fx = 0.0, fy = 0.0, fz = 0.0;
+            FlatEntry<AW> n0{0, 0, 0}, n1{0, 0, 0};
+            double4_32a p0 = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+            double2 d0 = make_double2(0.0, 0.0);
+            if (lane < end) n0.fetch(A, R, i0, lane);
+            if (lane + 32 < end) n1.fetch(A, R, i0, lane + 32);
+            if (lane < end) {
+                p0 = ld_phase(A.p2d + n0.j);
+                d0 = ld_phase(dcache_row(A, i0 + n0.a).ptr(n0.k));
+            }
+            for (int e = lane; e < end; e += 32) {
+                const FlatEntry<AW> x = n0;
+                const double4_32a pj = p0;
+                const double2 d = d0;
+                n0 = n1;
+                if (e + 32 < end) {
+                    p0 = ld_phase(A.p2d + n1.j);
+                    d0 = ld_phase(dcache_row(A, i0 + n1.a).ptr(n1.k));
+                }
+                if (e + 64 < end) n1.fetch(A, R, i0, e + 64);
+                // beyond r_cut: nothing to add (the skin segment mostly ends here)
+                if ((__double_as_longlong(d.x) | __double_as_longlong(d.y)) == 0) continue;
+                if (x.a != cur) {
+                    if (cur >= 0) {
+                        put_slot(S + cur * 32 + lane, fx, seg);
+                        put_slot(S + (AW + cur) * 32 + lane, fy, seg);
+                        put_slot(S + (2 * AW + cur) * 32 + lane, fz, seg);
+                    }
+                    cur = x.a;
+                    fx = fy = fz = 0.0;
+                }
+                double ngx, ngy, ngz, sx, sy, sz;
+                pair_share<MD_POT_TABLES, W>(A, P, boxes[W::value ? ph::replica_of(A, i0 + x.a) : 0], record(rec, x.a), pj, d,
+                                             ngx, ngy, ngz, sx, sy, sz);
+                fx -= ngx;
+                fy -= ngy;
+                fz -= ngz;
+                if (ENERGY && W::value) virial_shift(sx, sy, sz, ngx, ngy, ngz, wxx, wyy, wzz, wyz, wxz, wxy);
+                double *acc = reinterpret_cast<double *>(A.f_acc + x.j);
+                atomicAdd(acc, ngx);
+                atomicAdd(acc + 1, ngy);
+                atomicAdd(acc + 2, ngz);
+            }
+            if (cur >= 0) {
+                put_slot(S + cur * 32 + lane, fx, seg);
+                put_slot(S + (AW + cur) * 32 + lane, fy, seg);
+                put_slot(S + (2 * AW + cur) * 32 + lane, fz, seg);
+            }
+        }
+    };
+    if (wrap) walk(std::true_type{});
+    else walk(std::false_type{});
+    if (ENERGY) {
+        part[2] += wxx; part[3] += wyy; part[4] += wzz;
+        part[5] += wyz; part[6] += wxz; part[7] += wxy;
+    }
+    __syncwarp();
+    const double fx = flat_sum<T>(S, 0), fy = flat_sum<T>(S, 1), fz = flat_sum<T>(S, 2);
+    __syncwarp();
+    if (me < A.n && (lane & (T - 1)) == 0) A.force[me] = make_double4_32a(fx, fy, fz, 0.0);
+}
+
 // The pair walk's passes: the flattened rows for T >= kFlatLanes lanes per atom (S: this warp's
 // kPairSlots(32 / T) doubles of shared memory), the per-atom rows otherwise.
 template <int T, int KIND>
 __device__ __forceinline__ void density64_pairs(const Atoms &A, const Pot &P, const Box *boxes, long long g,
                                                 bool energy, double *S) {
+    if constexpr (T >= kFlatLanes && KIND == MD_POT_TABLES) {
+        if (A.qfb) return density64_pairs_flat_q<T>(A, P, boxes, g, energy, S);
+    }
     if constexpr (T >= kFlatLanes) density64_pairs_flat<T, KIND>(A, P, boxes, g, energy, S);
     else density64_pairs_item<T, KIND>(A, P, boxes, g, energy);
 }
 template <int T, int KIND, bool ENERGY>
 __device__ __forceinline__ void force64_pairs(const Atoms &A, const Pot &P, const Box *boxes, long long g,
                                               double (&part)[kPartials], double *S) {
+    if constexpr (T >= kFlatLanes && KIND == MD_POT_TABLES) {
+        if (A.qfb) return force64_pairs_flat_q<T, ENERGY>(A, P, boxes, g, part, S);
+    }
     if constexpr (T >= kFlatLanes) force64_pairs_flat<T, KIND, ENERGY>(A, P, boxes, g, part, S);
     else force64_pairs_item<T, KIND, ENERGY>(A, P, boxes, g, part);
 }

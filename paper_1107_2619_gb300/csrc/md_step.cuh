@@ -182,8 +182,8 @@ __device__ __forceinline__ void thermo_update(const StepParams &sp, int n_rep, l
 #endif
 // Blocks of 128 threads per SM the FP64 step kernel is built for: 4 (128 registers) measured 2-3 %
 // faster than 8 (64 registers, with spills) and 6 on fcc Cu 500k with the full list; the pair
-// walk over the half list is built for 5 (96 registers): 2.80 -> 2.74 ms per step against 4, 2.86
-// at 6 (the full list at 5: 4.79 -> 4.89).
+// walk over the half list is built for 5 (96 registers): 1.94 / 1.92 / 1.97 ms per step at 4 / 5 / 6
+// and 4 lanes per atom, 1.96 / 1.88 / 1.87 at 8 (the full list was 2 % slower at 5 than at 4).
 #ifndef MD_STEP_MIN_BLOCKS_FP64
 #define MD_STEP_MIN_BLOCKS_FP64 4
 #endif
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
     __shared__ uint16_t cells_q[WALK == kWalkCells ? NT / 32 : 1][kCellsQueue];
     // the FP64 pair walk's per-warp sums (flattened rows, T >= kFlatLanes)
     constexpr int kPairSlotsW = WALK == kWalkPairs && T >= ps::kFlatLanes ? ps::kPairSlots(32 / T) : 0;
-    __shared__ double pair_sums[kPairSlotsW > 0 ? NT / 32 * kPairSlotsW : 1];
+    __shared__ __align__(16) double pair_sums[kPairSlotsW > 0 ? NT / 32 * kPairSlotsW : 1];
     double *const psum = pair_sums + (threadIdx.x >> 5) * kPairSlotsW;
     extern __shared__ float4 sm_table_f4[];   // [SMT table][stage]
     // The group walks' stage needs the room: their shared copy holds only the rows of the pass
