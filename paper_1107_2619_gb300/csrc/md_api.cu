@@ -963,23 +963,28 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
                 P.idr_l = idr.l;
                 P.x0_h = x0.h;
                 P.x0_l = x0.l;
-                TQ.resize(4 * (size_t)nk);
-                for (int k = 0; k < nk; k++) {
-                    // the row's cubics about rho_k, s rows beyond its knot
+                TQ.resize(4 * (size_t)(nk + 1));
+                P.t0 = (float)(((long double)rmf - pot->r_min) * P.inv_dr);
+                for (int row = 0; row <= nk; row++) {
+                    // the row's cubics about rho_k, s rows beyond its knot (row nk: the lines at the first)
+                    const int k = row < nk ? row : 0;
                     const long double s = ((long double)std::fma((float)k, hrf, rmf) - pot->r_min) * P.inv_dr - k;
                     auto about = [s](const double4_32a &c) {
                         return make_double4_32a((double)(c.x + s * (c.y + s * (c.z + s * c.w))),
                                                 (double)(c.y + s * (2 * c.z + 3 * s * c.w)), (double)(c.z + 3 * s * c.w), c.w);
                     };
-                    const double4_32a v = about(VP64[2 * k]), p = about(VP64[2 * k + 1]);
+                    double4_32a v = VP64[2 * k], p = VP64[2 * k + 1];
+                    if (row == nk) v.z = v.w = p.z = p.w = 0.0;
+                    v = about(v);
+                    p = about(p);
                     auto two = [](double x, double y) {
                         const df::F2 a = df::from_double(x), b = df::from_double(y);
                         return make_float4(a.h, a.l, b.h, b.l);
                     };
-                    TQ[4 * k] = two(p.x, p.y);
-                    TQ[4 * k + 1] = two(p.z, p.w);
-                    TQ[4 * k + 2] = two(v.y, v.z);
-                    TQ[4 * k + 3] = two(v.w, v.x);
+                    TQ[4 * (size_t)row] = two(p.x, p.y);
+                    TQ[4 * (size_t)row + 1] = two(p.z, p.w);
+                    TQ[4 * (size_t)row + 2] = two(v.y, v.z);
+                    TQ[4 * (size_t)row + 3] = two(v.w, v.x);
                 }
                 float4 *dTQ;
                 chk(dalloc(ctx, &A.posq, n));

@@ -97,9 +97,10 @@ struct Pot {
     const float4 *TVx;
     // one species, FP64 path: the cubics of V and phi of an interval about rho_k (ps::pair_terms_q),
     // each coefficient as hi + lo: [4k]: phi (c0, c1), [4k + 1]: phi (c2, c3), [4k + 2]: V (c1, c2),
-    // [4k + 3]: V (c3, c0).  rho_k = fma(k, hr_f, r_min_f)
+    // [4k + 3]: V (c3, c0).  rho_k = fma(k, hr_f, r_min_f); row nk: the lines that continue V and
+    // phi below r_min, t0 rows below rho_0
     const float4 *TQ;
-    float hr_f, r_min_f;
+    float hr_f, r_min_f, t0;
     // fixed-point coordinates in units of 2^-qfb (Atoms::qfb), r^2 in units of 2^-U, U = 2 qfb - 42
     unsigned long long rc2q;  // r_cut^2
     float qs1;                // 2^(29 - qfb)

@@ -547,8 +547,7 @@ __device__ __forceinline__ void pair_terms_q(const Pot &P, unsigned long long r2
     // (two 32-byte loads: rows read at random cost the L1 a look-up per lane and load)
     float4 p0, p1, v0, v1;
     load_row_q(P, (int)kf, p0, p1, v0, v1);
-    const bool below = x < 0.f;   // linear continuation below the first knot, any distance from it
-    if (below) atomicAdd(&flags->range_violations, 1ull);
+    const bool deep = x < -0.5f;   // below the first knot, any distance from it
     // t = (r^2 - rho^2) / (r + rho) / h
     auto coord = [&](float k) {
         const float rho = __fmaf_rn(k, P.hr_f, P.r_min_f);
@@ -557,7 +556,7 @@ __device__ __forceinline__ void pair_terms_q(const Pot &P, unsigned long long r2
         const long long del = (long long)(r2 - rho2);
         df::F2 dd = df::make(__fmul_rn(__int2float_rn((int)(del >> P.dsh)), P.dsc1),
                              __fmul_rn(__uint2float_rn((unsigned)del & ((1u << P.dsh) - 1u)), P.dsc0));
-        if (below) {
+        if (deep) {
             const float f = __ll2float_rn(del);
             dd = df::make(__fmul_rn(f, P.dsc0), __fmul_rn(__ll2float_rn(del - (long long)f), P.dsc0));
         }
@@ -574,14 +573,16 @@ __device__ __forceinline__ void pair_terms_q(const Pot &P, unsigned long long r2
     // slope is off by about 1e-12 (its second derivative jumps at the knots), which such rows, one in
     // some thousand, would make the largest error of all.
     const float move = t.h < 0.f ? -1.f : (t.h > 1.f || (t.h == 1.f && t.l >= 0.f) ? 1.f : 0.f);
-    if (move != 0.f && !below && kf + move >= 0.f && kf + move <= last) {
+    if (kf == 0.f && __fadd_rn(__fadd_rn(t.h, P.t0), t.l) < 0.f) {   // below it: the line that continues it
+        atomicAdd(&flags->range_violations, 1ull);
+        load_row_q(P, P.nk, p0, p1, v0, v1);
+    } else if (move != 0.f && kf + move >= 0.f && kf + move <= last) {
         kf += move;
         load_row_q(P, (int)kf, p0, p1, v0, v1);
         t = coord(kf);
     }
-    const float on = below ? 0.f : 1.f;
-    const df::F2 c2 = df::make(p1.x * on, p1.y * on), c3 = df::make(p1.z * on, p1.w * on);
-    const df::F2 w2 = df::make(v0.z * on, v0.w * on), w3 = df::make(v1.x * on, v1.y * on);
+    const df::F2 c2 = df::make(p1.x, p1.y), c3 = df::make(p1.z, p1.w);
+    const df::F2 w2 = df::make(v0.z, v0.w), w3 = df::make(v1.x, v1.y);
     // q = c3 t, then c2 + q for the value and 2 c2 + 3 q for the slope
     const df::F2 q = mul_raw(t, c3), u = add_raw(c2, q);
     const df::F2 du = add_raw(df::make(2.f * u.h, 2.f * u.l), q);
