@@ -12,6 +12,7 @@
 
 #include "md_bits.cuh"
 #include "md_internal.cuh"
+#include "md_pack2.cuh"
 
 namespace mdk {
 namespace ph {
@@ -630,7 +631,11 @@ __device__ __forceinline__ int build_cell_group(const Atoms &A, const Cells &C, 
 // A lane per home atom (build_cell_group) appended candidate by candidate with most lanes idle,
 // and the appends' address chain bounded it.  Per rebuild, list phase, before -> after (us): 32 bcc
 // Fe replicas of 623,572 atoms 473 -> 350, Fe-C 250,250 221 -> 129, bcc Fe 2,000 65 -> 29, fcc Cu
-// 500,000 994 -> 984 (57 instructions per home atom and 32 candidates; issue slots 75 % busy).
+// 500,000 994 -> 984 (57 instructions per home atom and 32 candidates; issue slots 75 % busy).  With the
+// candidates' shifted positions formed once, two homes at a time in packed FP32 arithmetic and the band
+// looked at only where a candidate was accepted, the issue slots bound it less: a 20-step call of
+// fcc Cu 500,000 mixed 12.55 -> 11.92 ms, its rebuilds 202 -> 169 us a step at FP64; the 32 replicas
+// 3.39 -> 3.20 ms.  (Cells r_list / 2 wide, 42 % fewer candidates: 165 us a step, and slower passes.)
 // MARK: entries inside r_cut (FP32) get kInsideMark, for partition_row_warp.
 template <bool MARK>
 __device__ __forceinline__ int build_slice(const Atoms &A, const Cells &C, const Box *boxes, int c, int slice, int S,
@@ -648,11 +653,14 @@ __device__ __forceinline__ int build_slice(const Atoms &A, const Cells &C, const
     const bool edge = cx < R || cx >= nx - R || cy < R || cy >= ny - R || cz < R || cz >= nz - R;
     const unsigned full = 0xffffffffu, below = (1u << lane) - 1u;
     const int homes = (e - s + S - 1) / S;
+    const unsigned row4 = 4u * (unsigned)A.n;
+    constexpr float kFar = 1e18f;   // an x further from every atom than any list reaches
     int longest = 0;
     for (int h0 = 0; h0 < homes; h0 += 32) {
         const int nh = min(32, homes - h0);
         const int mine = s + S * (h0 + min(lane, nh - 1));   // this lane's home atom
-        const float4 fh = A.posf[mine];
+        const float4 fp = A.posf[mine];
+        const float hx = lane < nh ? -fp.x : kFar, hy = -fp.y, hz = -fp.z;
         int cnt = 0;
         for (int q0 = 0; q0 < nst; q0 += 32) {   // (one round for reach 1)
             // this lane's stencil cell: its first atom, length and shift by whole box edges
@@ -701,24 +709,38 @@ __device__ __forceinline__ int build_slice(const Atoms &A, const Cells &C, const
                 const int t = base + __popc(starts & (below | (1u << lane)));
                 const int j = __shfl_sync(full, first, t) + p0 + lane - __shfl_sync(full, off, t);
                 const float ox = __shfl_sync(full, sx, t), oy = __shfl_sync(full, sy, t), oz = __shfl_sync(full, sz, t);
-                const bool live = p0 + lane < total;
-                float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (live) f = A.posf[j];
-                for (int a = 0; a < nh; a++) {
-                    const float dx = f.x + (ox - __shfl_sync(full, fh.x, a)), dy = f.y + (oy - __shfl_sync(full, fh.y, a)),
-                                dz = f.z + (oz - __shfl_sync(full, fh.z, a));
-                    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                float x = kFar, y = 0.f, z = 0.f;
+                if (p0 + lane < total) {
+                    const float4 f = A.posf[j];
+                    x = f.x + ox;
+                    y = f.y + oy;
+                    z = f.z + oz;
+                }
+                auto append = [&](float r2, int a) {
                     const int i = s + S * (h0 + a);
-                    bool in = live && r2 <= band_hi && j != i;
+                    bool in = r2 <= band_hi && j != i;
+                    unsigned m = __ballot_sync(full, in);
+                    if (m == 0u) return;
                     if (__any_sync(full, in && r2 >= band_lo)) {   // the band: the exact test decides
                         if (in && r2 >= band_lo) in = within_exact_band(A.pos, i, j, B, rl2);
+                        m = __ballot_sync(full, in);
                     }
-                    const unsigned m = __ballot_sync(full, in);
-                    if (m == 0u) continue;
                     const int k = __shfl_sync(full, cnt, a) + __popc(m & below);
                     if (in && k < kmax)
-                        A.nbr[4 * ((long long)(k >> 2) * A.n + i) + (k & 3)] = MARK && r2 < A.pair_rc2f ? j | kInsideMark : j;
+                        A.nbr[4 * (size_t)i + (unsigned long long)(unsigned)(k >> 2) * row4 + (k & 3)] =
+                            MARK && r2 < A.pair_rc2f ? j | kInsideMark : j;
                     if (lane == a) cnt += __popc(m);
+                };
+                for (int a = 0; a < nh; a += 2) {   // two home atoms at a time (an odd last one: kFar)
+                    auto less = [&](float c, float h) {   // c + the two homes' negated coordinates
+                        return pk::add2(pk::pack(c, c),
+                                        pk::pack(__shfl_sync(full, h, a), __shfl_sync(full, h, a + 1)));
+                    };
+                    const pk::F2 dx = less(x, hx), dy = less(y, hy), dz = less(z, hz);
+                    float r0, r1;
+                    pk::unpack(pk::fma2(dx, dx, pk::fma2(dy, dy, pk::mul2(dz, dz))), r0, r1);
+                    append(r0, a);
+                    append(r1, a + 1);
                 }
             }
         }

@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "md_eam_common.cuh"
+#include "md_pack2.cuh"
 #include "md_phases.cuh"
 
 namespace mdk {
@@ -27,33 +28,8 @@ constexpr float kLog2e = 1.4426950408889634f;
 
 __device__ __forceinline__ float mi(float d, float L, float iL) { return d - L * rintf(d * iL); }
 
-// Two FP32 values in one 64-bit register pair and the packed operations on them (PTX f32x2: each
-// half rounded as the scalar operation), which halve the issue slots of the channel loops: those
-// bound these kernels.  The halves are two consecutive pairs of the row.
-struct F2 {
-    unsigned long long v;
-};
-__device__ __forceinline__ F2 pack(float a, float b) {
-    F2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack(F2 x, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v)); }
-__device__ __forceinline__ F2 add2(F2 a, F2 b) {
-    F2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
-    F2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
-    F2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return r;
-}
+using namespace pk;   // the packed operations of the channel loops (the halves: consecutive pairs of the row)
+
 __device__ __forceinline__ float both(F2 x) {
     float a, b;
     unpack(x, a, b);
