@@ -97,7 +97,9 @@ struct md_ctx {
 
 namespace {
 
-constexpr int kRebuildLaunches = 9;                     // kernels of one stand-alone launch_rebuild
+// Kernels of one stand-alone rebuild: the cooperative one, or launch_rebuild's nine and the clearing
+// one for the contexts with local rows.
+int rebuild_launches(const md_ctx *c, bool clear = true) { return c->C.tile ? 9 + (clear ? 1 : 0) : 1; }
 constexpr unsigned long long kSpinLimit = 20000000ull;  // barrier polls (~2 s) before giving up
 
 md_status fail(md_ctx *c, md_status s, const std::string &what, cudaError_t e = cudaSuccess) {
@@ -258,10 +260,23 @@ cudaError_t reset_errors(md_ctx *ctx) {
     return cudaMemsetAsync(ctx->d_bar, 0, sizeof(GridBarrier) + 2 * sizeof(int32_t), ctx->stream);
 }
 
-cudaError_t enqueue_rebuild(md_ctx *ctx) {
+StepParams step_params(md_ctx *ctx, int n_steps);
+
+// The list rebuild if it is requested, and the request cleared: one cooperative kernel, which costs
+// about 4 us where nothing is requested; nine kernels that return at once and the clearing one cost
+// 35 (five surrogate steps of 524,288 atoms 3.15 -> 2.98 ms; two single points of 432 atoms, which do
+// rebuild, 287 -> 281 us).  The contexts with local rows (group walks) keep the nine: those
+// rows are built by 8 blocks a SM, and a step of theirs rebuilds in the step kernel anyway.
+// clear: whether nothing behind it clears the request (the density kernel does).
+cudaError_t enqueue_rebuild(md_ctx *ctx, cudaStream_t s, bool clear = true) {
+    if (!ctx->C.tile) {
+        StepParams sp = step_params(ctx, INT32_MAX);   // (of md_step's segments: stopped before any last step)
+        return launch_rebuild_step(ctx->A, ctx->C, ctx->P, ctx->precision, ctx->lanes, sp, ctx->d_bar, nullptr, s);
+    }
     float lo, hi;
     list_band(ctx, lo, hi);
-    return launch_rebuild(ctx->A, ctx->C, ctx->rl2, lo, hi, ph_list_group(ctx), ctx->stream);
+    cudaError_t e = launch_rebuild(ctx->A, ctx->C, ctx->rl2, lo, hi, ph_list_group(ctx), s);
+    return e == cudaSuccess && clear ? launch_clear_rebuild(ctx->d_flags, s) : e;
 }
 
 // Surrogate network at the current positions (list valid): descriptors, then energies and
@@ -285,14 +300,11 @@ cudaError_t enqueue_sur_net(md_ctx *ctx, cudaStream_t s) {
 cudaError_t enqueue_sur_step(md_ctx *ctx, bool energy, bool scheduled_rebuild, int *rows, cudaStream_t s) {
     cudaError_t e = launch_sur_kick_drift(ctx->A, ctx->half_dt, ctx->dt, ctx->lim, s);
     if (e == cudaSuccess && scheduled_rebuild) e = launch_set_rebuild(ctx->d_flags, s);
-    float lo, hi;
-    list_band(ctx, lo, hi);
-    if (e == cudaSuccess) e = launch_rebuild(ctx->A, ctx->C, ctx->rl2, lo, hi, ph_list_group(ctx), s);
-    if (e == cudaSuccess) e = launch_clear_rebuild(ctx->d_flags, s);
+    if (e == cudaSuccess) e = enqueue_rebuild(ctx, s);
     if (e == cudaSuccess) e = enqueue_sur_net(ctx, s);
     if (e == cudaSuccess)
         e = launch_sur_force(ctx->A, ctx->S, 0, (int)ctx->n, true, energy, ctx->half_dt, 0.0, rows, s);
-    ctx->launches += 3 + kRebuildLaunches + (scheduled_rebuild ? 1 : 0);
+    ctx->launches += 2 + rebuild_launches(ctx) + (scheduled_rebuild ? 1 : 0);
     return e;
 }
 
@@ -300,11 +312,10 @@ cudaError_t enqueue_sur_step(md_ctx *ctx, bool energy, bool scheduled_rebuild, i
 // needed), with the FP64 partial sums; enqueue only.
 cudaError_t enqueue_forces(md_ctx *ctx) {
     if (ctx->sur) {
-        ctx->launches += 4 + kRebuildLaunches + (ctx->list_valid ? 0 : 1);
+        ctx->launches += 3 + rebuild_launches(ctx) + (ctx->list_valid ? 0 : 1);
         cudaError_t e = launch_check_displacement(ctx->A, ctx->lim, ctx->stream);
         if (e == cudaSuccess && !ctx->list_valid) e = launch_set_rebuild(ctx->d_flags, ctx->stream);
-        if (e == cudaSuccess) e = enqueue_rebuild(ctx);
-        if (e == cudaSuccess) e = launch_clear_rebuild(ctx->d_flags, ctx->stream);
+        if (e == cudaSuccess) e = enqueue_rebuild(ctx, ctx->stream);
         if (e == cudaSuccess) e = enqueue_sur_net(ctx, ctx->stream);
         int rows = 0;
         if (e == cudaSuccess)
@@ -316,10 +327,10 @@ cudaError_t enqueue_forces(md_ctx *ctx) {
                                 ctx->stream);
         return e;
     }
-    ctx->launches += 4 + kRebuildLaunches + (ctx->list_valid ? 0 : 1);
+    ctx->launches += 4 + rebuild_launches(ctx, false) + (ctx->list_valid ? 0 : 1);
     cudaError_t e = launch_check_displacement(ctx->A, ctx->lim, ctx->stream);
     if (e == cudaSuccess && !ctx->list_valid) e = launch_set_rebuild(ctx->d_flags, ctx->stream);
-    if (e == cudaSuccess) e = enqueue_rebuild(ctx);
+    if (e == cudaSuccess) e = enqueue_rebuild(ctx, ctx->stream, false);
     if (e == cudaSuccess) e = launch_density(ctx->A, ctx->P, ctx->precision, ctx->lanes, ctx->stream);
     if (e == cudaSuccess)
         e = launch_force(ctx->A, ctx->P, ctx->precision, ctx->lanes, false, true, 0.0, ctx->stream);
@@ -1155,9 +1166,8 @@ md_status sur_ensure_list(md_ctx *ctx) {
     MD_CK(reset_errors(ctx));
     MD_CK(launch_check_displacement(ctx->A, ctx->lim, ctx->stream));
     if (!ctx->list_valid) MD_CK(launch_set_rebuild(ctx->d_flags, ctx->stream));
-    MD_CK(enqueue_rebuild(ctx));
-    MD_CK(launch_clear_rebuild(ctx->d_flags, ctx->stream));
-    ctx->launches += 3 + kRebuildLaunches;
+    MD_CK(enqueue_rebuild(ctx, ctx->stream));
+    ctx->launches += 2 + rebuild_launches(ctx);
     md_status s = sync_and_check(ctx, false);
     if (s == MD_OK) ctx->list_valid = true;
     return s;
@@ -1340,9 +1350,8 @@ md_status md_build_neighbours(md_ctx *ctx) {
     if (!ctx) return MD_ERR_ARG;
     MD_CK(reset_errors(ctx));
     MD_CK(launch_set_rebuild(ctx->d_flags, ctx->stream));
-    MD_CK(enqueue_rebuild(ctx));
-    MD_CK(launch_clear_rebuild(ctx->d_flags, ctx->stream));
-    ctx->launches += 2 + kRebuildLaunches;
+    MD_CK(enqueue_rebuild(ctx, ctx->stream));
+    ctx->launches += 1 + rebuild_launches(ctx);
     md_status s = sync_and_check(ctx, false);
     if (s != MD_OK) return s;
     ctx->list_valid = true;

@@ -388,6 +388,7 @@ int step_walk(const Atoms &A, const Cells &C, const Pot &P, int precision, int l
 // The list rebuild of an md_step call between two launches of the step kernel: a cooperative
 // kernel of its own (more warps per SM than the step kernel keeps), which does nothing unless
 // the last launch stopped at a rebuild request (Flags::seg_done < sp.n_steps, need_rebuild set).
+// With sp.n_steps = INT32_MAX it is the stand-alone rebuild: whenever need_rebuild is set.
 cudaError_t launch_rebuild_step(const Atoms &A, const Cells &C, const Pot &P, int precision, int lanes,
                                 const StepParams &sp, GridBarrier *bar, unsigned long long *stamps, cudaStream_t s);
 

@@ -1,6 +1,7 @@
 // Link-cell binning and Verlet neighbour list (§3.2.1 of the MOLDY paper), as stand-alone
-// kernels (used by md_build_neighbours and md_eam_forces; the step kernel runs the same
-// per-item functions inside one persistent launch).
+// kernels for the contexts of the group walks (md_build_neighbours and md_eam_forces there; other
+// contexts rebuild in the cooperative kernel k_rebuild, and the step kernel runs the same per-item
+// functions inside its persistent launch).
 //
 // Rebuild pipeline, all on the launching stream and all returning at once when the device
 // flag `need_rebuild` is clear.  The per-atom and per-cell kernels loop over their items with a
@@ -69,8 +70,7 @@ __global__ void k_scan_apply(Cells C, const Flags *f) {
 __global__ void k_scatter(Atoms A, Cells C) {
     if (!ph::rebuild_requested(A.flags)) return;
     for (long long i = gtid(); i < A.n; i += gstride()) ph::scatter_atom(A, C, (int)i);
-    if (C.tile)
-        for (long long g = gtid(); g < C.n_groups; g += gstride()) ph::group_table(C, (int)g, A.flags);
+    for (long long g = gtid(); g < C.n_groups; g += gstride()) ph::group_table(C, (int)g, A.flags);
 }
 
 __global__ void k_cell_sort(Atoms A, Cells C) {
@@ -100,10 +100,9 @@ __global__ void __launch_bounds__(kThreads, 8) k_build_local(Atoms A, Cells C, d
     if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(&A.flags->max_count, m);
 }
 
-template <bool MARK>
 __global__ void __launch_bounds__(kThreads, 8) k_build_list(Atoms A, Cells C, double rl2, float band_lo, float band_hi) {
     if (!ph::rebuild_requested(A.flags)) return;
-    int m = ph::build_slices<MARK>(A, C, A.boxes, gtid() >> 5, gstride() >> 5, threadIdx.x & 31, rl2, band_lo, band_hi);
+    int m = ph::build_slices<false>(A, C, A.boxes, gtid() >> 5, gstride() >> 5, threadIdx.x & 31, rl2, band_lo, band_hi);
     m = __reduce_max_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(&A.flags->max_count, m);
 }
@@ -140,12 +139,6 @@ cudaError_t launch_clear_rebuild(Flags *f, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// FP64 pair walk: each row's entries j > i first (one warp per atom), after a build only.
-__global__ void k_partition_rows(Atoms A) {
-    if (!ph::rebuild_requested(A.flags)) return;
-    for (long long w = gtid() >> 5; w < A.n; w += gstride() >> 5) ph::partition_row_warp(A, (int)w, threadIdx.x & 31);
-}
-
 cudaError_t launch_rebuild(const Atoms &A, const Cells &C, double rl2, float band_lo, float band_hi,
                            int list_group, cudaStream_t s) {
     const int nb = capped_blocks(A.n, kThreads);
@@ -164,9 +157,7 @@ cudaError_t launch_rebuild(const Atoms &A, const Cells &C, double rl2, float ban
         const int nbs = capped_blocks((long long)A.n * 32, kThreads);
         if (C.tile == kWalkStaged) launch_build<1>(A, C, rl2, band_lo, band_hi, list_group, nbl, s);
         else if (C.tile == kWalkHalf) launch_build<2>(A, C, rl2, band_lo, band_hi, list_group, nbl, s);
-        else if (A.pairs) k_build_list<true><<<nbs, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
-        else k_build_list<false><<<nbs, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
-        if (A.pairs) k_partition_rows<<<nbs, kThreads, 0, s>>>(A);
+        else k_build_list<<<nbs, kThreads, 0, s>>>(A, C, rl2, band_lo, band_hi);
     }
     return cudaGetLastError();
 }

@@ -676,7 +676,8 @@ cudaError_t launch_t(const Atoms &A, const Cells &C, const Pot &P, const StepPar
                                        args, dyn, s);
 }
 
-// The rebuild between two launches of the step kernel (md_internal.cuh launch_rebuild_step).
+// The rebuild between two launches of the step kernel, and the stand-alone one (md_internal.cuh
+// launch_rebuild_step).
 constexpr int kRebuildThreads = 256;
 #ifndef MD_REBUILD_MIN_BLOCKS   // blocks of kRebuildThreads per SM the rebuild kernel is built for
 #define MD_REBUILD_MIN_BLOCKS 4
@@ -714,12 +715,13 @@ cudaError_t launch_rebuild_t(const Atoms &A, const Cells &C, const StepParams &s
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
         grid = std::min(per_sm * n_sm, kGridMax);
     }
+    // up to a warp per atom: a small system's barriers are cheaper among fewer blocks
+    const int nb = (int)std::min<long long>(grid, std::max<long long>(1, ((long long)A.n * 32 + kRebuildThreads - 1) / kRebuildThreads));
     Atoms a = A;
     Cells c = C;
     StepParams q = sp;
     void *args[] = {&a, &c, &q, &bar, &stamps};
-    return cudaLaunchCooperativeKernel((const void *)k_rebuild<WALK>, dim3(grid), dim3(kRebuildThreads), args, 0,
-                                       s);
+    return cudaLaunchCooperativeKernel((const void *)k_rebuild<WALK>, dim3(nb), dim3(kRebuildThreads), args, 0, s);
 }
 
 template <int PREC, int T>
