@@ -637,9 +637,10 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
             const bool mixed = cfg->precision == MD_PREC_MIXED;
             int t = 1, dev = 0, n_sm = 0;
             while (t < 8 && t * (mixed ? 24 : 20) < k_est) t *= 2;
+            // (without a device the checks below still come first, and the allocations report it)
             if (cudaGetDevice(&dev) != cudaSuccess ||
                 cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-                return MD_ERR_CUDA;
+                n_sm = 1;
             if (mixed && t > 1 && n * t > 16 * (int64_t)n_sm * 1024) t /= 2;
             const int64_t fill = (int64_t)n_sm * (mixed ? 192 : 512);
             while (t < 8 && 2 * n * t <= fill && 4 * t <= k_est) t *= 2;
