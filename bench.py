@@ -65,8 +65,9 @@ def _peaks():
         return 6800.0, "fallback (6.8 TB/s)"
 
 
-# FP64 operations per list entry of the FP64 passes, counted from the pair code (an add or a
-# multiply is 1 flop, an FMA 2; conversions and rounding to integer not counted).  Entries
+# FP64 operations per list entry of the FP64 passes when every pair term is FP64 arithmetic (an add
+# or a multiply is 1 flop, an FMA 2; conversions and rounding to integer not counted): the work at
+# FP64 accuracy, of which the passes do most on the FP32 and integer pipes.  Entries
 # inside r_cut: density 35 (separation 3, r^2 5, FP64 refinement of the reciprocal square root 6,
 # r 1, knot index 3, the cubic of phi 6, the sum 1, the derivative cubics of phi and V 8, their
 # scaling by 1/r 2) + force 12 (separation 3, the pair scalar from the cached derivatives 3, the
@@ -428,8 +429,9 @@ def run_ours(args):
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": r64["ms"] / args.steps,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
         "data": "synthetic",
-        "config": dict(_config("fp64: every sum, the integration and every reduction in FP64; the pair terms in FP64 "
-                               "arithmetic, 1/r and r^2 formed from exact FP32 pieces to <= 4e-13 relative"),
+        "config": dict(_config("fp64: every sum, the integration and every reduction in FP64; the pair terms as sums of "
+                               "two FP32 numbers over exact whole-number separations, forces closer to 64-bit "
+                               "arithmetic than one Newton step of 1/r in FP64 gives (5e-14 of the RMS force)"),
                        fp64_walk=("half list: each pair once, the neighbour's share by FP64 atomics"
                                   if fp64_leg == "fp64_half" else "full list: each pair from both sides")),
         "roofline": {"bound": "alu", "achieved": achieved, "peak": fp64_tflops, "unit": "TFLOP/s",
@@ -437,8 +439,9 @@ def run_ours(args):
                      "kernel": "k_step (persistent: all phases of the K steps, stopping at each rebuild request "
                                "for the k_rebuild kernel and resuming), FP64 pipe",
                      "peak_source": "measured in this run: md_measure_fp64_peak (FP64 FMA chains, CUDA events)",
-                     "flop_model": "47 FP64 flop per list entry inside r_cut over both passes, 20 in the skin "
-                                   "shell (an FMA counts 2); half of it with the half list",
+                     "flop_model": "work at FP64 accuracy: 47 flop per list entry inside r_cut over both passes, 20 "
+                                   "in the skin shell (an FMA counts 2), half of it with the half list; most of it is "
+                                   "done on the FP32 and integer pipes",
                      "flop_per_launch": flop, "avg_launch_ms": r64["ms"], "hbm": hbm(r64, "fp64")},
         "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": r64["launches"], "clocks": r64["clocks"],
         "nve_drift_ev_per_atom": (r64["e1"]["te"] - r64["e0"]["te"]) / n,

@@ -113,9 +113,9 @@ typedef struct {
     int32_t rebuild_every; /* `nbrupdate`: rebuild every n steps; 0 = only when needed */
     double dt_fs;          /* `deltat` */
     int32_t precision;     /* MD_PREC_FP64 (every sum, the integration and the reductions in
-                              FP64; of the pair terms, 1/r and, in the half list's density
-                              pass, r^2 are formed to FP64 accuracy from exact FP32 pieces,
-                              relative error <= 4e-13, the rest is FP64 arithmetic), or
+                              FP64; the pair terms of one-species tables as sums of two FP32
+                              numbers over whole-number separations (about 2^-46), else FP64
+                              arithmetic with 1/r formed to <= 4e-13 relative), or
                               MD_PREC_MIXED (FP32 pair/density terms,
                               FP64 positions, velocities, density sum and reductions; with
                               one species and knot tables the force pass takes the quadratic
@@ -134,7 +134,7 @@ typedef struct {
     void *stream;          /* cudaStream_t, or NULL */
     int32_t lanes_per_atom; /* threads sharing one atom's neighbour sums in the force passes:
                                1, 2, 4, 8, 16 or 32, or 0 = chosen from the expected neighbour
-                               count (see md_tune).  Results depend on it only in rounding. */
+                               count and the number of atoms (see md_tune).  Results depend on it only in rounding. */
     int32_t passes;         /* MD_PASSES_AUTO (0), MD_PASSES_LIST, MD_PASSES_STAGED, MD_PASSES_CELLS or
                                MD_PASSES_HALF: how the mixed-precision step kernel walks the neighbours */
     int32_t integrator;     /* MD_INTEGRATOR_VERLET (0) or MD_INTEGRATOR_PC3 (Table 1 `iverlet`: 1 and 0
