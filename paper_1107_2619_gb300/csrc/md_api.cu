@@ -976,14 +976,16 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
                 P.x0_h = x0.h;
                 P.x0_l = x0.l;
                 TQ.resize(4 * (size_t)(nk + 1));
-                P.t0 = (float)(((long double)rmf - pot->r_min) * P.inv_dr);
+                P.t0 = (float)(((double)rmf - pot->r_min) * P.inv_dr);
                 for (int row = 0; row <= nk; row++) {
                     // the row's cubics about rho_k, s rows beyond its knot (row nk: the lines at the first)
                     const int k = row < nk ? row : 0;
-                    const long double s = ((long double)std::fma((float)k, hrf, rmf) - pot->r_min) * P.inv_dr - k;
+                    // (s is small: FP64 is enough, and long double is software on Arm)
+                    const double s = std::fma((double)std::fma((float)k, hrf, rmf) - pot->r_min, P.inv_dr, -(double)k);
                     auto about = [s](const double4_32a &c) {
-                        return make_double4_32a((double)(c.x + s * (c.y + s * (c.z + s * c.w))),
-                                                (double)(c.y + s * (2 * c.z + 3 * s * c.w)), (double)(c.z + 3 * s * c.w), c.w);
+                        return make_double4_32a(std::fma(s, std::fma(s, std::fma(s, c.w, c.z), c.y), c.x),
+                                                std::fma(s, std::fma(3.0 * s, c.w, 2.0 * c.z), c.y), std::fma(3.0 * s, c.w, c.z),
+                                                c.w);
                     };
                     double4_32a v = VP64[2 * k], p = VP64[2 * k + 1];
                     if (row == nk) v.z = v.w = p.z = p.w = 0.0;
