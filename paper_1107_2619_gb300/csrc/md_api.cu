@@ -955,7 +955,9 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
             }
             // (rho_0^2 a whole number of the units; rho_k within 1e-3 of a row of its knot)
             const int whole = rmf > 0.f ? U - 300 + 2 * (std::ilogb(rmf) + 127) : -1;
-            if (fb >= 45 && fb <= 51 && nk <= 20000 && whole >= 0 && dbits >= 25 && dbits <= 55 && fits(mv) &&
+            // (r_cut beyond what the pieces leave to FP64, ps::kCloseR2)
+            const bool far = pot->r_cut > std::ldexp(1.0, 46 - fb);
+            if (fb >= 45 && fb <= 51 && nk <= 20000 && whole >= 0 && dbits >= 25 && dbits <= 55 && far && fits(mv) &&
                 fits(mp) && fits(mf) && fits(P.inv_dr)) {
                 A.qfb = fb;
                 P.hr_f = hrf;
@@ -964,8 +966,8 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
                 P.qs1 = (float)std::ldexp(1.0, 29 - fb);
                 P.qe1 = (unsigned)(127 + 23 + 14 - fb) << 23;
                 P.qe0 = (unsigned)(127 + 23 - fb) << 23;
-                P.q2h = (float)std::ldexp(1.0, 40 - U);
-                P.q2l = (float)std::ldexp(1.0, 8 - U);
+                P.q2h = (unsigned)(127 + 22 + 40 - U) << 23;
+                P.q2l = (unsigned)(127 + 8 - U) << 23;
                 P.q2e = U - 300;
                 P.dsh = dbits - 24;
                 P.dsc1 = (float)std::ldexp(1.0, P.dsh - U);

@@ -47,6 +47,7 @@ struct Box {
 struct Flags {
     int32_t error;          // FLAG_* bits (this word and the next are cleared at the start of every call)
     int32_t skin_exceeded;  // an atom moved more than skin/2 since the last build
+    int32_t close_pairs;    // a density pass since the last build met a close pair (ps::kCloseR2)
     int32_t need_rebuild;   // set by the displacement check or the schedule; cleared by pass 1
     int32_t max_count;      // longest list at the last build
     unsigned long long n_rebuilds;
@@ -105,7 +106,7 @@ struct Pot {
     unsigned long long rc2q;  // r_cut^2
     float qs1;                // 2^(29 - qfb)
     unsigned qe1, qe0;        // the FP32 numbers whose last bit is worth 2^(14 - qfb), 2^-qfb
-    float q2h, q2l;           // 2^(40 - U), 2^(8 - U)
+    unsigned q2h, q2l;        // FP32 bit patterns: of 2^(40 - U) times 2^23 less its leading bit, of 2^(8 - U)
     int q2e;                  // U - 300: rho^2 = significand^2 2^(q2e + 2 exponent field)
     int dsh;                  // low bits of r^2 - rho^2 taken as the low part
     float dsc1, dsc0;         // 2^(dsh - U), 2^-U

@@ -528,10 +528,15 @@ __device__ __forceinline__ void load_row_q(const Pot &P, int k, float4 &p0, floa
     load2(P.TQ + 4 * (size_t)k + 2, v0, v1);
 }
 
-// The terms of a pair at r2 = r^2 (r2_fixed), inside r_cut.
+// The terms of a pair at r2 = r^2 (r2_fixed), inside r_cut and not close (outside_q).
 __device__ __forceinline__ void pair_terms_q(const Pot &P, unsigned long long r2, bool energy, PairQ &o, Flags *flags) {
-    const df::F2 x2 = df::make(__fmul_rn(__uint2float_rn((unsigned)(r2 >> 40)), P.q2h),
-                               __fmul_rn(__uint2float_rn((unsigned)(r2 >> 8)), P.q2l));
+    // r^2 from its leading bit on, 24 bits and the 32 below them, so that its relative error does not
+    // depend on r or on the unit (cut at fixed bits, 1/r was off by 1.5e-13 at 2.5 A, qfb 49, and by 1e-9 at 0.1)
+    const int lz = __clz((unsigned)(r2 >> 32));
+    const unsigned long long n2 = r2 << lz;
+    const unsigned down = (unsigned)lz << 23;
+    const df::F2 x2 = df::make(__uint_as_float((unsigned)(n2 >> 40) + (P.q2h - down)),
+                               __fmul_rn(__uint2float_rn((unsigned)(n2 >> 8)), __uint_as_float(P.q2l - down)));
     // 1/r: estimate y, e = 1 - r^2 y^2 as hi + lo, 1/r = y + y (e/2 + 3 e^2/8)
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x2.h));
@@ -629,6 +634,93 @@ __device__ __forceinline__ void store_pass2(const Atoms &A, int i, double dF) {
     }
 }
 
+// Close pairs: r^2 < 2^48 units, that is r < 2^(45 - qfb) Å (0.03 Å at qfb 50, 1 Å at 45).  There the
+// unit itself would show (2^-qfb against r; further apart it stays below 2^-44 of r) and pair_terms_q's
+// numbers run out of bits, so their terms are FP64 arithmetic on the FP64 positions, as without the
+// pieces.  They are rare: the walks pass them by with the pairs beyond r_cut (one comparison for both,
+// a zero in the derivative cache), and a density walk that met one goes over its entries once more for
+// them and raises Flags::close_pairs (until the next rebuild), at which the force walks do the same.
+// (Handled inside the walks the FP64 code cost registers: fcc Cu 83,000 atoms 403 -> 427 us a step.)
+// The force pass reads A.posq and A.posd for them, so no atom moves before all have passed it (k_step).
+constexpr unsigned long long kCloseR2 = 1ull << 48;
+__device__ __forceinline__ bool outside_q(const Pot &P, unsigned long long r2) { return r2 - kCloseR2 >= P.rc2q - kCloseR2; }
+
+struct CloseTerms {
+    double phi, V, gV, gphi;   // as PairQ
+    double dx, dy, dz, sx, sy, sz;   // x_j - x_i in the minimum image, and the box edges taken off
+};
+static __device__ __noinline__ CloseTerms close_terms(const double4_32a *posd, const Box *B, int i, int j,
+                                                      const double4_32a *VP64, const double4_32a *D64, int nk,
+                                                      double inv_dr, double xneg, Flags *flags) {
+    const double4_32a a = ld_phase(posd + i), b = ld_phase(posd + j);
+    CloseTerms o;
+    o.dx = mi64s(b.x - a.x, B->L[0], o.sx);
+    o.dy = mi64s(b.y - a.y, B->L[1], o.sy);
+    o.dz = mi64s(b.z - a.z, B->L[2], o.sz);
+    const double r2 = fma(o.dx, o.dx, fma(o.dy, o.dy, o.dz * o.dz));
+    const double rinv = rsqrt64(r2);
+    double t;
+    bool below;
+    const int k = knot_row64(fma(r2 * rinv, inv_dr, xneg), nk, t, below);
+    if (below && flags) atomicAdd(&flags->range_violations, 1ull);
+    const double4_32a dv = D64[2 * k], dp = D64[2 * k + 1];
+    o.phi = cubic64(t, VP64[2 * (size_t)k + 1], below);
+    o.V = cubic64(t, VP64[2 * (size_t)k], below);
+    o.gV = (below ? dv.x : fma(t, fma(dv.z, t, dv.y), dv.x)) * rinv;
+    o.gphi = (below ? dp.x : fma(t, fma(dp.z, t, dp.y), dp.x)) * rinv;
+    return o;
+}
+// fn(j, terms) for the close pairs among entries k0, k0 + step, ... < end of atom i's row.
+template <typename Fn>
+__device__ __forceinline__ void for_close(const Atoms &A, const Pot &P, const Box *boxes, int i, int k0, int step, int end,
+                                          Flags *flags, Fn &&fn) {
+    const Box &B = boxes[ph::replica_of(A, i)];
+    const double4_32a qi = ld_phase(A.posq + i);
+    const NbrRow row = nbr_row(A, i);
+    for (int k = k0; k < end; k += step) {
+        const int j = ld_phase(row.ptr(k));
+        if (r2_fixed<std::true_type>(ld_phase(A.posq + j), qi, B) < kCloseR2)
+            fn(j, close_terms(A.posd, &B, i, j, P.VP64, P.D64, P.nk, P.inv_dr, P.xneg, flags));
+    }
+}
+// The radial factor of the pair (i, j) in the force pass.
+__device__ __forceinline__ double close_radial(const Atoms &A, int i, int j, const CloseTerms &c) {
+    return fma(to64(fprime_q(ld_phase(A.p2d + i).w)) + to64(fprime_q(ld_phase(A.p2d + j).w)), c.gphi, c.gV);
+}
+// The half list's close pairs: both atoms' shares by atomic adds.
+__device__ __forceinline__ void close_density_pairs(const Atoms &A, const Pot &P, const Box *boxes, int i, int k0, int step,
+                                                    bool energy) {
+    A.flags->close_pairs = 1;
+    for_close(A, P, boxes, i, k0, step, ld_phase(A.cup + i), A.flags, [&](int j, const CloseTerms &c) {
+        atomicAdd(A.rho_acc + i, c.phi);
+        atomicAdd(A.rho_acc + j, c.phi);
+        if (energy) {
+            atomicAdd(A.e_acc + i, half64(c.V));
+            atomicAdd(A.e_acc + j, half64(c.V));
+        }
+    });
+}
+template <bool ENERGY>
+__device__ __forceinline__ void close_force_pairs(const Atoms &A, const Pot &P, const Box *boxes, int i, int k0, int step,
+                                                  double (&part)[kPartials]) {
+    for_close(A, P, boxes, i, k0, step, ld_phase(A.cup + i), nullptr, [&](int j, const CloseTerms &c) {
+        const double g = close_radial(A, i, j, c);
+        const double gx = g * c.dx, gy = g * c.dy, gz = g * c.dz;
+        double *fi = reinterpret_cast<double *>(A.f_acc + i), *fj = reinterpret_cast<double *>(A.f_acc + j);
+        atomicAdd(fi, gx);
+        atomicAdd(fi + 1, gy);
+        atomicAdd(fi + 2, gz);
+        atomicAdd(fj, -gx);
+        atomicAdd(fj + 1, -gy);
+        atomicAdd(fj + 2, -gz);
+        if (ENERGY)
+            virial_shift(c.sx, c.sy, c.sz, -gx, -gy, -gz, part[2], part[3], part[4], part[5], part[6], part[7]);
+    });
+}
+__device__ __forceinline__ bool close_pairs(const Atoms &A) {
+    return A.qfb && *reinterpret_cast<volatile int32_t *>(&A.flags->close_pairs) != 0;
+}
+
 // ======================================================================= FP64
 // Per-atom sums of the FP64 force pass (and of the double-float pass, converted).
 struct Acc64 {
@@ -698,6 +790,7 @@ __device__ __forceinline__ void density64_sum(const Atoms &A, const Pot &P, cons
         // loaded while an entry is worked on (entries past the row's end: the last one again).
         // The chain list entry -> record bounded the walk at 16 warps an SM: full list, fcc Cu 83,000 atoms,
         // 8 lanes, us a step: density 229 -> 184, force 281 -> 188.
+        bool close = false;
         auto walk_q = [&](auto wrapt) {
             using W = decltype(wrapt);
             const double4_32a qi = ld_phase(A.posq + i);
@@ -710,8 +803,9 @@ __device__ __forceinline__ void density64_sum(const Atoms &A, const Pot &P, cons
                 jn = ld_phase(row.ptr(min(k + 2 * T, cnt - 1)));
                 float4 *dc = reinterpret_cast<float4 *>(drow.ptr(k));
                 const unsigned long long r2 = r2_fixed<W>(qj, qi, B);
-                if (r2 >= P.rc2q) {
+                if (outside_q(P, r2)) {
                     *dc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    close |= r2 < kCloseR2;
                     continue;
                 }
                 PairQ o;
@@ -725,6 +819,13 @@ __device__ __forceinline__ void density64_sum(const Atoms &A, const Pot &P, cons
             if (A.qfb) {
                 if (wrap) walk_q(std::true_type{});
                 else walk_q(std::false_type{});
+                if (close) {
+                    A.flags->close_pairs = 1;
+                    for_close(A, P, boxes, i, lane, T, cnt, A.flags, [&](int, const CloseTerms &c) {
+                        rho += c.phi;
+                        if (energy) ep = fma(0.5, c.V, ep);
+                    });
+                }
             }
         }
         auto walk = [&](auto wrapt) {
@@ -871,6 +972,21 @@ __device__ __forceinline__ void force64_cached_sum(const Atoms &A, const Pot &P,
             if (A.qfb) {
                 if (wrap) walk_q(std::true_type{});
                 else walk_q(std::false_type{});
+                if (close_pairs(A))
+                    for_close(A, P, boxes, i, lane, T, cnt, nullptr, [&](int j, const CloseTerms &c) {
+                        const double g = close_radial(A, i, j, c), gx = g * c.dx, gy = g * c.dy, gz = g * c.dz;
+                        fx += gx;
+                        fy += gy;
+                        fz += gz;
+                        if (ENERGY) {   // -1/2 g d (x) d
+                            wxx = fma(-0.5 * gx, c.dx, wxx);
+                            wyy = fma(-0.5 * gy, c.dy, wyy);
+                            wzz = fma(-0.5 * gz, c.dz, wzz);
+                            wyz = fma(-0.5 * gy, c.dz, wyz);
+                            wxz = fma(-0.5 * gx, c.dz, wxz);
+                            wxy = fma(-0.5 * gx, c.dy, wxy);
+                        }
+                    });
                 return;
             }
         }
@@ -1034,6 +1150,7 @@ __device__ __forceinline__ void density64_pairs_item(const Atoms &A, const Pot &
         const int cnt = ld_phase(A.cup + i);
         const NbrRow row = nbr_row(A, i);
         const DRow drow = dcache_row(A, i);
+        bool close = false;
         auto walk_q = [&](auto wrapt) {   // the pair terms from FP32 pieces
             using W = decltype(wrapt);
             const double4_32a qi = ld_phase(A.posq + i);
@@ -1042,8 +1159,9 @@ __device__ __forceinline__ void density64_pairs_item(const Atoms &A, const Pot &
                 const double4_32a qj = ld_phase(A.posq + j);
                 float4 *dc = reinterpret_cast<float4 *>(drow.ptr(k));
                 const unsigned long long r2 = r2_fixed<W>(qj, qi, B);
-                if (r2 >= P.rc2q) {
+                if (outside_q(P, r2)) {
                     *dc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    close |= r2 < kCloseR2;
                     continue;
                 }
                 PairQ o;
@@ -1063,6 +1181,7 @@ __device__ __forceinline__ void density64_pairs_item(const Atoms &A, const Pot &
             if (A.qfb) {
                 if (wrap) walk_q(std::true_type{});
                 else walk_q(std::false_type{});
+                if (close) close_density_pairs(A, P, boxes, i, lane, T, energy);
             }
         }
         auto walk = [&](auto wrapt) {
@@ -1538,6 +1657,7 @@ __device__ __forceinline__ void density64_pairs_flat_q(const Atoms &A, const Pot
     for (int q = 0; q < 2 * AW; q++) S[q * 32 + lane] = 0.0;
     double *const rec = S + 3 * AW * 32;
     stage_records<AW>(A, A.posq, i0, lane, rec);
+    bool close = false;
     auto walk = [&](auto wrapt) {
         using W = decltype(wrapt);
         for (int seg = 0; seg < 2; seg++) {
@@ -1567,8 +1687,9 @@ __device__ __forceinline__ void density64_pairs_flat_q(const Atoms &A, const Pot
                 const int i = i0 + x.a;
                 float4 *dc = reinterpret_cast<float4 *>(dcache_row(A, i).ptr(x.k));
                 const unsigned long long r2 = r2_fixed<W>(pj, record(rec, x.a), boxes[W::value ? ph::replica_of(A, i) : 0]);
-                if (r2 >= P.rc2q) {
+                if (outside_q(P, r2)) {
                     *dc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    close |= r2 < kCloseR2;
                     continue;
                 }
                 PairQ o;
@@ -1599,6 +1720,8 @@ __device__ __forceinline__ void density64_pairs_flat_q(const Atoms &A, const Pot
         A.rho[me] = rho;
         if (energy) atomicAdd(A.e_acc + me, ep);
     }
+    if (__any_sync(0xffffffffu, close))
+        for (int i = i0; i < min(i0 + AW, A.n); i++) close_density_pairs(A, P, boxes, i, lane, 32, energy);
 }
 
 template <int T, bool ENERGY>
@@ -1701,6 +1824,11 @@ __device__ __forceinline__ void density64_pairs(const Atoms &A, const Pot &P, co
 template <int T, int KIND, bool ENERGY>
 __device__ __forceinline__ void force64_pairs(const Atoms &A, const Pot &P, const Box *boxes, long long g,
                                               double (&part)[kPartials], double *S) {
+    if constexpr (KIND == MD_POT_TABLES) {
+        if (close_pairs(A))
+            for (int i = (int)(g >> 5) * (32 / T), e = min(i + 32 / T, A.n); i < e; i++)
+                close_force_pairs<ENERGY>(A, P, boxes, i, (int)(g & 31), 32, part);
+    }
     if constexpr (T >= kFlatLanes && KIND == MD_POT_TABLES) {
         if (A.qfb) return force64_pairs_flat_q<T, ENERGY>(A, P, boxes, g, part, S);
     }

@@ -225,6 +225,7 @@ __device__ __forceinline__ bool rebuild_phases(const Atoms &A, const Cells &C, B
             A.flags->max_count = 0;
             A.flags->tile_bad = 0;
             A.flags->tile_max = 0;
+            A.flags->close_pairs = 0;
         }
         ph::scan_top(C, ws);
     }
@@ -468,7 +469,11 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
         }
         // ------------------------------------------------ force pass (+ kicks)
         const bool last = s == sp.n_steps - 1;
-        const bool fuse = !last && !strain && !thermo;
+        // (close pairs: the full list's force pass reads positions, so that the next step opens after it)
+        bool apart = strain;
+        if constexpr (PREC == MD_PREC_FP64 && WALK == kWalkList && KIND == MD_POT_TABLES && !MULTI)
+            apart = apart || ps::close_pairs(A);
+        const bool fuse = !last && !apart && !thermo;
         if (fuse && lead && sp.rebuild_every > 0 && (step + s + 2) % sp.rebuild_every == 0)
             A.flags->need_rebuild = 1;
         // (the group walks' own passes do not add the kinetic energies: a pass of their own does)
@@ -612,14 +617,14 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
                     A.vel[i] = v;
                 }
             }
-        } else if (!last && strain) {
+        } else if (!last && apart) {
             if (lead) {
-                strain_boxes(boxes, A.n_rep, sp.strain_scale, A.qfb);
+                if (strain) strain_boxes(boxes, A.n_rep, sp.strain_scale, A.qfb);
                 if (sp.rebuild_every > 0 && (step + s + 2) % sp.rebuild_every == 0) A.flags->need_rebuild = 1;
             }
             MD_SYNC();
             for (long long i = tid; i < A.n; i += stride)
-                ph::kick_drift(A, boxes, (int)i, sp.half_dt, sp.dt, sp.strain_scale, true, sp.lim);
+                ph::open_step(A, boxes, (int)i, sp.motion, sp.half_dt, sp.dt, sp.strain_scale, strain, sp.lim);
             MD_SYNC();
         }
     }
