@@ -564,9 +564,10 @@ __device__ __forceinline__ void pair_terms_q(const Pot &P, unsigned long long r2
         const long long del = (long long)(r2 - rho2);
         df::F2 dd = df::make(__fmul_rn(__int2float_rn((int)(del >> P.dsh)), P.dsc1),
                              __fmul_rn(__uint2float_rn((unsigned)del & ((1u << P.dsh) - 1u)), P.dsc0));
-        if (deep) {
-            const float f = __ll2float_rn(del);
-            dd = df::make(__fmul_rn(f, P.dsc0), __fmul_rn(__ll2float_rn(del - (long long)f), P.dsc0));
+        if (deep) {   // r < rho: the difference's size may take all 64 bits
+            const unsigned long long m = rho2 - r2;
+            const float f = __ull2float_rz(m);
+            dd = df::make(-__fmul_rn(f, P.dsc0), -__fmul_rn(__ull2float_rn(m - (unsigned long long)f), P.dsc0));
         }
         df::F2 sum = df::two_sum(r.h, rho);
         sum.l = __fadd_rn(sum.l, r.l);
