@@ -953,12 +953,14 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
                 mp = std::max({mp, std::fabs(p.x), std::fabs(p.y), std::fabs(p.z), std::fabs(p.w)});
                 mf = std::max({mf, std::fabs(FD64[k].x), std::fabs(FD64[k].y), std::fabs(FD64[k].z)});
             }
-            // (rho_0^2 a whole number of the units; rho_k within 1e-3 of a row of its knot)
+            // rho_k lies within s_max rows of its knot: three roundings to FP32 (r_min, h, the sum), one to spare
+            const double s_max = std::ldexp(4.0 * pot->r_cut * P.inv_dr, -24);
+            // (rho_0^2 a whole number of the units)
             const int whole = rmf > 0.f ? U - 300 + 2 * (std::ilogb(rmf) + 127) : -1;
             // (r_cut beyond what the pieces leave to FP64, ps::kCloseR2)
             const bool far = pot->r_cut > std::ldexp(1.0, 46 - fb);
-            if (fb >= 45 && fb <= 51 && nk <= 20000 && whole >= 0 && dbits >= 25 && dbits <= 55 && far && fits(mv) &&
-                fits(mp) && fits(mf) && fits(P.inv_dr)) {
+            if (fb >= 45 && fb <= 51 && nk <= 20000 && whole >= 0 && dbits >= 25 && dbits <= 55 && far &&
+                s_max <= 0.02 && fits(mv) && fits(mp) && fits(mf) && fits(P.inv_dr)) {
                 A.qfb = fb;
                 P.hr_f = hrf;
                 P.r_min_f = rmf;
@@ -979,6 +981,8 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
                 P.x0_l = x0.l;
                 TQ.resize(4 * (size_t)(nk + 1));
                 P.t0 = (float)(((double)rmf - pot->r_min) * P.inv_dr);
+                P.hr_s = (float)((hr - (double)hrf) * P.inv_dr);
+                P.near_s = (float)s_max;
                 for (int row = 0; row <= nk; row++) {
                     // the row's cubics about rho_k, s rows beyond its knot (row nk: the lines at the first)
                     const int k = row < nk ? row : 0;

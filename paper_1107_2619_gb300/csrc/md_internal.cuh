@@ -101,7 +101,8 @@ struct Pot {
     // [4k + 3]: V (c3, c0).  rho_k = fma(k, hr_f, r_min_f); row nk: the lines that continue V and
     // phi below r_min, t0 rows below rho_0
     const float4 *TQ;
-    float hr_f, r_min_f, t0;
+    float hr_f, r_min_f, t0, hr_s;   // hr_s: (h - hr_f) / h
+    float near_s;                    // rho_k lies within this many rows of its knot
     // fixed-point coordinates in units of 2^-qfb (Atoms::qfb), r^2 in units of 2^-U, U = 2 qfb - 42
     unsigned long long rc2q;  // r_cut^2
     float qs1;                // 2^(29 - qfb)

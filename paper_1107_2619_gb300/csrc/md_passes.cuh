@@ -578,11 +578,21 @@ __device__ __forceinline__ void pair_terms_q(const Pot &P, unsigned long long r2
         return df::fast_two_sum(tr.h, tr.l);
     };
     df::F2 t = coord(kf);
-    // The neighbouring row where t lies outside [0, 1): beside its interval by 1e-4 of a row a cubic's
-    // slope is off by about 1e-12 (its second derivative jumps at the knots), which such rows, one in
-    // some thousand, would make the largest error of all.
-    const float move = t.h < 0.f ? -1.f : (t.h > 1.f || (t.h == 1.f && t.l >= 0.f) ? 1.f : 0.f);
-    if (kf == 0.f && __fadd_rn(__fadd_rn(t.h, P.t0), t.l) < 0.f) {   // below it: the line that continues it
+    // The neighbouring row where r lies outside [r_k, r_k+1): beside its interval by 1e-4 of a row a cubic's
+    // slope is off by about 1e-12 at 5,000 knots and by 1e-10 at 300 (its second derivative jumps at the
+    // knots), which such pairs, one in some thousand, would make the largest error of all.  lo, hi: the
+    // signs of r - r_k, r - r_k+1; within near_s of a knot from rho_k - r_k = s rows, to 1e-7 of itself.
+    float lo = t.h, hi = __fsub_rn(t.h, 1.f);
+    if (fminf(fabsf(lo), fabsf(hi)) < P.near_s) {
+        const float rho = __fmaf_rn(kf, P.hr_f, P.r_min_f);
+        const df::F2 p = df::two_prod(kf, P.hr_f), z = df::two_sum(p.h, P.r_min_f);
+        const float e = __fadd_rn(__fadd_rn(__fsub_rn(z.h, rho), z.l), p.l);   // k hr + r_min - rho_k
+        const float s = __fmaf_rn(-kf, P.hr_s, __fmaf_rn(-e, P.idr_h, P.t0));
+        lo = __fadd_rn(__fadd_rn(lo, s), t.l);
+        hi = __fadd_rn(__fadd_rn(hi, s), t.l);
+    }
+    const float move = lo < 0.f ? -1.f : (hi >= 0.f ? 1.f : 0.f);
+    if (kf == 0.f && lo < 0.f) {   // below the first knot: the line that continues it
         atomicAdd(&flags->range_violations, 1ull);
         load_row_q(P, P.nk, p0, p1, v0, v1);
     } else if (move != 0.f && kf + move >= 0.f && kf + move <= last) {

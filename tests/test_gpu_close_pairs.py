@@ -101,3 +101,25 @@ def test_steps_with_close_pairs(walk, lanes):
         pos, vel = s.positions(), s.velocities()
     assert np.abs(pos - ref["pos"]).max() <= 4.0 * np.spacing(400.0)
     assert np.abs(vel - ref["vel"]).max() <= 100.0 * EPS * np.abs(ref["vel"]).max()
+
+
+@pytest.mark.parametrize("walk,lanes", WALKS)
+@pytest.mark.parametrize("n_knots,r_min", [(300, 1.3), (777, 1.7)])
+def test_pairs_beside_a_knot(n_knots, r_min, walk, lanes):
+    """Pairs between a knot and its FP32 value, which the row's interval must not be confused with: a
+    cubic beside its interval has another slope."""
+    w = dimers(1000.0, 1.0, False)
+    w.potential = pot = I.sc_cu_tables(n_knots=n_knots, r_min=r_min)
+    h = (pot.r_cut - r_min) / (n_knots - 1)
+    k = np.arange(1, n_knots)
+    knot = r_min + k * h
+    rounded = (k * float(np.float32(h)) + float(np.float32(r_min))).astype(np.float32).astype(np.float64)
+    pick = np.argsort(-np.abs(rounded - knot) * (knot < 3.0))[:40]   # the widest gaps
+    z = np.linspace(3.0, 990.0, len(pick))
+    a = np.stack([np.full(len(pick), 4.0), np.full(len(pick), 5.0), z], axis=1)
+    a = np.round(a * 2.0 ** 38) / 2.0 ** 38
+    b = a.copy()
+    b[:, 0] += np.round(0.5 * (knot + rounded)[pick] * 2.0 ** 38) / 2.0 ** 38
+    n = 2 * len(pick)
+    w.pos, w.vel, w.species = np.concatenate([a, b]), np.zeros((n, 3)), np.zeros(n, np.int32)
+    check_pair_forces(w, walk, lanes)
