@@ -318,6 +318,15 @@ md_status md_step(md_ctx *ctx, int32_t n_steps);
  * step boundary (positions have been drifted once); the next call recomputes forces. */
 md_status md_selftest_timeout(md_ctx *ctx);
 
+/* The same for the stand-alone list rebuild: a force evaluation that rebuilds, in which one block
+ * withholds its arrival at the given barrier of the rebuild (1 to 8: after the binning, the tile
+ * sums, their scan, the cell starts, the scatter, the cell sort, the gather, the copying back; 9, half
+ * list only: after the list build; 10: at the end).  The passes behind it read nothing and the call reports
+ * MD_ERR_TIMEOUT; no atom has moved, and the next call rebuilds.  Not for the contexts of the
+ * group walks (MD_PASSES_STAGED, CELLS, HALF at mixed precision), whose stand-alone rebuild has no
+ * barrier: MD_ERR_STATE. */
+md_status md_selftest_timeout_at(md_ctx *ctx, int32_t barrier);
+
 /* Graph mode (on = 1): md_step(n) records its device work for this n (the persistent
  * launch, the reduction, the copies back) as a CUDA graph the first time and replays the
  * graph afterwards.  Not used while profiling or under a strain ramp; on = 0 frees the

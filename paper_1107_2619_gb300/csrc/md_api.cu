@@ -65,6 +65,7 @@ struct md_ctx {
     int lanes = 1;
     int part_rows = 0;                   // rows of partial sums written by the last energy pass
     bool list_valid = false, forces_valid = false, energy_valid = false;
+    int withhold = 0;                    // md_selftest_timeout_at: the rebuild's barrier that runs out
     std::string err;
     // tracing
     int64_t launches = 0;
@@ -101,6 +102,7 @@ namespace {
 // one for the contexts with local rows.
 int rebuild_launches(const md_ctx *c, bool clear = true) { return c->C.tile ? 9 + (clear ? 1 : 0) : 1; }
 constexpr unsigned long long kSpinLimit = 20000000ull;  // barrier polls (~2 s) before giving up
+constexpr unsigned long long kSpinSelftest = 20000;     // of the self-tests: milliseconds
 
 md_status fail(md_ctx *c, md_status s, const std::string &what, cudaError_t e = cudaSuccess) {
     if (c) {
@@ -233,14 +235,33 @@ void cubic_rows(const double *tab, int nk, double h, double4_32a *out64) {
     }
 }
 
+// After a bounded wait gave up (the stream is idle, the flags are in h_flags): what a launch that left
+// early may have left unfinished, so that the next call starts over from whole arrays.  The list counts
+// as missing, the atoms are all renumbered or none is, and sums that later calls add to are empty.
+// The state is not a clean step boundary where the launch was advancing it.
+md_status recover_timeout(md_ctx *ctx) {
+    ctx->list_valid = ctx->forces_valid = ctx->energy_valid = false;
+    const Atoms &A = ctx->A;
+    const size_t n = (size_t)ctx->n;
+    if (ctx->h_flags->renumber) {
+        MD_CK(launch_copyback(A, ctx->stream));
+        MD_CK(cudaMemsetAsync(&ctx->d_flags->renumber, 0, sizeof(int32_t), ctx->stream));
+        ctx->launches++;
+    }
+    MD_CK(cudaMemsetAsync(ctx->C.cell_count, 0, sizeof(int32_t) * ctx->C.ncell, ctx->stream));
+    if (A.rho_acc) MD_CK(cudaMemsetAsync(A.rho_acc, 0, sizeof(double) * n, ctx->stream));
+    if (A.e_acc) MD_CK(cudaMemsetAsync(A.e_acc, 0, sizeof(double) * n, ctx->stream));
+    if (ctx->d_thermo)
+        MD_CK(cudaMemset2DAsync(&ctx->d_thermo->ke_fix, sizeof(Thermo), 0, sizeof(ctx->d_thermo->ke_fix), ctx->n_rep,
+                                ctx->stream));
+    return fail(ctx, MD_ERR_TIMEOUT, "a bounded device-side wait gave up");
+}
+
 md_status sync_and_check(md_ctx *ctx, bool strict_skin) {
     MD_CK(cudaMemcpyAsync(ctx->h_flags, ctx->d_flags, sizeof(Flags), cudaMemcpyDeviceToHost, ctx->stream));
     MD_CK(cudaStreamSynchronize(ctx->stream));
     const Flags &f = *ctx->h_flags;
-    if (f.error & FLAG_TIMEOUT) {
-        ctx->forces_valid = ctx->energy_valid = false;
-        return fail(ctx, MD_ERR_TIMEOUT, "a grid barrier of the step kernel gave up waiting");
-    }
+    if (f.error & FLAG_TIMEOUT) return recover_timeout(ctx);
     if (f.error & FLAG_OVERFLOW) {
         ctx->list_valid = false;
         return fail(ctx, MD_ERR_NBR_OVERFLOW,
@@ -401,7 +422,8 @@ StepParams step_params(md_ctx *ctx, int n_steps) {
     if (ctx->thermo_on) {
         sp.thermo = ctx->d_thermo;
     }
-    sp.spin_limit = kSpinLimit;
+    sp.withhold_rebuild = ctx->withhold;
+    sp.spin_limit = ctx->withhold ? kSpinSelftest : kSpinLimit;
     sp.motion = ctx->cfg.integrator == MD_INTEGRATOR_PC3 ? kMotionPC3 : kMotionVerlet;
     return sp;
 }
@@ -1817,7 +1839,7 @@ md_status md_selftest_timeout(md_ctx *ctx) {
     }
     StepParams sp = step_params(ctx, 1);
     sp.thermo = nullptr;
-    sp.spin_limit = 20000;  // ~2-5 ms of polling
+    sp.spin_limit = kSpinSelftest;
     // a step kernel that stages cell groups (and fits them: no fallback to the list walk) tests
     // its staging pipeline's waits instead of the grid barrier's
     const int walk = step_walk(ctx->A, ctx->C, ctx->P, ctx->precision, ctx->lanes);
@@ -1832,6 +1854,18 @@ md_status md_selftest_timeout(md_ctx *ctx) {
     md_status st = sync_and_check(ctx, false);
     // the state is no longer a clean step boundary: recompute before the next step
     ctx->forces_valid = ctx->energy_valid = false;
+    return st;
+}
+
+md_status md_selftest_timeout_at(md_ctx *ctx, int32_t barrier) {
+    if (!ctx || ctx->n == 0) return MD_ERR_ARG;
+    if (ctx->C.tile) return fail(ctx, MD_ERR_STATE, "this context's stand-alone rebuild has no grid barrier");
+    if (barrier < 1 || barrier > 10 || (barrier == 9 && !ctx->A.pairs))
+        return fail(ctx, MD_ERR_ARG, "no such barrier in the rebuild");
+    ctx->list_valid = false;
+    ctx->withhold = barrier;
+    md_status st = compute_forces(ctx);
+    ctx->withhold = 0;
     return st;
 }
 

@@ -10,12 +10,13 @@ namespace {
 
 template <int T, int KIND, bool MULTI>
 __global__ void __launch_bounds__(kThreads) k_density32(Atoms A, Pot P) {
-    eam::clear_rebuild_once(A.flags);
+    if (!eam::begin_density(A.flags)) return;
     ps::density32_item<T, KIND, MULTI>(A, P, A.boxes, (long long)blockIdx.x * kThreads + threadIdx.x);
 }
 
 template <int T, int KIND, bool MULTI, bool ENERGY>
 __global__ void __launch_bounds__(kThreads) k_force32(Atoms A, Pot P, double half_dt, int kick) {
+    if (eam::timed_out(A.flags)) return;
     double part[kPartials];
 #pragma unroll
     for (int q = 0; q < kPartials; q++) part[q] = 0.0;

@@ -19,12 +19,13 @@ namespace {
 
 template <int T, int KIND, bool MULTI>
 __global__ void __launch_bounds__(kThreads) k_density64(Atoms A, Pot P) {
-    clear_rebuild_once(A.flags);
+    if (!begin_density(A.flags)) return;
     ps::density64_item<T, KIND, MULTI>(A, P, A.boxes, (long long)blockIdx.x * kThreads + threadIdx.x, true);
 }
 
 template <int T, int KIND, bool MULTI, bool ENERGY>
 __global__ void __launch_bounds__(kThreads) k_force64(Atoms A, Pot P, double half_dt, int kick) {
+    if (timed_out(A.flags)) return;
     double part[kPartials];
 #pragma unroll
     for (int q = 0; q < kPartials; q++) part[q] = 0.0;
@@ -37,18 +38,20 @@ __global__ void __launch_bounds__(kThreads) k_force64(Atoms A, Pot P, double hal
 template <int T, int KIND>
 __global__ void __launch_bounds__(kThreads) k_density64_pairs(Atoms A, Pot P) {
     __shared__ __align__(16) double sums[T >= ps::kFlatLanes ? kThreads / 32 * ps::kPairSlots(32 / T) : 1];
-    clear_rebuild_once(A.flags);
+    if (!begin_density(A.flags)) return;
     ps::density64_pairs<T, KIND>(A, P, A.boxes, (long long)blockIdx.x * kThreads + threadIdx.x, true,
                                  sums + (T >= ps::kFlatLanes ? (threadIdx.x >> 5) * ps::kPairSlots(32 / T) : 0));
 }
 
 __global__ void __launch_bounds__(kThreads) k_embed64_pairs(Atoms A, Pot P) {
+    if (timed_out(A.flags)) return;
     const int i = blockIdx.x * kThreads + threadIdx.x;
     if (i < A.n) ps::pairs_embed64<true>(A, P, i);
 }
 
 template <int T, int KIND, bool ENERGY>
 __global__ void __launch_bounds__(kThreads) k_force64_pairs(Atoms A, Pot P) {
+    if (timed_out(A.flags)) return;
     double part[kPartials];
 #pragma unroll
     for (int q = 0; q < kPartials; q++) part[q] = 0.0;
@@ -62,6 +65,7 @@ __global__ void __launch_bounds__(kThreads) k_force64_pairs(Atoms A, Pot P) {
 // force pass's (virial) rows, and the reduction adds both sets.
 template <bool ENERGY>
 __global__ void __launch_bounds__(kThreads) k_finish64_pairs(Atoms A, double half_dt, int kick, int row0) {
+    if (timed_out(A.flags)) return;
     double part[kPartials];
 #pragma unroll
     for (int q = 0; q < kPartials; q++) part[q] = 0.0;

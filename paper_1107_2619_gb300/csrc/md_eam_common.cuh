@@ -277,11 +277,19 @@ __device__ __forceinline__ void block_partials(double (&v)[kPartials], double *o
     }
 }
 
-__device__ __forceinline__ void clear_rebuild_once(Flags *f) {
+// Whether a bounded wait of this call gave up.  The list may then be half built, or not at all: the
+// kernels behind the stand-alone rebuild read no row and move no atom.
+__device__ __forceinline__ bool timed_out(const Flags *f) {
+    return (*reinterpret_cast<const volatile int32_t *>(&f->error) & FLAG_TIMEOUT) != 0;
+}
+// The start of a stand-alone density pass: the rebuild request cleared, unless the rebuild gave up.
+__device__ __forceinline__ bool begin_density(Flags *f) {
+    if (timed_out(f)) return false;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (f->need_rebuild) f->n_rebuilds++;
         f->need_rebuild = 0;
     }
+    return true;
 }
 
 // Second half kick v += (dt/2 * f) * (acc/m) with the separately rounded operations of the

@@ -12,12 +12,13 @@ namespace {
 
 template <int T>
 __global__ void __launch_bounds__(kThreads) k_density_df(Atoms A, Pot P) {
-    clear_rebuild_once(A.flags);
+    if (!begin_density(A.flags)) return;
     ps::density_df_item<T>(A, P, A.boxes, (long long)blockIdx.x * kThreads + threadIdx.x, true);
 }
 
 template <int T, bool ENERGY>
 __global__ void __launch_bounds__(kThreads) k_force_df(Atoms A, Pot P, double half_dt, int kick) {
+    if (timed_out(A.flags)) return;
     double part[kPartials];
 #pragma unroll
     for (int q = 0; q < kPartials; q++) part[q] = 0.0;

@@ -48,6 +48,7 @@ struct Flags {
     int32_t error;          // FLAG_* bits (this word and the next are cleared at the start of every call)
     int32_t skin_exceeded;  // an atom moved more than skin/2 since the last build
     int32_t close_pairs;    // a density pass since the last build met a close pair (ps::kCloseR2)
+    int32_t renumber;       // a rebuild is copying the renumbered atoms back (left set by one that gave up there)
     int32_t need_rebuild;   // set by the displacement check or the schedule; cleared by pass 1
     int32_t max_count;      // longest list at the last build
     unsigned long long n_rebuilds;
@@ -326,6 +327,8 @@ cudaError_t launch_set_rebuild(Flags *f, cudaStream_t s);
 cudaError_t launch_clear_rebuild(Flags *f, cudaStream_t s);
 cudaError_t launch_rebuild(const Atoms &A, const Cells &C, double rl2, float band_lo, float band_hi,
                            int list_group, cudaStream_t s);
+// What a rebuild that gave up while copying back (Flags::renumber) left undone.
+cudaError_t launch_copyback(const Atoms &A, cudaStream_t s);
 cudaError_t launch_check_displacement(const Atoms &A, SkinLimit lim, cudaStream_t s);
 cudaError_t launch_wrap(const Atoms &A, cudaStream_t s);
 // lanes = T lanes per atom (1, 2, 4, 8, 16 or 32)
@@ -371,6 +374,7 @@ struct StepParams {
     unsigned long long spin_limit;
     int withhold_arrival;  // self-test of the bounded waits: 1, block 0 skips its first grid-barrier
                            // arrival; 2 (group walks), block 0's staging producer releases no group
+    int withhold_rebuild;  // self-test: block 0 skips this grid-barrier arrival of a rebuild (0: none)
     int motion;            // kMotionVerlet or kMotionPC3: what the force pass does to each atom after
                            // its force (second half kick, or the corrector) and what opens a step
                            // (half kick + drift, or the predictor)

@@ -139,6 +139,11 @@ cudaError_t launch_clear_rebuild(Flags *f, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+cudaError_t launch_copyback(const Atoms &A, cudaStream_t s) {
+    if (A.n > 0) k_copyback<<<capped_blocks(A.n, kThreads), kThreads, 0, s>>>(A);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_rebuild(const Atoms &A, const Cells &C, double rl2, float band_lo, float band_hi,
                            int list_group, cudaStream_t s) {
     const int nb = capped_blocks(A.n, kThreads);

@@ -113,6 +113,17 @@ __device__ __forceinline__ bool grid_sync(GridBarrier *b, unsigned nblocks, unsi
     return grid_sync(b, nblocks, limit, f, nullptr);
 }
 
+// Self-test of the bounded wait, in place of grid_sync: this block never arrives; it waits (bounded)
+// until the others have given up and marked the launch aborted, then leaves.
+__device__ __forceinline__ void withhold_arrival(GridBarrier *b, unsigned long long limit, Flags *f) {
+    if (threadIdx.x == 0) {
+        unsigned long long polls = 0;
+        while (!*reinterpret_cast<volatile int *>(&b->abort) && ++polls < 4 * limit) __nanosleep(100);
+        if (gridDim.x == 1) atomicOr(&f->error, FLAG_TIMEOUT);  // nobody else to give up
+    }
+    __syncthreads();
+}
+
 // Box matrix times the strain matrix diag(1, 1, s) (§2.2), every replica.
 __device__ __forceinline__ void strain_boxes(Box *boxes, int n_rep, double s, int qfb) {
     for (int r = 0; r < n_rep; r++) {
@@ -206,19 +217,23 @@ __device__ __forceinline__ bool rebuild_phases(const Atoms &A, const Cells &C, B
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long stride = (long long)nb * blockDim.x;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
-#define RB_SYNC()                                                   \
-    do {                                                            \
-        if (!grid_sync(bar, nb, sp.spin_limit, A.flags)) return false; \
+#define RB_SYNC(q)                                                      \
+    do {                                                                \
+        if (sp.withhold_rebuild == (q) && blockIdx.x == 0) {            \
+            withhold_arrival(bar, sp.spin_limit, A.flags);              \
+            return false;                                               \
+        }                                                               \
+        if (!grid_sync(bar, nb, sp.spin_limit, A.flags)) return false;  \
     } while (0)
 #define MD_STAMP(q) \
     if (srow) srow[q] = globaltimer()
 
     for (long long i = tid; i < A.n; i += stride) ph::bin_atom(A, C, boxes, (int)i);
-    RB_SYNC();
+    RB_SYNC(1);
     MD_STAMP(1);
     const int ntiles = ph::scan_tiles(C);
     for (int t = blockIdx.x; t < ntiles; t += nb) ph::scan_tile_sum(C, t, ws);
-    RB_SYNC();
+    RB_SYNC(2);
     MD_STAMP(2);
     if (blockIdx.x == 0) {
         if (threadIdx.x == 0) {
@@ -229,10 +244,10 @@ __device__ __forceinline__ bool rebuild_phases(const Atoms &A, const Cells &C, B
         }
         ph::scan_top(C, ws);
     }
-    RB_SYNC();
+    RB_SYNC(3);
     MD_STAMP(3);
     for (int t = blockIdx.x; t < ntiles; t += nb) ph::scan_apply(C, t, ws);
-    RB_SYNC();
+    RB_SYNC(4);
     MD_STAMP(4);
     for (long long i = tid; i < A.n; i += stride) ph::scatter_atom(A, C, (int)i);
     if constexpr (kGroupWalk<WALK>) {
@@ -240,16 +255,18 @@ __device__ __forceinline__ bool rebuild_phases(const Atoms &A, const Cells &C, B
     } else {
         if (C.tile && lead) A.flags->tile_bad = 1;   // this build writes no local lists
     }
-    RB_SYNC();
+    RB_SYNC(5);
     MD_STAMP(5);
     for (long long c = tid >> 5; c < C.ncell; c += stride >> 5) ph::sort_cell_warp(A, C, (int)c, threadIdx.x & 31);
-    RB_SYNC();
+    RB_SYNC(6);
     MD_STAMP(6);
     for (long long k = tid; k < A.n; k += stride) ph::gather_atom(A, (int)k);
-    RB_SYNC();
+    RB_SYNC(7);
     MD_STAMP(7);
+    if (threadIdx.x == 0) A.flags->renumber = 1;   // until all are through (launch_copyback)
     for (long long k = tid; k < A.n; k += stride) ph::copyback_atom(A, boxes, (int)k);
-    RB_SYNC();
+    RB_SYNC(8);
+    if (lead) A.flags->renumber = 0;
     MD_STAMP(8);
     // the group walks need the global rows only when some group does not fit its stage
     const bool rows = !kGroupWalk<WALK> || *reinterpret_cast<volatile int32_t *>(&A.flags->tile_bad);
@@ -265,10 +282,10 @@ __device__ __forceinline__ bool rebuild_phases(const Atoms &A, const Cells &C, B
         if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(&A.flags->max_count, m);
     }
     if constexpr (WALK == kWalkPairs) {   // each row's entries j > i first
-        RB_SYNC();
+        RB_SYNC(9);
         for (long long i = tid >> 5; i < A.n; i += stride >> 5) ph::partition_row_warp(A, (int)i, threadIdx.x & 31);
     }
-    RB_SYNC();
+    RB_SYNC(10);
     MD_STAMP(9);
     return true;
 #undef MD_STAMP
@@ -308,10 +325,11 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
     const unsigned nb = gridDim.x;
     const long long tid = (long long)blockIdx.x * NT + threadIdx.x;
     const long long stride = (long long)nb * NT;
+    if (eam::timed_out(A.flags)) return;   // (a launch before this one, or the rebuild of its forces)
     int s0 = 0;
     if (sp.resume) {   // the step was opened by the launch that stopped at its rebuild request
         s0 = *reinterpret_cast<volatile int32_t *>(&A.flags->seg_done);
-        if (s0 >= sp.n_steps || (*reinterpret_cast<volatile int32_t *>(&A.flags->error) & FLAG_TIMEOUT)) return;
+        if (s0 >= sp.n_steps) return;
     }
     if (SMT && !kSplitTable) {
         const float4 *src = reinterpret_cast<const float4 *>(P.VP32);
@@ -364,14 +382,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads ? (PREC == MD_PREC_DF      
             if constexpr (WALK == kWalkHalf) A.rho_acc[i] = 0.0;
         }
         if (sp.withhold_arrival == 1 && blockIdx.x == 0) {
-            // self-test of the bounded wait: this block never arrives; it waits (bounded) until
-            // the others have given up and marked the launch aborted, then leaves.
-            if (threadIdx.x == 0) {
-                unsigned long long polls = 0;
-                while (!*reinterpret_cast<volatile int *>(&bar->abort) && ++polls < 4 * sp.spin_limit) __nanosleep(100);
-                if (gridDim.x == 1) atomicOr(&A.flags->error, FLAG_TIMEOUT);  // nobody else to give up
-            }
-            __syncthreads();
+            withhold_arrival(bar, sp.spin_limit, A.flags);
             return;
         }
         MD_SYNC();
@@ -694,9 +705,7 @@ __global__ void __launch_bounds__(kRebuildThreads, MD_REBUILD_MIN_BLOCKS)
     __shared__ int ws[32];
     // every block reads the same words, written before this launch: all take part or none
     const int s = *reinterpret_cast<volatile int32_t *>(&A.flags->seg_done);
-    if (s >= sp.n_steps || !ph::rebuild_requested(A.flags) ||
-        (*reinterpret_cast<volatile int32_t *>(&A.flags->error) & FLAG_TIMEOUT))
-        return;
+    if (s >= sp.n_steps || !ph::rebuild_requested(A.flags) || eam::timed_out(A.flags)) return;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     unsigned long long *srow = stamps && lead ? stamps + kStampsPerStep * (s + 1) : nullptr;
     if (!rebuild_phases<WALK>(A, C, A.boxes, sp, bar, ws, srow)) return;

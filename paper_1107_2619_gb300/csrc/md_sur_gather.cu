@@ -132,6 +132,7 @@ __device__ __forceinline__ void block_range(int a0, int a1, int &b0, int &b1) {
 // x = (G - gmu) ginv rounded to bf16 in the 128-atom tile layout the MMA reads (S.Gt):
 // tile t = i / 128, row r = i % 128, column k at byte t*8192 + (r/8)*512 + (k/8)*128 + (r%8)*16 + (k%8)*2.
 __global__ void __launch_bounds__(kThreads) k_sur_desc(Atoms A, SurNet S, int a0, int a1, int bf16) {
+    if (eam::timed_out(A.flags)) return;
     __shared__ Stage<2> stage[kWarps];   // r, fc
     __shared__ __align__(16) __nv_bfloat16 out[kWarps][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -196,6 +197,7 @@ __global__ void __launch_bounds__(kThreads) k_sur_desc(Atoms A, SurNet S, int a0
 template <bool ENERGY, bool TRAIN>
 __global__ void __launch_bounds__(kThreads, 8) k_sur_force(Atoms A, SurNet S, int a0, int a1, int kick, double half_dt,
                                                            float phi_scale) {
+    if (eam::timed_out(A.flags)) return;
     constexpr bool VIRIAL = ENERGY && !TRAIN;
     __shared__ float4 P0[kWarps][32], P1[kWarps][32];   // (r, fc', -fc/w^2, u_x), (u_y, u_z, j bits, 0)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -416,6 +418,7 @@ __global__ void k_sur_stats(Atoms A, SurNet S, double *part) {
 }
 
 __global__ void k_sur_kick_drift(Atoms A, double half_dt, double dt, SkinLimit lim) {
+    if (eam::timed_out(A.flags)) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= A.n) return;
     ph::kick_drift(A, A.boxes, i, half_dt, dt, 1.0, false, lim);

@@ -35,6 +35,7 @@ PRECISIONS = {"fp64": MD_PREC_FP64, "mixed": MD_PREC_MIXED, "df": MD_PREC_DF}
 EXPORTS = ["md_abi_version", "md_status_string", "md_create", "md_create_batch", "md_build_neighbours",
            "md_eam_forces", "md_step", "md_step_io", "md_set_graph", "md_energy", "md_replica_energies", "md_get",
            "md_set_state", "md_tune", "md_set_profiling", "md_get_profile", "md_get_passes", "md_selftest_timeout",
+           "md_selftest_timeout_at",
            "md_neighbours_noalloc", "md_set_thermostat", "md_get_thermostat", "md_set_surrogate", "md_sur_get_params", "md_sur_standardize",
            "md_sur_get", "md_sur_set_reference", "md_sur_loss_grad", "md_sur_train", "md_measure_fp64_peak",
            "md_last_error", "md_destroy"]
@@ -120,6 +121,8 @@ def lib():
         L.md_replica_energies.argtypes = [P, C.POINTER(md_energies)]
         L.md_selftest_timeout.restype = C.c_int
         L.md_selftest_timeout.argtypes = [P]
+        L.md_selftest_timeout_at.restype = C.c_int
+        L.md_selftest_timeout_at.argtypes = [P, C.c_int32]
         L.md_set_graph.restype = C.c_int
         L.md_set_graph.argtypes = [P, i32]
         L.md_build_neighbours.restype = C.c_int
@@ -239,6 +242,11 @@ def md_replica_energies(ctx, n_replicas: int) -> list:
 def md_selftest_timeout(ctx) -> int:
     """Run the bounded-wait self-test; returns the md_status (MD_ERR_TIMEOUT expected)."""
     return lib().md_selftest_timeout(ctx)
+
+
+def md_selftest_timeout_at(ctx, barrier: int) -> int:
+    """The self-test of one barrier of the stand-alone rebuild (md.h); returns the md_status."""
+    return lib().md_selftest_timeout_at(ctx, barrier)
 
 
 def md_set_graph(ctx, on: bool):
