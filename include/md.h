@@ -324,7 +324,8 @@ md_status md_selftest_timeout(md_ctx *ctx);
  * list only: after the list build; 10: at the end).  The passes behind it read nothing and the call reports
  * MD_ERR_TIMEOUT; no atom has moved, and the next call rebuilds.  Not for the contexts of the
  * group walks (MD_PASSES_STAGED, CELLS, HALF at mixed precision), whose stand-alone rebuild has no
- * barrier: MD_ERR_STATE. */
+ * barrier: MD_ERR_STATE.  11: md_tune, its first trial step timing out; the state and the lane
+ * count stay. */
 md_status md_selftest_timeout_at(md_ctx *ctx, int32_t barrier);
 
 /* Graph mode (on = 1): md_step(n) records its device work for this n (the persistent
@@ -363,7 +364,8 @@ md_status md_step_io(md_ctx *ctx, int32_t n_steps, const double *pos_in, const d
  * with each lanes_per_atom in {1, 2, 4, 8, 16, 32} (CUDA events; the trial steps rebuild no
  * list, and positions, velocities, forces and counters are put back after each), keep the
  * fastest for this context and return it in *lanes_out (nullable).  Computes the forces first
- * if needed.  Because the lane count fixes the summation order, results after md_tune are
+ * if needed.  A trial whose bounded wait gives up ends it: MD_ERR_TIMEOUT, the lane count kept.
+ * Because the lane count fixes the summation order, results after md_tune are
  * reproducible but may differ in the last bits from those before it. */
 md_status md_tune(md_ctx *ctx, int32_t *lanes_out);
 

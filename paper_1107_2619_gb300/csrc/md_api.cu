@@ -65,7 +65,7 @@ struct md_ctx {
     int lanes = 1;
     int part_rows = 0;                   // rows of partial sums written by the last energy pass
     bool list_valid = false, forces_valid = false, energy_valid = false;
-    int withhold = 0;                    // md_selftest_timeout_at: the rebuild's barrier that runs out
+    int withhold = 0;                    // md_selftest_timeout_at: the barrier that runs out
     std::string err;
     // tracing
     int64_t launches = 0;
@@ -103,6 +103,7 @@ namespace {
 int rebuild_launches(const md_ctx *c, bool clear = true) { return c->C.tile ? 9 + (clear ? 1 : 0) : 1; }
 constexpr unsigned long long kSpinLimit = 20000000ull;  // barrier polls (~2 s) before giving up
 constexpr unsigned long long kSpinSelftest = 20000;     // of the self-tests: milliseconds
+constexpr int kWithholdTune = 11;                       // md_selftest_timeout_at: md_tune's trial steps
 
 md_status fail(md_ctx *c, md_status s, const std::string &what, cudaError_t e = cudaSuccess) {
     if (c) {
@@ -1785,23 +1786,31 @@ md_status md_tune(md_ctx *ctx, int32_t *lanes_out) {
         sp.strain_scale = 1.0;
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         cudaError_t e = reset_errors(ctx);
+        bool gave_up = false;
         if (e == cudaSuccess) e = copy(true);
         if (e == cudaSuccess) e = cudaEventCreate(&e0);
         if (e == cudaSuccess) e = cudaEventCreate(&e1);
         float best = 1e30f;
         int best_t = ctx->lanes;
-        for (int t = 1; t <= 32 && e == cudaSuccess; t *= 2) {
-            for (int rep = 0; rep < 3 && e == cudaSuccess; rep++) {  // first round is a warm-up
+        for (int t = 1; t <= 32 && e == cudaSuccess && !gave_up; t *= 2) {
+            for (int rep = 0; rep < 3 && e == cudaSuccess && !gave_up; rep++) {  // first round is a warm-up
                 int grid = 0;
                 StepParams prep = sp;
                 prep.n_steps = 0;  // attributes and occupancy before the timed launch
                 e = launch_step(A, ctx->C, ctx->P, ctx->precision, t, prep, ctx->d_bar, nullptr, &grid, ctx->stream);
+                sp.withhold_arrival = ctx->withhold == kWithholdTune ? 1 : 0;
+                if (e == cudaSuccess) e = reset_errors(ctx);
                 if (e == cudaSuccess) e = cudaEventRecord(e0, ctx->stream);
                 if (e == cudaSuccess)
                     e = launch_step(A, ctx->C, ctx->P, ctx->precision, t, sp, ctx->d_bar, nullptr, &grid, ctx->stream);
                 if (e == cudaSuccess) e = cudaEventRecord(e1, ctx->stream);
+                if (e == cudaSuccess)
+                    e = cudaMemcpyAsync(ctx->h_flags, ctx->d_flags, sizeof(Flags), cudaMemcpyDeviceToHost, ctx->stream);
                 if (e == cudaSuccess) e = copy(false);
-                if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+                if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+                // (a trial that gave up took no step: its time means nothing)
+                gave_up = e == cudaSuccess && (ctx->h_flags->error & FLAG_TIMEOUT);
+                if (gave_up) break;
                 float ms = 0.f;
                 if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
                 if (e == cudaSuccess && rep > 0 && ms < best) {
@@ -1820,6 +1829,7 @@ md_status md_tune(md_ctx *ctx, int32_t *lanes_out) {
             ctx->forces_valid = ctx->energy_valid = false;
             return fail(ctx, MD_ERR_CUDA, "md_tune trial steps", e);
         }
+        if (gave_up) return recover_timeout(ctx);   // the lane count stays
         if (best_t != ctx->lanes) drop_graphs(ctx);
         ctx->lanes = best_t;
         ctx->energy_valid = false;  // the per-atom energies are those of a trial step
@@ -1859,6 +1869,15 @@ md_status md_selftest_timeout(md_ctx *ctx) {
 
 md_status md_selftest_timeout_at(md_ctx *ctx, int32_t barrier) {
     if (!ctx || ctx->n == 0) return MD_ERR_ARG;
+    if (barrier == kWithholdTune) {
+        if (ctx->sur) return fail(ctx, MD_ERR_STATE, "a surrogate has no trial steps");
+        md_status st = ctx->forces_valid ? MD_OK : compute_forces(ctx);
+        if (st != MD_OK) return st;
+        ctx->withhold = barrier;
+        st = md_tune(ctx, nullptr);
+        ctx->withhold = 0;
+        return st;
+    }
     if (ctx->C.tile) return fail(ctx, MD_ERR_STATE, "this context's stand-alone rebuild has no grid barrier");
     if (barrier < 1 || barrier > 10 || (barrier == 9 && !ctx->A.pairs))
         return fail(ctx, MD_ERR_ARG, "no such barrier in the rebuild");

@@ -73,3 +73,19 @@ def test_contexts_without_a_barrier_say_so():
         assert md.md_selftest_timeout_at(s.ctx, 1) == 11   # wrong state
     with make("fp64-list") as s:
         assert md.md_selftest_timeout_at(s.ctx, 9) == md.md_selftest_timeout_at(s.ctx, 0) == 1   # bad argument
+
+
+@pytest.mark.parametrize("kind", ["fp64-half", "mixed-list"])
+def test_tuning_reports_a_trial_that_gave_up(kind):
+    """A trial step that gives up would otherwise be the fastest of all."""
+    f0, _, _ = fresh(kind)
+    tol = 1e-11 if kind.startswith("fp64") else 1e-5
+    with make(kind) as s:
+        s.eam_forces()
+        before = s.positions(), s.velocities()
+        assert md.md_selftest_timeout_at(s.ctx, 11) == md.MD_ERR_TIMEOUT
+        assert np.array_equal(s.positions(), before[0]) and np.array_equal(s.velocities(), before[1])
+        s.eam_forces()
+        assert np.abs(s.forces() - f0).max() <= tol * np.abs(f0).max()
+        assert s.tune() in (1, 2, 4, 8, 16, 32)
+        s.step(1)
