@@ -1145,6 +1145,7 @@ bool fetch(void *dst, const void *src, size_t bytes, int on_device) {
 // --------------------------------------------------------------------------- surrogate
 md_status sur_alloc(md_ctx *ctx) {
     if (ctx->d_theta) return MD_OK;
+    MD_CK(sur_gather_grids(ctx->S));
     const int64_t n = std::max<int64_t>(ctx->n, 1);
     const int64_t ntiles = (n + kSurTile - 1) / kSurTile;
     SurNet &S = ctx->S;

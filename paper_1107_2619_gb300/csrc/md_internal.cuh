@@ -411,7 +411,12 @@ constexpr int kSurTileBytes = kSurTile * kSurNb * 2;  // bf16 descriptor tile, c
 // K-major core-matrix layout: W1 (64 x 32), W2 (64 x 64), W2^T (64 x 64), W1^T (32 x 64)
 constexpr int kSurImgW1 = 0, kSurImgW2 = 4096, kSurImgW2T = 12288, kSurImgW1T = 20480, kSurImgBytes = 24576;
 
+// The gather kernels (md_sur_gather.cu): descriptors, forces, forces with energies, forces of a training
+// pass, descriptor tangents.
+enum { kGatherDesc, kGatherForce, kGatherEnergy, kGatherTrain, kGatherU, kGathers };
+
 struct SurNet {
+    int gather[kGathers];     // blocks of each gather kernel that stay resident on the context's device at once
     float mu0, dmu, inv2w2, invw2, rd, rd2, pi_rd;
     int bf16;                 // 1: tensor-core BF16 network, 0: FP32 network
     const float *theta;       // [kSurParams] parameters (FP32 master)
@@ -428,6 +433,8 @@ struct SurNet {
     float *gpart;             // training: per-block parameter gradients [blocks][kSurParams]
 };
 
+// Fills SurNet::gather for the current device.
+cudaError_t sur_gather_grids(SurNet &S);
 // Surrogate launchers (md_sur_*.cu).  Atom ranges [a0, a1) are contiguous replicas.
 cudaError_t launch_sur_kick_drift(const Atoms &A, double half_dt, double dt, SkinLimit lim, cudaStream_t s);
 cudaError_t launch_sur_descriptors(const Atoms &A, const SurNet &S, int a0, int a1, cudaStream_t s);

@@ -432,25 +432,24 @@ __global__ void k_sur_unsort_rows(Atoms A, const float *src, float *dst) {
     dst[(size_t)A.id[i] * kSurNb + k] = src[t];
 }
 
-// Blocks of a gather: as many as stay resident at once (blocks_per_sm of this kernel, fewer for few
-// atoms), so that each warp has the most atoms to finish together; at most one block per kWarps atoms.
-template <auto Kernel>
-int gather_blocks(int n_atoms) {
-    static int resident = 0;
-    if (!resident) {
-        int dev = 0, n_sm = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kernel, kThreads, 0);
-        resident = std::min(8192, std::max(1, n_sm * per_sm));
-    }
-    return std::max(1, std::min(blocks_for(n_atoms, kWarps), resident));
+// Blocks of a gather: as many as stay resident at once (SurNet::gather, fewer for few atoms), so that
+// each warp has the most atoms to finish together; at most one block per kWarps atoms.
+int gather_blocks(const SurNet &S, int kernel, int n_atoms) {
+    return std::max(1, std::min(blocks_for(n_atoms, kWarps), S.gather[kernel]));
+}
+cudaError_t resident_blocks(const void *kernel, int n_sm, int &out) {
+    int per_sm = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1 || n_sm < 1) return cudaErrorInvalidConfiguration;
+    out = std::min(8192, n_sm * per_sm);
+    return cudaSuccess;
 }
 
 template <bool ENERGY, bool TRAIN>
 cudaError_t force_t(const Atoms &A, const SurNet &S, int a0, int a1, int kick, double half_dt, float phi_scale,
                     int *rows_out, cudaStream_t s) {
-    const int nb = gather_blocks<k_sur_force<ENERGY, TRAIN>>(a1 - a0);
+    const int nb = gather_blocks(S, TRAIN ? kGatherTrain : (ENERGY ? kGatherEnergy : kGatherForce), a1 - a0);
     if (rows_out) *rows_out = nb;
     if (a1 <= a0) return cudaSuccess;
     k_sur_force<ENERGY, TRAIN><<<nb, kThreads, 0, s>>>(A, S, a0, a1, kick, half_dt, phi_scale);
@@ -458,6 +457,18 @@ cudaError_t force_t(const Atoms &A, const SurNet &S, int a0, int a1, int kick, d
 }
 
 }  // namespace
+
+cudaError_t sur_gather_grids(SurNet &S) {
+    int dev = 0, n_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = resident_blocks((const void *)k_sur_desc, n_sm, S.gather[kGatherDesc]);
+    if (e == cudaSuccess) e = resident_blocks((const void *)k_sur_force<false, false>, n_sm, S.gather[kGatherForce]);
+    if (e == cudaSuccess) e = resident_blocks((const void *)k_sur_force<true, false>, n_sm, S.gather[kGatherEnergy]);
+    if (e == cudaSuccess) e = resident_blocks((const void *)k_sur_force<true, true>, n_sm, S.gather[kGatherTrain]);
+    if (e == cudaSuccess) e = resident_blocks((const void *)k_sur_u, n_sm, S.gather[kGatherU]);
+    return e;
+}
 
 cudaError_t launch_sur_kick_drift(const Atoms &A, double half_dt, double dt, SkinLimit lim, cudaStream_t s) {
     if (A.n == 0) return cudaSuccess;
@@ -467,7 +478,7 @@ cudaError_t launch_sur_kick_drift(const Atoms &A, double half_dt, double dt, Ski
 
 cudaError_t launch_sur_descriptors(const Atoms &A, const SurNet &S, int a0, int a1, cudaStream_t s) {
     if (a1 <= a0) return cudaSuccess;
-    k_sur_desc<<<gather_blocks<k_sur_desc>(a1 - a0), kThreads, 0, s>>>(A, S, a0, a1, S.bf16);
+    k_sur_desc<<<gather_blocks(S, kGatherDesc, a1 - a0), kThreads, 0, s>>>(A, S, a0, a1, S.bf16);
     return cudaGetLastError();
 }
 
@@ -480,7 +491,7 @@ cudaError_t launch_sur_force(const Atoms &A, const SurNet &S, int a0, int a1, bo
 
 cudaError_t launch_sur_u(const Atoms &A, const SurNet &S, int a0, int a1, cudaStream_t s) {
     if (a1 <= a0) return cudaSuccess;
-    k_sur_u<<<gather_blocks<k_sur_u>(a1 - a0), kThreads, 0, s>>>(A, S, a0, a1);
+    k_sur_u<<<gather_blocks(S, kGatherU, a1 - a0), kThreads, 0, s>>>(A, S, a0, a1);
     return cudaGetLastError();
 }
 
