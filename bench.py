@@ -65,23 +65,45 @@ def _peaks():
         return 6800.0, "fallback (6.8 TB/s)"
 
 
-# FP64 operations per list entry of the FP64 passes when every pair term is FP64 arithmetic (an add
-# or a multiply is 1 flop, an FMA 2; conversions and rounding to integer not counted): the work at
-# FP64 accuracy, of which the passes do most on the FP32 and integer pipes.  Entries
-# inside r_cut: density 35 (separation 3, r^2 5, FP64 refinement of the reciprocal square root 6,
-# r 1, knot index 3, the cubic of phi 6, the sum 1, the derivative cubics of phi and V 8, their
-# scaling by 1/r 2) + force 12 (separation 3, the pair scalar from the cached derivatives 3, the
-# force 6).  Entries in the skin shell: 8 in the density pass (up to r^2), and the force pass's 12
-# on zero terms.  The half list takes each pair once: half of these per list entry.
+# FP64 operations per list entry inside r_cut if every pair term were FP64 arithmetic (an add or a
+# multiply is 1 flop, an FMA 2; conversions and rounding to integer not counted): density 35
+# (separation 3, r^2 5, FP64 refinement of the reciprocal square root 6, r 1, knot index 3, the
+# cubic of phi 6, the sum 1, the derivative cubics of phi and V 8, their scaling by 1/r 2) + force
+# 12 (separation 3, the pair scalar from the cached derivatives 3, the force 6).  Entries in the
+# skin shell: 8 in the density pass (up to r^2), and the force pass's 12 on zero terms.  The half
+# list takes each pair once: half of these per list entry.  The passes do nearly all of it on the
+# FP32 and integer pipes, so this is a throughput at FP64 accuracy without a peak.
 FP64_FLOP_IN, FP64_FLOP_SHELL = 47.0, 20.0
+# What the FP64 pipe still executes: per pair inside r_cut, 2 additions in the density pass (phi as
+# one FP64 number, its sum) and 6 in the force pass (three components, three sums); per atom the
+# sums over its lanes' slots, F(rho), the kicks and the drift, 190 with the half list at 4 lanes
+# (the counters of profiles/fp64_half_pieces.md: 739 operations per atom-step of fcc Cu in all, of
+# which 68.5 pairs).
+FP64_OPS_PAIR, FP64_OPS_ATOM = 8.0, 190.0
+
+
+def entries_inside(pos, w, sample=64):
+    """List entries inside r_cut per atom at positions pos: the mean over a sample of atoms."""
+    box, rc2 = np.asarray(w.box), float(w.potential.r_cut) ** 2
+    total = 0
+    for i in np.linspace(0, len(pos) - 1, sample).astype(int):
+        d = pos - pos[i]
+        d -= box * np.rint(d / box)
+        total += int((np.einsum("ij,ij->i", d, d) < rc2).sum()) - 1
+    return total / sample
 
 
 def fp64_flop_per_step(sum_counts, w):
-    """FP64 flop of one step of the FP64 passes by the per-entry model above; the share of list
-    entries inside r_cut is taken as (r_cut / r_list)^3 (uniform density)."""
+    """FP64-equivalent flop of one step of the FP64 passes by the per-entry model above; the share of
+    list entries inside r_cut is taken as (r_cut / r_list)^3 (uniform density)."""
     rc = float(w.potential.r_cut)
     f_in = (rc / (rc + w.skin)) ** 3
     return sum_counts * (f_in * FP64_FLOP_IN + (1.0 - f_in) * FP64_FLOP_SHELL)
+
+
+def fp64_pipe_ops_per_step(n, inside, half):
+    """FP64 operations of one step that execute on the FP64 pipe, by the model above."""
+    return n * (inside * FP64_OPS_PAIR * (0.5 if half else 1.0) + FP64_OPS_ATOM)
 
 
 def fp64_peak(md, stream, repeats=3, iters=5000):
@@ -394,7 +416,9 @@ def run_ours(args):
 
     r64, r32 = res[fp64_leg], res["mixed"]
     flop = fp64_flop_per_step(sum_counts, w) * args.steps * (0.5 if fp64_leg == "fp64_half" else 1.0)
-    achieved = flop / (r64["ms"] * 1e-3) / 1e12
+    equivalent = flop / (r64["ms"] * 1e-3) / 1e12
+    ops = fp64_pipe_ops_per_step(n, entries_inside(snapshot["pos"], w), fp64_leg == "fp64_half") * args.steps
+    achieved, op_peak = ops / (r64["ms"] * 1e-3) / 1e12, 0.5 * fp64_tflops
     f64, f32 = snapshot[fp64_leg], snapshot["mixed"]
     ferr = np.abs(f32 - f64)
     cpu = None
@@ -434,14 +458,20 @@ def run_ours(args):
                                "arithmetic than one Newton step of 1/r in FP64 gives (5e-14 of the RMS force)"),
                        fp64_walk=("half list: each pair once, the neighbour's share by FP64 atomics"
                                   if fp64_leg == "fp64_half" else "full list: each pair from both sides")),
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": fp64_tflops, "unit": "TFLOP/s",
-                     "frac": achieved / fp64_tflops, "traffic": _traffic("k_step_fp64", n, args.steps),
+        "roofline": {"bound": "alu", "achieved": achieved, "peak": op_peak, "unit": "T FP64 operations/s",
+                     "frac": achieved / op_peak, "traffic": _traffic("k_step_fp64", n, args.steps),
                      "kernel": "k_step (persistent: all phases of the K steps, stopping at each rebuild request "
                                "for the k_rebuild kernel and resuming), FP64 pipe",
-                     "peak_source": "measured in this run: md_measure_fp64_peak (FP64 FMA chains, CUDA events)",
-                     "flop_model": "work at FP64 accuracy: 47 flop per list entry inside r_cut over both passes, 20 "
-                                   "in the skin shell (an FMA counts 2), half of it with the half list; most of it is "
-                                   "done on the FP32 and integer pipes",
+                     "peak_source": "measured in this run: md_measure_fp64_peak (FP64 FMA chains, CUDA events); an "
+                                    "addition takes the pipe as long as an FMA",
+                     "op_model": "operations on the FP64 pipe: 8 additions per pair inside r_cut over both passes, "
+                                 "190 per atom (lane sums, F(rho), integration); the force pass is bound by this pipe "
+                                 "and the FP64 atomics, the density pass by issue slots",
+                     "ops_per_launch": ops,
+                     "fp64_equivalent": {"value": equivalent, "unit": "TFLOP/s",
+                                         "model": "work at FP64 accuracy: 47 flop per list entry inside r_cut over both "
+                                                  "passes, 20 in the skin shell (an FMA counts 2), half of it with the "
+                                                  "half list; nearly all of it on the FP32 and integer pipes"},
                      "flop_per_launch": flop, "avg_launch_ms": r64["ms"], "hbm": hbm(r64, "fp64")},
         "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": r64["launches"], "clocks": r64["clocks"],
         "nve_drift_ev_per_atom": (r64["e1"]["te"] - r64["e0"]["te"]) / n,

@@ -114,8 +114,12 @@ typedef struct {
     double dt_fs;          /* `deltat` */
     int32_t precision;     /* MD_PREC_FP64 (every sum, the integration and the reductions in
                               FP64; the pair terms of one-species tables as sums of two FP32
-                              numbers over whole-number separations (about 2^-46), else FP64
-                              arithmetic with 1/r formed to <= 4e-13 relative), or
+                              numbers over whole-number separations, 1/r and r to <= 6e-14
+                              relative, where box and tables are in their range (box edges to
+                              32,767 Å, at most 20,000 knots, the first not near 0, rows not
+                              above about 0.02 Å) and for pairs not closer than 0.03 Å (1 Å in
+                              the longest boxes); else FP64 arithmetic with 1/r formed to
+                              <= 4e-13 relative), or
                               MD_PREC_MIXED (FP32 pair/density terms,
                               FP64 positions, velocities, density sum and reductions; with
                               one species and knot tables the force pass takes the quadratic

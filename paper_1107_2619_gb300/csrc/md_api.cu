@@ -101,8 +101,8 @@ namespace {
 // Kernels of one stand-alone rebuild: the cooperative one, or launch_rebuild's nine and the clearing
 // one for the contexts with local rows.
 int rebuild_launches(const md_ctx *c, bool clear = true) { return c->C.tile ? 9 + (clear ? 1 : 0) : 1; }
-constexpr unsigned long long kSpinLimit = 20000000ull;  // barrier polls (~2 s) before giving up
-constexpr unsigned long long kSpinSelftest = 20000;     // of the self-tests: milliseconds
+constexpr unsigned long long kSpinLimit = 20000000ull;  // barrier polls (8 s: 0.4 us each) before giving up
+constexpr unsigned long long kSpinSelftest = 20000;     // of the self-tests: 8 ms
 constexpr int kWithholdTune = 11;                       // md_selftest_timeout_at: md_tune's trial steps
 
 md_status fail(md_ctx *c, md_status s, const std::string &what, cudaError_t e = cudaSuccess) {
@@ -641,12 +641,14 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
     }
     // lanes per atom: given, or from the expected neighbour count (4/3 pi r_list^3 x density) and the
     // number of atoms, measured on GB300, us a step at 1 / 2 / 4 / 8 lanes.  About 20 entries a lane (24
-    // for the FP32 terms): bcc Fe mixed 624,000 atoms 135 / 149 / 175 / 220, 35,000 22.7 / 24.2 / 27.8 /
-    // 30.2; fcc Cu FP64 83,000 - / 1319 / 1040 / 906, half list 88,000 - / 919 / 687 / 658, mixed 88,000 - /
-    // 176 / 148 / 136.  Half of that once the mixed lanes fill the chip 16 times, where fewer, longer walks
-    // gather better: fcc Cu 500,000 682 / 592 / 575 / 626.  A system that does not fill the chip takes
-    // more lanes, up to 8 (the group walks' most) and one for every other entry: bcc Fe FP64 2,000
-    // - / 33.9 / 24.3 / 18.2, mixed 3,456 21.2 / 18.2 / 16.6 / 16.2 but 11,664 21.1 / 19.5 / 22.3 / 24.9.
+    // for the FP32 terms): bcc Fe mixed 628,864 atoms 107 / 115 / 135 / 181, 35,152 23.2 / 24.6 / 28.9 /
+    // 30.9; fcc Cu 87,808 FP64 650 / 499 / 428 / 440, half list 515 / 460 / 411 / 399, double-float 343 /
+    // 428 / 344 / 303, mixed 173 / 160 / 130 / 117.  (FP64 full list: set where its pair terms were FP64
+    // arithmetic, 1319 / 1040 / 906 at 2 / 4 / 8; from pieces 8 is 3 to 5 % off the best.)  Half of that
+    // once the mixed lanes fill the chip 16 times, where fewer, longer walks gather better: fcc Cu 500,000
+    // 628 / 541 / 522 / 574.  A system that does not fill the chip takes more lanes, up to 8 (the group
+    // walks' most) and one for every other entry: bcc Fe FP64 2,000 49.2 / 33.0 / 24.1 / 18.3, mixed 3,456
+    // 18.4 / 15.9 / 14.9 / 15.1 but 11,664 18.8 / 17.4 / 20.2 / 22.6.
     {
         const int want = cfg->lanes_per_atom;
         if (want != 0 && want != 1 && want != 2 && want != 4 && want != 8 && want != 16 && want != 32)
@@ -956,7 +958,9 @@ md_status create_common(md_ctx *ctx, const md_config *cfg, const md_potential *p
         P.xmax_rho = nk - 1;
         // FP64, one species: the pair terms from FP32 pieces (ps::pair_terms_q), where every coefficient
         // is well inside FP32's range, relative to the largest of its function, and the fixed-point
-        // numbers hold the list's separations, the knots and the box; else FP64 arithmetic throughout
+        // numbers hold the list's separations, the knots and the box: edges up to 32,767 Å; a first knot
+        // from 0.016 Å (qfb 50) to 0.5 Å (45) on; rows up to 2^(55 - U) / (3 r_cut) Å high (0.02 Å at a
+        // cutoff of 7.23 Å), at most 20,000 of them.  Else FP64 arithmetic throughout
         std::vector<float4> TQ;
         if (ns == 1 && cfg->precision == MD_PREC_FP64) {
             double Lmax = 0.0;

@@ -451,17 +451,19 @@ __device__ __forceinline__ void force32_item(const Atoms &A, const Pot &P, const
 // One species with knot tables.  GB300's FP64 pipe runs at 1/64 of the FP32 rate, so the terms of a
 // pair are formed as unevaluated sums of two FP32 numbers (md_df.cuh) and enter the FP64 sums with one
 // FP64 addition each; sums, F(rho), integration and reductions are FP64 as before.
-//  - Separations are exact whole-number differences of fixed-point coordinates (Atoms::posq, 2^-50 Å
-//    for r_list up to 6.6 Å, 2^-49 Å up to 13.9 Å), and r^2 their sum of squares in 64 bits, rounded to
-//    about 2^-58 Å^2; the cut is a comparison of whole numbers.
+//  - Separations are exact whole-number differences of fixed-point coordinates (Atoms::posq) in units of
+//    2^-qfb Å: 2^-50 for r_list up to 6.6 Å and box edges up to 1,023 Å, 2^-49 up to 13.9 and 2,047 Å (the
+//    list decides up to there), a factor of two for each further doubling of the longest edge, to 2^-45
+//    at 32,767 Å.  r^2 is their sum of squares in 64 bits, in units of 2^(42 - 2 qfb) Å^2; the cut is a
+//    comparison of whole numbers.  Pairs so close that the unit would show: close_terms, below.
 //  - 1/r by Newton's step from the FP32 estimate with its second-order term, as hi + lo.
 //  - The knot coordinate t = (r - rho_k) / h from r^2 - rho_k^2, an exact whole-number difference, over
 //    r + rho_k: rho_k, the knot rounded to FP32, has an exact square, and the rows are cubics about it
 //    (the difference r - r_k itself, at 5,000 knots, would cost t twelve bits).
 //  - The cubic of phi and the slopes of V and phi with every coefficient as hi + lo.
-// Against 64-bit arithmetic the forces are closer than those of the FP64 evaluation they replace,
-// whose 1/r took one Newton step without the second-order term (on thermal fcc Cu 3e-14 of the RMS
-// force from the pair terms, 1.1e-13 before).  About 250 FP32 and whole-number operations a pair stand
+// 1/r is within 1e-14 of itself for any r^2 and unit; the unit adds at most 5e-14, at the closest.  Against 64-bit arithmetic the forces
+// are closer than those of the FP64 evaluation they replace, whose 1/r took one Newton step without the
+// second-order term (thermal fcc Cu, of the RMS force after 20 steps: 4.7e-14, 1.2e-13 before).  About 250 FP32 and whole-number operations a pair stand
 // in place of 16 on the FP64 pipe, each of which takes the time of 75.
 
 struct PairQ {
@@ -1628,9 +1630,10 @@ __device__ __forceinline__ void force64_pairs_flat(const Atoms &A, const Pot &P,
 // cached factors in the force pass) and the list entry after that are on their way.  The records of
 // the warp's own atoms wait in shared memory (after the slots of S).  fcc Cu 500,000 atoms, us per
 // step, before -> after: density 842 -> 800, force 926 -> 840 (of that, rows in two 32-byte loads
-// instead of four of 16 bytes: density 828 -> 800).  What bounds them now: density the L1's data pipe
-// (88 %: scattered rows and records), force the FP64 pipe (81 %: to64 and the sums) and the FP64
-// atomics (three a pair).  Double-float lane sums in place of the FP64 ones gained nothing.
+// instead of four of 16 bytes: density 828 -> 800).  What bounds them now (4 lanes): density the
+// issue slots (73 % busy; L1's data pipe 55 %), force the FP64 pipe (six additions a pair and the lane sums,
+// about 57 % of the pass) and the FP64 atomics (three a pair).  Double-float lane sums in place of the FP64
+// ones gained nothing.
 template <int AW>
 struct FlatEntry {
     int a, k, j;

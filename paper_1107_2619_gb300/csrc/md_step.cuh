@@ -191,10 +191,11 @@ __device__ __forceinline__ void thermo_update(const StepParams &sp, int n_rep, l
 #ifndef MD_STEP_MIN_BLOCKS
 #define MD_STEP_MIN_BLOCKS 8
 #endif
-// Blocks of 128 threads per SM the FP64 step kernel is built for: 4 (128 registers) measured 2-3 %
-// faster than 8 (64 registers, with spills) and 6 on fcc Cu 500k with the full list; the pair
+// Blocks of 128 threads per SM the FP64 step kernel is built for: 4 (128 registers) with the full
+// list, us per step of fcc Cu at 4 / 5 / 6 blocks and 4 lanes per atom: 500,000 atoms 2152 / 2331 / 2415,
+// 87,808 448 / 474 / 476 (but 19,652 152 / 137 / 140, where the blocks of one round are too few); the pair
 // walk over the half list is built for 5 (96 registers): 1.94 / 1.92 / 1.97 ms per step at 4 / 5 / 6
-// and 4 lanes per atom, 1.96 / 1.88 / 1.87 at 8 (the full list was 2 % slower at 5 than at 4).
+// and 4 lanes per atom, 1.96 / 1.88 / 1.87 at 8.
 #ifndef MD_STEP_MIN_BLOCKS_FP64
 #define MD_STEP_MIN_BLOCKS_FP64 4
 #endif
