@@ -123,3 +123,52 @@ def test_pairs_beside_a_knot(n_knots, r_min, walk, lanes):
     n = 2 * len(pick)
     w.pos, w.vel, w.species = np.concatenate([a, b]), np.zeros((n, 3)), np.zeros(n, np.int32)
     check_pair_forces(w, walk, lanes)
+
+
+@pytest.mark.parametrize("walk,lanes", WALKS)
+@pytest.mark.parametrize("length,fine", [(400.0, True), (30000.0, False)])
+def test_energy_and_virial_with_close_pairs(length, fine, walk, lanes):
+    """The close pairs' shares of E_i and of the virial (across the faces too) at the FP64 bar, by the
+    stand-alone passes and by an energy step of the step kernel; two replicas in one batch give the same."""
+    w = dimers(length, 1.0, fine)
+    ref = oracle.forces(w.pos, w.species, w.box, w.potential, skin=w.skin, k_max=w.k_max)
+    with md.System(w, precision="fp64", passes=walk, lanes_per_atom=lanes) as s:
+        s.eam_forces()
+        for step in (0, 1):
+            s.step(step)
+            e = s.energy()
+            assert abs(e["pe"] - ref["pe"]) <= 1e-10 * abs(ref["pe"])
+            assert np.abs(e["virial"] - ref["virial"]).max() <= 1e-10 * np.abs(ref["virial"]).max()
+    with md.Batch([w, w], precision="fp64", passes=walk, lanes_per_atom=lanes) as b:
+        b.eam_forces()
+        f = b.forces()
+    sc = oracle.eam_error_scales(w.pos, w.species, w.box, w.potential, ref["count"], ref["list"], ref["dF"])
+    bound = EPS * (2.0 * sc["m"] + sc["q"] + sc["e"])
+    assert np.all(np.abs(f - np.tile(ref["force"], (2, 1))).max(axis=1) <= np.tile(bound, 2))
+
+
+@pytest.mark.parametrize("walk,lanes", [("auto", 4), ("half", 8)])
+@pytest.mark.parametrize("kind", ["pc3", "nvt", "strain"])
+def test_other_motions_with_close_pairs(kind, walk, lanes):
+    """As test_steps_with_close_pairs, for the predictor-corrector, the thermostat and the strain ramp."""
+    w = dimers(400.0, 1.0, False)
+    steps = 7
+    w.dt_fs = dt = 1e-3
+    w.vel = np.random.default_rng(5).normal(0.0, 1e-4, w.pos.shape)
+    args = (w.pos, w.vel, w.species, w.potential.masses, w.box, w.potential, dt, steps, w.skin, w.k_max)
+    if kind == "strain":
+        w.strain_rate_zz = -1.0e9
+    with md.System(w, precision="fp64", passes=walk, lanes_per_atom=lanes,
+                   integrator="pc3" if kind == "pc3" else "verlet") as s:
+        if kind == "pc3":
+            ref = oracle.run_pc3(*args)
+        elif kind == "nvt":
+            s.set_thermostat(300.0, tau_fs=20.0)
+            s.eam_forces()
+            ref = oracle.run_nvt(*args, 300.0, s.thermostat()[0, 2])
+        else:
+            ref = oracle.run_vv(*args, strain_rate_zz=w.strain_rate_zz)
+        s.step(steps)
+        pos, vel = s.positions(), s.velocities()
+    assert np.abs(pos - ref["pos"]).max() <= 4.0 * np.spacing(400.0)
+    assert np.abs(vel - ref["vel"]).max() <= 100.0 * EPS * np.abs(ref["vel"]).max()
